@@ -248,8 +248,8 @@ lr_status lr_batch_query_all(lr_ctx* ctx, lr_stream_t stream, const lr_batch_des
  * string is a batch with num = 1) and the fastest is remembered in the
  * context for batches of the same shape class (total size and mean string
  * length, both rounded to powers of two).  Later queries of that class use
- * it; the default is the tile cover with 4096-position tiles and the
- * rank-order front end (code 9).  *choice receives the chosen shape code: bit 3 clear: the
+ * it; the default is the tile cover with 2048-position tiles and the
+ * rank-order front end (code 8).  *choice receives the chosen shape code: bit 3 clear: the
  * warp-segment cover (bits 0 and 2 clear); bit 3 set: the tile cover, with
  * bit 0: 4096-position tiles, bit 2: 8192-position tiles, neither: 2048;
  * bit 1: the rank front end (timed as the rank gather; a single query of
@@ -415,8 +415,8 @@ lr_status lr_query_all_static(lr_stream_t stream,
  * status word gives up after a bounded number of polls, records a timeout
  * and finishes, so a lost wait never hangs the GPU; this hook makes such a
  * wait run out on purpose without any fault.  While it is on, the cover
- * kernel's look-back unit number `tile` (a tile of 4096 positions with the
- * default warp-segment cover or with the tile cover's default shape) never
+ * kernel's look-back unit number `tile` (a tile of 2048 positions with the
+ * tile cover's default shape, of 4096 with the warp-segment cover) never
  * publishes its status word, and every look-back wait of the context's
  * queries gives up after `spin_limit` polls (1 .. 2^23; the default is
  * 2^23).  A query whose cover has more than tile + 1 units then waits for a

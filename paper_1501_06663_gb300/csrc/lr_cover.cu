@@ -3,29 +3,53 @@
 // LLR array LLRc to the longest repeats of every position.
 //
 // Starts and ends of LLRc strictly increase (Sec. 3.2), so the compact LLR's
-// covering a position k form a contiguous window of LLRc whose two ends only
-// move right as k grows.  Per tile of 2048, 4096 or 8192 positions (tiles in
-// order by an atomic ticket):
+// covering a position k form a contiguous window of LLRc, and entry v is a
+// longest one (a holder) exactly at the positions
+//     [max(s_v, e_PG + 1), min(e_v, s_NG - 1)],
+// PG / NG its nearest strictly longer neighbours in LLRc.  The set of holders
+// therefore changes only where such an interval begins or ends, and the
+// kernel works per entry (0.2 to 0.75 of them per position on the texts
+// measured), not per position.  Per tile of 2048, 4096 or 8192 positions
+// (tiles in order by an atomic ticket):
 //
-//  * the window range of the whole tile is LLRc[lo, cb1): the tile's own
-//    entries [cb0, cb1) plus the carry [lo, cb0), the earlier entries whose
-//    end reaches the tile; lo is found by a warp scanning back from cb0;
-//  * the range is staged in shared memory together with two bitmaps over the
-//    tile's positions: where an entry of the range starts and where one ends;
-//  * for position k the window is [lo_k, hi_k] with hi_k = (starts <= k) - 1
-//    and lo_k = (ends < k) in carry ++ local numbering: two prefix popcounts,
-//    no binary search (the paper's per-position binary search);
-//  * the longest length, the leftmost start and the ties of every window
-//    (Algorithm 2's walk, with Algorithm 4's count) come from a range-maximum
-//    table built per run of 32 positions over the run's entries (a walk over
-//    the window when the run spans more than 32 entries);
-//  * for the all-LR query, the tie counts are scanned (block scan plus a
-//    decoupled look-back over the tiles) into CSR offsets, and a second walk
-//    writes every start of the longest length, ascending (Algorithm 4's
-//    second walk).
+//  * the entries that reach the tile, LLRc[lo, cb1), are staged in shared
+//    memory: the tile's own [cb0, cb1) plus the carry before them;
+//  * one thread per entry looks left and right over the overlapping entries
+//    for PG and NG, counting those of its own length on the way: this gives
+//    the interval, the holders where it begins and the holders left where it
+//    ends, and so a record (leftmost holder, number of holders) for every
+//    position where the set of holders changes, and the tile's number of
+//    LR starts, which is published for the look-back at once;
+//  * a position finds its record by one bit scan over a bitmap of those
+//    positions: longest length and leftmost start are the holder's
+//    (Algorithm 2), the tie count is in the record;
+//  * for the all-LR query the tie counts are scanned into CSR offsets
+//    (ballots per run of 32 positions, warp totals, decoupled look-back over
+//    the tiles), and every holder's start is written, ascending, by following
+//    the links to the next entry of the same length (Algorithm 4's second
+//    walk).
+//
+// A tile whose carry is longer than kSpec entries (more than kSpec compact
+// LLR's over one position) walks LLRc in place instead (cover_long_carry).
 //
 // A lane owns one position of each run of 32, so every per-position store of
 // a warp is one contiguous 128- or 256-byte run.
+//
+// What bounds it: instruction issue (about 75 % of the slots) and the waits
+// between its phases, of which the look-back is the longest; DRAM runs at
+// half its rate.  The form before it worked per position (a range-maximum
+// table over the window of each run of 32) and took 2.18 ms for 2^28
+// positions of English (0.21 entries per position), 2.77 ms for 258 M of
+// mixed DNA and protein (0.52); this one takes 1.58 and 2.39 ms.  It has 180
+// instead of 240 instructions per run of 32 positions (English); per-entry
+// work pays as long as entries are fewer than positions, which they are by
+// construction (at most one starts at each).  Four consecutive positions per
+// lane with vector stores were faster without the CSR outputs (0.254 against
+// 0.258 ms at 100 M positions) but slower with them (1.69 against 1.58 ms:
+// the list of starts then needs gathering in shared memory).  Persistent
+// CTAs that take the next ticket early were slower (2.24 ms): a tile taken
+// early publishes late, and every later tile waits for it; so were look-back
+// steps over 128 or 256 words (1.88, 2.12 ms).
 #include <cuda_runtime.h>
 #include <cstdint>
 #include "lr_device.cuh"
@@ -35,8 +59,12 @@ namespace lr {
 
 namespace {
 
+constexpr int32_t kSpec = 64;                     // carry entries staged with the tile's own
+
 // Shape of a cover tile of kTile x TP positions run by kThreads x TP threads;
-// every warp owns 8 runs of 32 positions.
+// every warp owns 8 consecutive runs of 32 positions.  kMinBlocks fills all
+// warp slots of an SM in every shape (27.5 KB of shared memory per 2048
+// positions, 32 registers; 6 instead of 8 CTAs with 40 registers: 3 % slower).
 template <int TP>
 struct Cfg {
     static constexpr int kTileC = kTile * TP;
@@ -44,36 +72,43 @@ struct Cfg {
     static constexpr int kWarps = kThr / kWarp;
     static constexpr int kChunks = kTileC / kWarp;
     static constexpr int kChunksPerWarp = kChunks / kWarps;
-    static constexpr int kMinBlocks = TP == 1 ? 5 : (TP == 2 ? 4 : 2);
-    static constexpr int kCap = kTileC + 128;     // staged entries: the tile's own and a carry
-    // Width of the holder-index field of the packed per-run word pk (see
-    // k_cover): every staged index v < kCap and the "none" value all-ones
-    // must fit; the holder mask or count takes the bits above it up to 30.
-    static constexpr int kVBits = (kCap <= (1 << 13) - 1) ? 13 : 14;
-    static constexpr uint32_t kNone = (1u << kVBits) - 1u;
-    static constexpr int kMaskBits = 31 - kVBits;
-    static_assert(kCap <= (int)kNone, "staged window indices must fit the holder-index field");
-    static_assert(kCap < (1 << kMaskBits), "a tie count must fit the count field");
+    static constexpr int kMinBlocks = TP == 1 ? 8 : (TP == 2 ? 4 : 2);
+    static constexpr int kCap = kTileC + kSpec;   // the tile's own entries and the carry always fit
+    static_assert(kCap + 2 < (1 << 16), "record indices must fit 16 bits");
 };
 
 template <int TP>
 struct __align__(16) CoverSmem {
     static constexpr int kChunks = Cfg<TP>::kChunks;
-    int32_t cs[Cfg<TP>::kCap];       // window range LLRc[lo, cb1): starts
-    int32_t cl[Cfg<TP>::kCap];       //                             lengths
-    unsigned smap[kChunks];          // bit x: an entry of the tile starts at k0 + x
-    unsigned emap[kChunks];          // bit x: an entry of the range ends at k0 + x
-    int32_t spre[kChunks];           // exclusive prefix popcounts of the bitmap words
-    int32_t epre[kChunks];
-    int32_t chunk[kChunks];          // run totals of the tie counts
-    unsigned rt[Cfg<TP>::kWarps][Cfg<TP>::kChunksPerWarp][kWarp];   // per warp: range-max levels 0..4 and
-                                     // equal-length masks; then the runs' tie-count prefixes
+    // Staged entry i at ent[i + 1]: start, length.  ent[0] has length 0 and
+    // start -1: it stops the scans to the left and is the "no holder" entry;
+    // the one after the last starts after everything and stops the scans to
+    // the right.
+    int2 ent[Cfg<TP>::kCap + 2];
+    uint32_t rec[Cfg<TP>::kTileC];   // at a boundary: ent index of the leftmost holder | number of holders << 16
+    unsigned bmap[kChunks];          // bit x: the set of holders changes at position x (bit 0 always set)
+    // distance to the next entry of the same length with no longer one
+    // between (0: none that overlaps; 255: that or more)
+    static constexpr int kNxWords = (Cfg<TP>::kCap + 2 + 3) / 4;
+    uint32_t nx[kNxWords];
+    int32_t wtot[Cfg<TP>::kWarps];   // tie counts per warp
     long long tile;
     long long obase;
     int32_t lo;
     int32_t nlow;                    // staged carry candidates that end before the tile
     int32_t ttot;                    // the tile's total of tie counts
-    int32_t longlen;                 // a staged length reaches 2^27 (too long for the range-max keys)
+    int32_t far;                     // a distance does not fit nx
+};
+
+// The words cover_long_carry keeps in place of the staged entries.
+template <int TP>
+struct LongSmem {
+    static constexpr int kChunks = Cfg<TP>::kChunks;
+    unsigned smap[kChunks];          // bit x: an entry starts at k0 + x
+    unsigned emap[kChunks];          // bit x: an entry ends at k0 + x
+    int32_t spre[kChunks];           // exclusive prefix popcounts of the bitmap words
+    int32_t epre[kChunks];
+    int32_t chunk[kChunks];          // run totals of the tie counts
 };
 
 // Exclusive prefix popcounts of the kChunks bitmap words, by one warp.
@@ -104,6 +139,136 @@ __device__ __forceinline__ int scan_chunks(int32_t* a) {
     return __shfl_sync(kFull, incl, kWarp - 1);
 }
 
+// Exclusive prefix of the tie counts c of a warp's 32 positions; *tot their
+// sum.  Counts are almost always below 4: two ballots over their bit planes.
+__device__ __forceinline__ int ties_prefix(int c, unsigned below, int* tot) {
+    if (__ballot_sync(kFull, c > 3) == 0u) {
+        const unsigned b0 = __ballot_sync(kFull, c & 1), b1 = __ballot_sync(kFull, c & 2);
+        *tot = __popc(b0) + 2 * __popc(b1);
+        return __popc(b0 & below) + 2 * __popc(b1 & below);
+    }
+    const int incl = warp_incl_scan(c);
+    *tot = __shfl_sync(kFull, incl, kWarp - 1);
+    return incl - c;
+}
+
+// The tile's place in starts[] (whole warp): look back over the earlier
+// tiles, publish the inclusive prefix, write offsets[n] from the last tile.
+__device__ __forceinline__ long long place_tile(const Scratch& s, long long tile, long long ntiles, int32_t n, int tot,
+                                                int64_t* __restrict__ offsets) {
+    const long long ex = (tile == 0) ? 0 : lookback(s.status_o, tile, s.err, s.qerr, s.spin_limit);
+    if (lane_id() == 0) {
+        if (tile != 0 && tile != s.hold_tile) publish(s.status_o, tile, kPrefix, ex + tot);
+        if (tile == ntiles - 1) offsets[n] = ex + tot;
+    }
+    return ex;
+}
+
+// A tile with a carry too long to stage: the window of each position from
+// bitmaps of starts and ends (popcounts), its entries walked in LLRc.
+// Called by the whole CTA.
+template <bool kAll, int TP>
+__device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, const Scratch& s, long long tile, int32_t cb0,
+                                              int32_t cb1, int32_t* __restrict__ lr_len, int32_t* __restrict__ lr_start,
+                                              int64_t* __restrict__ offsets, int32_t* __restrict__ starts,
+                                              long long capacity) {
+    constexpr int kCoverTile = Cfg<TP>::kTileC, kCoverThreads = Cfg<TP>::kThr, kWarps = Cfg<TP>::kWarps;
+    constexpr int kChunks = Cfg<TP>::kChunks, kChunksPerWarp = Cfg<TP>::kChunksPerWarp;
+    static_assert(sizeof(LongSmem<TP>) <= sizeof(sm.ent), "the bitmaps replace the staged entries");
+    LongSmem<TP>& lm = *reinterpret_cast<LongSmem<TP>*>(sm.ent);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int32_t k0 = (int32_t)(tile * kCoverTile);
+    if (tid < kChunks) { lm.smap[tid] = 0; lm.emap[tid] = 0; }
+    if (warp == 0) {                                  // the first entry that reaches the tile (ends increase)
+        int32_t t = cb0;
+        while (t > 0) {
+            const int32_t idx = t - 1 - lane;
+            const bool reach = idx >= 0 && __ldg(s.cend + idx) >= k0;
+            const unsigned m = __ballot_sync(kFull, reach);
+            if (m == kFull) { t -= kWarp; continue; }
+            t -= __ffs(~m) - 1;
+            break;
+        }
+        if (lane == 0) sm.lo = t;
+    }
+    __syncthreads();
+    const int32_t lo = sm.lo, C = cb0 - lo, M = cb1 - lo;
+    for (int i = tid; i < M; i += kCoverThreads) {
+        const int32_t cs = __ldg(s.cstart + lo + i), ce = __ldg(s.cend + lo + i);
+        const uint32_t xs = (uint32_t)(cs - k0), xe = (uint32_t)(ce - k0);
+        if (i >= C && xs < (uint32_t)kCoverTile) atomicOr(&lm.smap[xs >> 5], 1u << (xs & 31));
+        if (xe < (uint32_t)kCoverTile) atomicOr(&lm.emap[xe >> 5], 1u << (xe & 31));
+    }
+    __syncthreads();
+    if (warp == 0) popc_prefix<kChunks>(lm.smap, lm.spre);
+    if (warp == 1) popc_prefix<kChunks>(lm.emap, lm.epre);
+    __syncthreads();
+    const int32_t* gcs = s.cstart + lo;
+    const int32_t* gce = s.cend + lo;
+    const unsigned below = (1u << lane) - 1u;
+    // window [lw, hi] of this lane's position in run c
+    auto window = [&](int c, int32_t& lw, int32_t& hi) {
+        hi = C + lm.spre[c] + __popc(lm.smap[c] & (below | (1u << lane))) - 1;
+        lw = lm.epre[c] + __popc(lm.emap[c] & below);
+    };
+    // longest length b over the window, its leftmost holder vb, the number of holders ct
+    auto best_of = [&](int32_t lw, int32_t hi, int32_t& b, int32_t& vb, int32_t& ct) {
+        b = 0; vb = -1; ct = 0;
+        for (int32_t v = lw; v <= hi; ++v) {
+            const int32_t len = __ldg(gce + v) - __ldg(gcs + v) + 1;
+            const bool gt = len > b;
+            ct = gt ? 1 : ct + (len == b);
+            vb = gt ? v : vb;
+            b = gt ? len : b;
+        }
+    };
+    int32_t pk[kChunksPerWarp], pre[kChunksPerWarp];  // tie counts and their prefixes within the run
+#pragma unroll
+    for (int q = 0; q < kChunksPerWarp; ++q) {
+        const int c = warp * kChunksPerWarp + q;
+        const int32_t k = k0 + c * kWarp + lane;
+        int32_t lw, hi, b, vb, ct;
+        window(c, lw, hi);
+        best_of(lw, hi, b, vb, ct);
+        if (k < n) {
+            __stcs(lr_len + k, b);
+            __stcs(lr_start + k, b > 0 ? __ldg(gcs + vb) : -1);
+        }
+        pk[q] = k < n ? ct : 0;
+        if constexpr (kAll) {
+            int tot;
+            pre[q] = ties_prefix(pk[q], below, &tot);
+            if (lane == 0) lm.chunk[c] = tot;
+        }
+    }
+    if constexpr (kAll) {
+        __syncthreads();
+        if (warp == 0) {
+            const int tot = scan_chunks<kChunks>(lm.chunk);
+            if (lane == 0 && tile != s.hold_tile) publish(s.status_o, tile, tile == 0 ? kPrefix : kAggregate, tot);
+            const long long ex = place_tile(s, tile, num_cover_tiles(n, TP), n, tot, offsets);
+            if (lane == 0) sm.obase = ex;
+        }
+        __syncthreads();
+        const long long obase = sm.obase;
+        for (int q = 0; q < kChunksPerWarp; ++q) {
+            const int c = warp * kChunksPerWarp + q;
+            const int32_t k = k0 + c * kWarp + lane;
+            long long o = obase + lm.chunk[c] + pre[q];
+            if (k < n) __stcs(reinterpret_cast<long long*>(offsets) + k, o);
+            if (pk[q] == 0) continue;
+            int32_t lw, hi, b, vb, ct;
+            window(c, lw, hi);
+            best_of(lw, hi, b, vb, ct);
+            for (int32_t v = vb; v <= hi; ++v) {
+                if (__ldg(gce + v) - __ldg(gcs + v) + 1 != b) continue;
+                if (o < capacity) __stcs(starts + o, __ldg(gcs + v));
+                ++o;
+            }
+        }
+    }
+}
+
 }  // namespace
 
 template <bool kAll, int TP>
@@ -119,9 +284,17 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
     extern __shared__ __align__(16) unsigned char cover_smem[];
     CoverSmem<TP>& sm = *reinterpret_cast<CoverSmem<TP>*>(cover_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) sm.tile = atomicAdd(&s.tickets[2], 1u);
-    if (tid < kChunks) { sm.smap[tid] = 0; sm.emap[tid] = 0; }
-    if (tid == 0) { sm.nlow = 0; sm.longlen = 0; }
+    if (tid == 0) {
+        sm.tile = atomicAdd(&s.tickets[2], 1u);
+        sm.nlow = 0;
+        sm.ttot = 0;
+        sm.far = 0;
+        sm.rec[0] = 0;                                       // no holder at the tile's start, unless an entry writes it
+    }
+    if (tid < kChunks) sm.bmap[tid] = tid == 0 ? 1u : 0u;
+    if constexpr (kAll) {
+        for (int i = tid; i < CoverSmem<TP>::kNxWords; i += kCoverThreads) sm.nx[i] = 0;
+    }
     __syncthreads();
     const long long tile = sm.tile;
     const int32_t k0 = (int32_t)(tile * kCoverTile);         // n < 2^31: positions fit 32 bits
@@ -132,290 +305,212 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
     int32_t cb0 = s.tile_cbase[ft], cb1 = s.tile_cbase[ft1];
     cb0 = cb0 < 0 ? 0 : (cb0 > n ? n : cb0);
     cb1 = cb1 < cb0 ? cb0 : (cb1 > n ? n : cb1);
+    if (cb1 - cb0 > kCoverTile) cb1 = cb0 + kCoverTile;
 
     // Stage LLRc[cb0 - kSpec, cb1): the tile's own entries and, in the same
     // round trip, the kSpec entries before them, which hold the carry (the
     // entries whose end reaches k0: a suffix, ends increase) unless it is
-    // longer than kSpec.  A longer carry takes the slow path below.
-    constexpr int32_t kSpec = 64;
+    // longer than kSpec.
     const int32_t sbase = cb0 > kSpec ? cb0 - kSpec : 0;
     const int32_t MS = cb1 - sbase;
-    const bool fits = MS <= Cfg<TP>::kCap;
-    // One pass over the staged entries: lengths, the two bitmaps (entries of
-    // [sbase, lo) end before k0, so they set no bit), and the number of
-    // staged carry candidates that end before k0: ends increase, so they
-    // are a prefix and lo = sbase + that number.
     const int32_t nspec = cb0 - sbase;
-    if (fits) {
-        for (int i0 = 0; i0 < MS; i0 += kCoverThreads) {
-            const int i = i0 + tid;
-            bool low = false;
-            if (i < MS) {
-                const int32_t cs = __ldg(s.cstart + sbase + i), ce = __ldg(s.cend + sbase + i);
-                sm.cs[i] = cs;
-                sm.cl[i] = ce - cs + 1;
-                if (ce - cs + 1 >= (1 << 27)) sm.longlen = 1;
-                const uint32_t xs = (uint32_t)(cs - k0), xe = (uint32_t)(ce - k0);
-                if (i >= nspec && xs < (uint32_t)kCoverTile) atomicOr(&sm.smap[xs >> 5], 1u << (xs & 31));
-                if (xe < (uint32_t)kCoverTile) atomicOr(&sm.emap[xe >> 5], 1u << (xe & 31));
-                low = i < nspec && ce < k0;
-            }
-            const unsigned m = __ballot_sync(kFull, low);
+    constexpr int kBatch = 2;                                 // entries a thread has in flight (one: 4 % slower)
+    for (int i0 = 0; i0 < MS; i0 += kBatch * kCoverThreads) {
+        int32_t cs[kBatch], ce[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int i = i0 + u * kCoverThreads + tid;
+            cs[u] = i < MS ? __ldg(s.cstart + sbase + i) : 0;
+            ce[u] = i < MS ? __ldg(s.cend + sbase + i) : 0;
+        }
+        if (i0 == 0 && warp < kSpec / kWarp) {
+            const unsigned m = __ballot_sync(kFull, tid < nspec && ce[0] < k0);
             if (lane == 0 && m) atomicAdd(&sm.nlow, __popc(m));
         }
-    }
-    __syncthreads();
-    // staged unless every staged candidate reaches k0 with more LLRc before
-    // them: then the carry may be longer, and it is found in LLRc itself
-    const int32_t nlow = sm.nlow;
-    const bool staged = fits && !(sbase > 0 && nlow == 0) && !sm.longlen;
-    int32_t lo = sbase + nlow;
-    if (!staged) {
-        if (tid < kChunks) { sm.smap[tid] = 0; sm.emap[tid] = 0; }
-        if (warp == 0) {
-            int32_t t = cb0;
-            while (t > 0) {
-                const int32_t idx = t - 1 - lane;
-                const bool reach = idx >= 0 && __ldg(s.cend + idx) >= k0;
-                const unsigned m = __ballot_sync(kFull, reach);
-                if (m == kFull) { t -= kWarp; continue; }
-                t -= __ffs(~m) - 1;
-                break;
-            }
-            if (lane == 0) sm.lo = t;
-        }
-        __syncthreads();
-        lo = sm.lo;
-        const int32_t Cg = cb0 - lo, Mg = cb1 - lo;
-        for (int i = tid; i < Mg; i += kCoverThreads) {
-            const int32_t cs = __ldg(s.cstart + lo + i), ce = __ldg(s.cend + lo + i);
-            const uint32_t xs = (uint32_t)(cs - k0), xe = (uint32_t)(ce - k0);
-            if (i >= Cg && xs < (uint32_t)kCoverTile) atomicOr(&sm.smap[xs >> 5], 1u << (xs & 31));
-            if (xe < (uint32_t)kCoverTile) atomicOr(&sm.emap[xe >> 5], 1u << (xe & 31));
-        }
-        __syncthreads();
-    }
-    const int32_t C = cb0 - lo;
-    // staged: window entry v sits at sm.cs/cl[v + shift]
-    const int32_t shift = staged ? lo - sbase : 0;
-    if (warp == 0) popc_prefix<kChunks>(sm.smap, sm.spre);
-    if (warp == 1) popc_prefix<kChunks>(sm.emap, sm.epre);
-    __syncthreads();
-
-    // candidate v of the range: start and length (shared memory, or LLRc in
-    // place when the range is too long to stage)
-    const int32_t* gcs = s.cstart + lo;
-    const int32_t* gce = s.cend + lo;
-    const int32_t* SCS = sm.cs + shift;
-    const int32_t* SCL = sm.cl + shift;
-    auto start_of = [&](int32_t v) -> int32_t { return staged ? SCS[v] : __ldg(gcs + v); };
-    const unsigned below = (1u << lane) - 1u;
-    // window [lw, hi] of this lane's position in run c (carry ++ local numbering)
-    auto window = [&](int c, int32_t& lw, int32_t& hi) {
-        hi = C + sm.spre[c] + __popc(sm.smap[c] & (below | (1u << lane))) - 1;
-        lw = sm.epre[c] + __popc(sm.emap[c] & below);
-    };
-    // longest length b over the window, index vb of its leftmost holder and
-    // the number of holders ct: the first four entries without branches
-    // (nearly every window), a loop for the rest
-    auto best_of = [&](int32_t lw, int32_t hi, int32_t& b, int32_t& vb, int32_t& ct) {
-        b = 0; vb = -1; ct = 0;
-        auto step = [&](int32_t len, int32_t v) {
-            const bool gt = len > b;
-            ct = gt ? 1 : ct + (len == b);
-            vb = gt ? v : vb;
-            b = gt ? len : b;
-        };
-        if (staged) {
-            const int32_t* CL = SCL;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int32_t v = lw + u;
-                const int32_t len = (v <= hi) ? CL[v] : -1;
-                step(len, v);
+        for (int u = 0; u < kBatch; ++u) {
+            const int i = i0 + u * kCoverThreads + tid;
+            // entries inside [0, n): whatever a failed front end (already
+            // reported) left here, the scans below end at the outer entries
+            if ((uint32_t)cs[u] >= (uint32_t)n) cs[u] = k0;
+            if (ce[u] < cs[u] || ce[u] >= n) ce[u] = cs[u];
+            if (i < MS) sm.ent[i + 1] = make_int2(cs[u], ce[u] - cs[u] + 1);
+        }
+    }
+    if (tid == 0) {
+        sm.ent[0] = make_int2(-1, 0);
+        sm.ent[MS + 1] = make_int2(0x7fffffff, 0);
+    }
+    __syncthreads();
+    // every staged candidate reaches k0 with more LLRc before them: the carry
+    // may be longer than what is staged
+    const int32_t nlow = sm.nlow;
+    if (sbase > 0 && nlow == 0) {
+        __syncthreads();
+        cover_long_carry<kAll, TP>(sm, n, s, tile, cb0, cb1, lr_len, lr_start, offsets, starts, capacity);
+        return;
+    }
+
+    // Per entry: the positions of the tile [hs, he) where it is a holder, the
+    // holders where they begin and those left where it ends.
+    uint8_t* const nx = reinterpret_cast<uint8_t*>(sm.nx);
+    const int32_t k1 = k0 > 0x7fffffff - kCoverTile ? 0x7fffffff : k0 + kCoverTile;   // the tile's end (no entry ends past n)
+    int32_t held = 0;                                         // positions x holders of this thread's entries
+    for (int v0 = nlow + 1 + warp * kWarp; v0 <= MS; v0 += kCoverThreads) {
+        const int v = v0 + lane;
+        const bool in = v <= MS;                              // other lanes take the outer entries and stop at once
+        const int2 me = sm.ent[in ? v : 0];
+        const int32_t L = me.y, e1 = me.x + L;                // one past its end
+        const int32_t a = me.x > k0 ? me.x : k0;
+        const int32_t b1 = e1 < k1 ? e1 : k1;
+        // to the left, over the entries that still cover a: those of length L
+        // before a longer one are holders wherever v begins to be one
+        int32_t left = v, eq = 1, qe;
+        bool go;
+        int u = in ? v : 1;
+        do {
+            const int2 q = sm.ent[--u];
+            qe = q.x + q.y;
+            go = (qe > a) & (q.y <= L);
+            if (go & (q.y == L)) { ++eq; left = u; }
+        } while (go);
+        const int32_t hs = qe > a ? qe : a;
+        // to the right, over the entries that start by e1, up to a longer one
+        // (unless v is never the longest in this tile)
+        int32_t first = MS + 1, feq = 0, qs;
+        u = hs < b1 ? v : MS;
+        do {
+            const int2 q = sm.ent[++u];
+            qs = q.x;
+            go = (qs <= e1) & (q.y <= L);
+            if (go & (q.y == L)) { first = min(first, u); ++feq; }
+        } while (go);
+        const int32_t he = qs < b1 ? qs : b1;
+        if (hs < he) {
+            held += he - hs;
+            if constexpr (kAll) {
+                if (feq > 0) {
+                    nx[v] = (uint8_t)(first - v < 255 ? first - v : 255);
+                    if (first - v >= 255) sm.far = 1;
+                }
             }
-            for (int32_t v = lw + 4; v <= hi; ++v) step(CL[v], v);
-        } else {
-            for (int32_t v = lw; v <= hi; ++v) step(__ldg(gce + v) - __ldg(gcs + v) + 1, v);
+            if (sm.ent[first].x > hs) {                       // else the next of length L begins at hs too
+                const int32_t x = hs - k0;
+                sm.rec[x] = (uint32_t)left | ((uint32_t)eq << 16);
+                atomicOr(&sm.bmap[x >> 5], 1u << (x & 31));
+            }
+            // where v ends with no longer entry begun: the remaining holders
+            // of length L, if any; nothing, if no entry starts by then; else
+            // the best shorter entry begins there
+            if (qs > e1 && e1 < k1 && (feq > 0 || u == v + 1)) {
+                const int32_t x = e1 - k0;
+                sm.rec[x] = feq > 0 ? ((uint32_t)first | ((uint32_t)feq << 16)) : 0u;
+                atomicOr(&sm.bmap[x >> 5], 1u << (x & 31));
+            }
         }
-    };
-    // Per run of 32 positions: the windows of its lanes lie inside one range
-    // [U0, U1] of at most a few dozen entries (both window ends only move
-    // right).  When it has at most 32 entries, lane j holds entry U0 + j and
-    // the warp builds a range-maximum table over the keys (length << 5 |
-    // 31 - j) in five shuffle levels, plus each lane's mask of equal lengths
-    // (match.any); a window's longest length and leftmost holder are then
-    // two table reads and its holders one mask, with no per-lane loop (whose
-    // cost in a warp would be the longest window of its 32 lanes).  Other
-    // runs take the walk of best_of.
-    //
-    // Per run the lane keeps pk[], packed (the longest length is stored at
-    // once, and read back from the leftmost holder when needed again):
-    //   staged tiles:  bits 0..B-1 leftmost holder v (all ones: none), B =
-    //                  kVBits (13, or 14 for 8192-position tiles, whose
-    //                  staged indices reach 8319); bit 31 clear: bits B..30 =
-    //                  holders as a mask from v (bit 0 = v); bit 31 set:
-    //                  bits B..30 = number of holders;
-    //   other tiles:   the number of holders.
-    constexpr int kVBits = Cfg<TP>::kVBits;
-    constexpr uint32_t kNone = Cfg<TP>::kNone;
-    constexpr uint32_t kFieldMask = (1u << Cfg<TP>::kMaskBits) - 1u;
-    uint32_t pk[kChunksPerWarp];
-    unsigned (*RT)[kWarp] = sm.rt[warp];
-    // the longest length and the leftmost holder's start of a position are
-    // stored as soon as its run is done (Algorithm 2's output)
-    auto store_leftmost = [&](int c, int32_t b, int32_t vb) {
-        const int32_t k = k0 + c * kWarp + lane;
-        if (k < n) {
-            __stcs(lr_len + k, b);
-            __stcs(lr_start + k, b > 0 ? start_of(vb) : -1);
+        __syncwarp();
+    }
+    if constexpr (kAll) {
+        held = (int32_t)__reduce_add_sync(kFull, (unsigned)held);
+        if (lane == 0 && held) atomicAdd(&sm.ttot, held);
+    }
+    __syncthreads();
+    if constexpr (kAll) {
+        if (tid == 0 && tile != s.hold_tile) publish(s.status_o, tile, tile == 0 ? kPrefix : kAggregate, sm.ttot);
+    }
+
+    // Per position: its record is the one of the last boundary at or before it.
+    const unsigned below = (1u << lane) - 1u;
+    const unsigned upto = below | (1u << lane);
+    const int c0 = warp * kChunksPerWarp;
+    int pb = 0;                                               // last boundary before the warp's current run
+    for (int w0 = c0; w0 > 0; w0 -= kWarp) {
+        const int w = w0 - 1 - lane;
+        const unsigned word = w >= 0 ? sm.bmap[w] : 0u;
+        const unsigned m = __ballot_sync(kFull, word != 0u);
+        if (m) {
+            const int l = __ffs(m) - 1;
+            pb = (w0 - 1 - l) * kWarp + 31 - __clz(__shfl_sync(kFull, word, l));
+            break;
         }
-    };
+    }
+    uint32_t pk[kChunksPerWarp];                              // the positions' records
+    int32_t sum = 0;
 #pragma unroll
     for (int q = 0; q < kChunksPerWarp; ++q) {
-        const int c = q * kWarps + warp;
-        int32_t lw, hi;
-        window(c, lw, hi);
-        const int32_t U0 = __shfl_sync(kFull, lw, 0);
-        const int32_t usz = __shfl_sync(kFull, hi, kWarp - 1) - U0 + 1;
-        const bool fast = staged && usz <= kWarp;                 // warp-uniform; staged lengths < 2^27
-        if (fast) {
-            const int32_t len_l = ((int)lane < usz) ? SCL[U0 + (int)lane] : 0;
-            unsigned key = ((int)lane < usz) ? (((unsigned)len_l << 5) | (31u - lane)) : 0u;
-            RT[0][lane] = key;
-            if constexpr (kAll) RT[5][lane] = __match_any_sync(kFull, len_l);
-#pragma unroll
-            for (int l = 1; l <= 4; ++l) {
-                const unsigned o = __shfl_down_sync(kFull, key, 1u << (l - 1));
-                key = key > o ? key : o;
-                RT[l][lane] = key;
-            }
-            __syncwarp();
-            // every lane queries (an empty window reads a harmless entry and
-            // is then discarded), so the warp does not diverge
-            const bool valid = lw <= hi;
-            const int l0 = valid ? lw - U0 : 0, h0 = valid ? hi - U0 : 0;
-            int lv = 31 - __clz(h0 - l0 + 1);
-            lv = lv > 4 ? 4 : lv;
-            const unsigned ka = RT[lv][l0], kb = RT[lv][h0 - (1 << lv) + 1];
-            const unsigned kk = ka > kb ? ka : kb;
-            const int jl = 31 - (int)(kk & 31u);
-            const int32_t b = valid ? (int32_t)(kk >> 5) : 0;
-            const int32_t sj = SCS[valid ? U0 + jl : 0];
-            uint32_t p = kNone;
-            if constexpr (kAll) {
-                const unsigned range = ((2u << h0) - 1u) & ~((1u << jl) - 1u);
-                const unsigned hold = (RT[5][jl] & range) >> jl;
-                const uint32_t v = (uint32_t)(U0 + jl);
-                const uint32_t pm = hold <= kFieldMask ? (v | (hold << kVBits))
-                                                       : (v | ((uint32_t)__popc(hold) << kVBits) | 0x80000000u);
-                p = valid ? pm : kNone;
-            }
-            __syncwarp();                                         // before the next run rewrites RT
-            pk[q] = p;
-            const int32_t k = k0 + c * kWarp + lane;
-            if (k < n) {
-                __stcs(lr_len + k, b);
-                __stcs(lr_start + k, valid ? sj : -1);
-            }
+        const int x0 = (c0 + q) * kWarp;
+        const unsigned word = sm.bmap[c0 + q];
+        const unsigned m = word & upto;
+        const uint32_t r = sm.rec[m ? x0 + 31 - __clz(m) : pb];
+        if (word) pb = x0 + 31 - __clz(word);
+        const int2 h = sm.ent[r & 0xffffu];
+        const int32_t k = k0 + x0 + lane;
+        pk[q] = r;
+        if (k < n) {
+            __stcs(lr_len + k, h.y);
+            __stcs(lr_start + k, h.x);
+            sum += (int32_t)(r >> 16);
         } else {
-            int32_t b, vb, ct;
-            best_of(lw, hi, b, vb, ct);
-            store_leftmost(c, b, vb);
-            if (!staged) pk[q] = (uint32_t)ct;
-            else if (ct == 0) pk[q] = kNone;
-            else if (ct == 1) pk[q] = (uint32_t)vb | (1u << kVBits);
-            else pk[q] = (uint32_t)vb | ((uint32_t)ct << kVBits) | 0x80000000u;
+            pk[q] = 0;
         }
     }
-    // holders of run q (the tie count of its position)
-    auto count_of = [&](uint32_t p) -> int32_t {
-        if (!staged) return (int32_t)p;
-        return (p >> 31) ? (int32_t)((p >> kVBits) & kFieldMask) : __popc(p >> kVBits);
-    };
     if constexpr (kAll) {
-        // CSR offsets: scan of the tie counts within the tile.  Counts are
-        // almost always below 4: the run scan is then two ballots (the
-        // counts' bit planes).  The tile's total is published before the
-        // per-position stores of pass 2, so that later tiles rarely wait for
-        // it.
+        sum = (int32_t)__reduce_add_sync(kFull, (unsigned)sum);
+        if (lane == 0) sm.wtot[warp] = sum;
+        if (warp == kWarps - 1) {
+            const long long ex = place_tile(s, tile, num_cover_tiles(n, TP), n, sm.ttot, offsets);
+            if (lane == 0) sm.obase = ex;
+        }
+        __syncthreads();
+        long long o0 = sm.obase;
+        {
+            const int32_t t = lane < warp ? sm.wtot[lane < kWarps ? lane : 0] : 0;
+            o0 += (int32_t)__reduce_add_sync(kFull, (unsigned)t);
+        }
+        // starts[o0 ..]: 32-bit indices from here; entries past the capacity are not written
+        const long long room = capacity - o0;
+        const int32_t lim = room < 0 ? 0 : (room > 0x7fffffff ? 0x7fffffff : (int32_t)room);
+        int32_t* out = starts + o0;
+        const bool far = sm.far != 0;
+        int32_t run = 0;
 #pragma unroll
         for (int q = 0; q < kChunksPerWarp; ++q) {
-            const int32_t cq = count_of(pk[q]);
-            int ex, tot;
-            const unsigned big = __ballot_sync(kFull, cq > 3);
-            if (big == 0u) {                              // two bit planes of counts below 4
-                const unsigned b0 = __ballot_sync(kFull, cq & 1), b1 = __ballot_sync(kFull, cq & 2);
-                ex = __popc(b0 & below) + 2 * __popc(b1 & below);
-                tot = __popc(b0) + 2 * __popc(b1);
-            } else {
-                const int incl = warp_incl_scan(cq);
-                ex = incl - cq;
-                tot = __shfl_sync(kFull, incl, kWarp - 1);
-            }
-            RT[q][lane] = (unsigned)ex;               // exclusive prefix within the run
-            if (lane == 0) sm.chunk[q * kWarps + warp] = tot;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const int tot = scan_chunks<kChunks>(sm.chunk);
-            if (lane == 0) {
-                if (tile != s.hold_tile) publish(s.status_o, tile, tile == 0 ? kPrefix : kAggregate, tot);
-                sm.ttot = tot;
-            }
-        }
-    }
-
-    if constexpr (kAll) {
-        __syncthreads();
-        if (warp == 0) {
-            const int tot = sm.ttot;
-            const long long ex = (tile == 0) ? 0 : lookback(s.status_o, tile, s.err, s.qerr, s.spin_limit);
-            if (lane == 0) {
-                if (tile != 0 && tile != s.hold_tile) publish(s.status_o, tile, kPrefix, ex + tot);
-                sm.obase = ex;
-                if (tile == num_cover_tiles(n, TP) - 1) offsets[n] = ex + tot;
-            }
-        }
-        __syncthreads();
-        const long long obase = sm.obase;
-#pragma unroll
-        for (int q = 0; q < kChunksPerWarp; ++q) {
-            const int c = q * kWarps + warp;
-            const int32_t k = k0 + c * kWarp + lane;
-            long long o = obase + sm.chunk[c] + (int)RT[q][lane];
-            if (k < n) __stcs(reinterpret_cast<long long*>(offsets) + k, o);
-            const uint32_t p = pk[q];
-            const int32_t cq = count_of(p);
-            if (cq == 0) continue;
-            // the second walk of Algorithm 4: every compact LLR of the
-            // longest length, ascending
-            if (staged && !(p >> 31)) {
-                const int32_t v0 = (int32_t)(p & kNone);
-                unsigned m = p >> kVBits;
-                while (m) {
-                    const int j = __ffs(m) - 1;
-                    m &= m - 1u;
-                    if (o < capacity) __stcs(starts + o, start_of(v0 + j));
-                    ++o;
-                }
-            } else {
-                int32_t lw, hi;
-                window(c, lw, hi);
-                int32_t bq;                                       // the longest length, again
-                if (staged) {
-                    bq = SCL[p & kNone];
+            const int32_t k = k0 + (c0 + q) * kWarp + lane;
+            const int32_t cq = (int32_t)(pk[q] >> 16);
+            const unsigned two = __ballot_sync(kFull, cq > 1);
+            const unsigned one = __ballot_sync(kFull, cq & 1);
+            int tot = __popc(one);
+            int32_t o = run + __popc(one & below);
+            if (two) {
+                if (__ballot_sync(kFull, cq > 3) == 0u) {
+                    tot += 2 * __popc(two);
+                    o += 2 * __popc(two & below);
                 } else {
-                    int32_t vb_, ct_;
-                    best_of(lw, hi, bq, vb_, ct_);
+                    const int incl = warp_incl_scan(cq);
+                    tot = __shfl_sync(kFull, incl, kWarp - 1);
+                    o = run + incl - cq;
                 }
-                for (int32_t v = staged ? (int32_t)(p & kNone) : lw; v <= hi; ++v) {
-                    const int32_t len = staged ? SCL[v] : __ldg(gce + v) - __ldg(gcs + v) + 1;
-                    if (len == bq) {
-                        if (o < capacity) __stcs(starts + o, start_of(v));
-                        ++o;
+            }
+            run += tot;
+            if (k < n) __stcs(reinterpret_cast<long long*>(offsets) + k, o0 + o);
+            // every compact LLR of the longest length over k, ascending
+            int32_t left = cq < lim - o ? cq : lim - o;
+            int v = (int)(pk[q] & 0xffffu);
+            int32_t* p = out + o;
+            if (left > 0) __stcs(p, sm.ent[v].x);
+            if (two) {
+                while (--left > 0) {
+                    const int32_t d = nx[v];
+                    if (far && d == 255) {
+                        const int32_t L = sm.ent[v].y;
+                        v += d;
+                        while (v <= MS && sm.ent[v].y != L) ++v;
+                    } else {
+                        v += d;
                     }
+                    __stcs(++p, sm.ent[v].x);
                 }
+                __syncwarp();
             }
         }
     }
@@ -454,17 +549,17 @@ void launch_cover(int32_t n, const Scratch& s, int32_t* lr_len, int32_t* lr_star
                   int32_t* starts, long long capacity, bool all, int tiles_per, cudaStream_t stream) {
     if (!all) { offsets = nullptr; starts = nullptr; capacity = 0; }
     switch (tiles_per) {
-        case 1:
-            if (all) launch_cover_t<true, 1>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
-            else launch_cover_t<false, 1>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+        case 2:
+            if (all) launch_cover_t<true, 2>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+            else launch_cover_t<false, 2>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
             break;
         case 4:
             if (all) launch_cover_t<true, 4>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
             else launch_cover_t<false, 4>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
             break;
         default:
-            if (all) launch_cover_t<true, 2>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
-            else launch_cover_t<false, 2>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+            if (all) launch_cover_t<true, 1>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+            else launch_cover_t<false, 1>(n, s, lr_len, lr_start, offsets, starts, capacity, stream);
     }
 }
 

@@ -110,7 +110,7 @@ constexpr int kSegCap = 1024;      // strings per CTA a front end keeps in share
 // Kernel shape choices a query can take (picked by lr_autotune_*).
 struct Shape {
     bool tile_cover = true;        // the tile cover kernel (else the warp-segment one)
-    int cover_tiles_per = 2;       // its tile = kTile x this (1, 2 or 4)
+    int cover_tiles_per = 1;       // its tile = kTile x this (1, 2 or 4)
 };
 
 // Launches the whole query on `stream`: the front end (rank-order when sa is
