@@ -291,7 +291,8 @@ struct PartSmem {
     uint32_t* hist;      // nb: entries of the round per bucket, then slot counters
     uint32_t* loff;      // nb + 1: exclusive prefix of hist (staging offsets), in
                          // place of hist (the scan reads hist before it writes)
-    uint32_t* base;      // nb: the round's reserved offset in each bucket
+    uint32_t* base;      // nb: where the round's entries of a bucket go, minus loff: staged
+                         // entry i of bucket b belongs at index base[b] + i of all buckets
     uint32_t* stage;     // kPartRound entries in bucket order
     uint16_t* sbk;       // kPartRound bucket ids of stage[]
 };
@@ -311,6 +312,7 @@ __device__ __forceinline__ PartSmem part_smem(unsigned char* raw, int nb) {
 // rounded out to 16-byte multiples: at most kPartRound + 8 entries), at a
 // 16-byte-aligned offset after the counters; it overlaps the stage area,
 // which is written only after every thread has read its entries.
+constexpr int kSms = 152;                // of a GB300: grids of the kernels whose CTAs stay
 constexpr int kPartLcpCap = kPartRound + 8;
 constexpr int kPartLoadBytes = kPartRound * 4 + kPartLcpCap * 4;
 __host__ __device__ inline size_t part_load_offset(int nb) { return ((size_t)(2 * nb + 1) * 4 + 15) & ~(size_t)15; }
@@ -321,15 +323,21 @@ size_t part_smem_bytes(int nb) {
     return a > b ? a : b;
 }
 
-// level 2 loads per thread: counters and stage area only
-size_t part2_smem_bytes() { return (size_t)(2 * kSubPerSuper + 1) * 4 + (size_t)kPartRound * 6; }
+// Room for c entries in bucket b (of 2^log entries) by one global atomic:
+// the index base of PartSmem.  More entries than the bucket holds (the
+// positions are not a permutation) set *over; the caller then checks every
+// index before it writes.
+__device__ __forceinline__ uint32_t part_room(unsigned* cursor, int b, uint32_t c, uint32_t loff, int log, int* over) {
+    const uint32_t at = atomicAdd(cursor + (size_t)b * kCursorStride, c);
+    if (at + c > (1u << log)) *over = 1;
+    return ((uint32_t)b << log) + at - loff;
+}
 
 // Exclusive scan of hist[0..nb) into loff[0..nb] by the whole CTA
 // (kPartThreads threads, R consecutive buckets each, nb <= R * kPartThreads),
-// and one global atomic per non-empty bucket to reserve the round's room:
-// base[b] = old cursor.
+// and one global atomic per non-empty bucket to reserve the round's room.
 template <int R>
-__device__ __forceinline__ void part_reserve_r(const PartSmem& p, int nb, unsigned* cursor) {
+__device__ __forceinline__ void part_reserve_r(const PartSmem& p, int nb, unsigned* cursor, int log, int* over) {
     __shared__ uint32_t wsum[kPartThreads / kWarp];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t a[R], sum = 0;
@@ -355,7 +363,7 @@ __device__ __forceinline__ void part_reserve_r(const PartSmem& p, int nb, unsign
         const int b = R * tid + u;
         if (b < nb) {
             p.loff[b] = ex;
-            if (a[u]) p.base[b] = atomicAdd(cursor + (size_t)b * kCursorStride, a[u]);
+            if (a[u]) p.base[b] = part_room(cursor, b, a[u], ex, log, over);
         }
         ex += a[u];
     }
@@ -364,9 +372,10 @@ __device__ __forceinline__ void part_reserve_r(const PartSmem& p, int nb, unsign
 // The same by warp 0 alone, for at most kWarp * R buckets (R consecutive
 // buckets per lane); the other warps wait at the caller's next barrier.
 // Each lane writes the staging offsets of its own buckets in place of their
-// counts after reading them.
+// counts after reading them.  Buckets from `last` on get no room.
 template <int R>
-__device__ __forceinline__ void part_reserve_w(const PartSmem& p, int nb, unsigned* cursor) {
+__device__ __forceinline__ void part_reserve_w(const PartSmem& p, int nb, int last, unsigned* cursor, int log,
+                                               int* over) {
     if (threadIdx.x >= kWarp) return;
     const int lane = threadIdx.x;
     uint32_t a[R], sum = 0;
@@ -383,7 +392,7 @@ __device__ __forceinline__ void part_reserve_w(const PartSmem& p, int nb, unsign
         const int b = R * lane + u;
         if (b < nb) {
             p.loff[b] = ex;
-            if (a[u]) p.base[b] = atomicAdd(cursor + (size_t)b * kCursorStride, a[u]);
+            if (a[u] && b < last) p.base[b] = part_room(cursor, b, a[u], ex, log, over);
         }
         ex += a[u];
     }
@@ -416,10 +425,56 @@ __device__ __forceinline__ void part_scan_w(const PartSmem& p, int nb) {
 }
 
 // up to 2048 super-buckets (n <= 2^31 positions in super-buckets of 2^20)
-__device__ __forceinline__ void part_reserve(const PartSmem& p, int nb, unsigned* cursor) {
+__device__ __forceinline__ void part_reserve(const PartSmem& p, int nb, unsigned* cursor, int log, int* over) {
     static_assert(4 * kPartThreads >= 2048, "partition CTAs too small for 2048 super-buckets");
-    if (nb <= 2 * kPartThreads) part_reserve_r<2>(p, nb, cursor);
-    else part_reserve_r<4>(p, nb, cursor);
+    if (nb <= 2 * kPartThreads) part_reserve_r<2>(p, nb, cursor, log, over);
+    else part_reserve_r<4>(p, nb, cursor, log, over);
+}
+
+// The level-1 entries of a round whose counts are complete: staging offsets,
+// room in the super-buckets, the entries staged in bucket order and written
+// out (a warp store is one run per bucket it touches).  key: bucket << 16 |
+// slot, or ~0u for none; `over` is zero before.  Returns 1 when a
+// super-bucket gets more than 2^20 entries.  Called by the whole CTA after
+// the barrier that completes the counts.
+__device__ __forceinline__ unsigned level1_write(const PartSmem& P, int nb, const Scratch& s,
+                                                 const uint32_t (&ent)[kPartPer], const uint32_t (&key)[kPartPer],
+                                                 bool all_valid, int* over) {
+    const bool wscan = nb <= 8 * kWarp;
+    if (wscan) part_scan_w<8>(P, nb);
+    else part_reserve(P, nb, s.cursor1, kSuperLog, over);
+    __syncthreads();
+    if (wscan) {
+        for (int b = threadIdx.x; b < nb; b += kPartThreads) {
+            const uint32_t o = P.loff[b], c = P.loff[b + 1] - o;
+            if (c) P.base[b] = part_room(s.cursor1, b, c, o, kSuperLog, over);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kPartPer; ++j) {
+        if (!all_valid && key[j] == 0xffffffffu) continue;
+        const uint32_t b1 = key[j] >> 16;
+        const uint32_t o = P.loff[b1] + (key[j] & 0xffffu);
+        P.stage[o] = ent[j];
+        P.sbk[o] = (uint16_t)b1;
+    }
+    __syncthreads();
+    unsigned bad = 0;
+    if (all_valid && *over == 0) {                      // kPartRound entries, all with room
+#pragma unroll
+        for (int j = 0; j < kPartPer; ++j) {
+            const uint32_t i = j * kPartThreads + threadIdx.x;
+            s.ent1[P.base[P.sbk[i]] + i] = P.stage[i];
+        }
+    } else {
+        const uint32_t total = P.loff[nb];
+        for (uint32_t i = threadIdx.x; i < total; i += kPartThreads) {
+            const uint32_t b1 = P.sbk[i], idx = P.base[b1] + i;
+            if (idx - (b1 << kSuperLog) < (uint32_t)kSuper) s.ent1[idx] = P.stage[i];
+            else bad = 1;                               // more than 2^20 positions: not a permutation
+        }
+    }
+    return bad;
 }
 
 // Slot of this lane's entry in bucket b among the entries counted so far,
@@ -457,7 +512,7 @@ __device__ __forceinline__ uint32_t run_slot(uint32_t* hist, uint32_t b, bool va
 // in a super-bucket: the positions are not a permutation).
 __device__ __forceinline__ unsigned level1_scatter(const PartSmem& P, int nb, const Scratch& s, int32_t n,
                                                    const uint32_t (&p)[kPartPer], const int32_t (&L)[kPartPer],
-                                                   int cnt) {
+                                                   int cnt, int* over) {
     unsigned bad = 0;
     uint32_t ent[kPartPer], key[kPartPer];          // key: bucket << 16 | slot, or ~0u
 #pragma unroll
@@ -478,34 +533,8 @@ __device__ __forceinline__ unsigned level1_scatter(const PartSmem& P, int nb, co
         const uint32_t slot = run_slot(P.hist, b1, ok);     // the pairs come in runs of one super-bucket
         key[j] = ok ? ((b1 << 16) | slot) : 0xffffffffu;
     }
-    __syncthreads();
-    const bool wscan = nb <= 8 * kWarp;
-    if (wscan) part_scan_w<8>(P, nb);
-    else part_reserve(P, nb, s.cursor1);
-    __syncthreads();
-    if (wscan) {
-        for (int b = threadIdx.x; b < nb; b += kPartThreads) {
-            const uint32_t c = P.loff[b + 1] - P.loff[b];
-            if (c) P.base[b] = atomicAdd(s.cursor1 + (size_t)b * kCursorStride, c);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kPartPer; ++j) {
-        if (key[j] == 0xffffffffu) continue;
-        const uint32_t b1 = key[j] >> 16;
-        const uint32_t o = P.loff[b1] + (key[j] & 0xffffu);
-        P.stage[o] = ent[j];
-        P.sbk[o] = (uint16_t)b1;
-    }
-    __syncthreads();
-    const uint32_t total = P.loff[nb];
-    for (uint32_t i = threadIdx.x; i < total; i += kPartThreads) {
-        const uint32_t b1 = P.sbk[i];
-        const uint32_t idx = P.base[b1] + (i - P.loff[b1]);
-        if (idx < (uint32_t)kSuper) s.ent1[((size_t)b1 << kSuperLog) + idx] = P.stage[i];
-        else bad = 1;
-    }
-    return bad;
+    const bool all_valid = __syncthreads_and(cnt == kPartRound && !bad) != 0;
+    return bad | level1_write(P, nb, s, ent, key, all_valid, over);
 }
 
 // Level 1: Lemma 1 in rank order.  Each CTA takes kPartRound consecutive
@@ -527,7 +556,7 @@ k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t
     // its first entry (shift entries earlier).  Other rounds load per thread.
     const int32_t* Ssa = reinterpret_cast<const int32_t*>(smem_raw + part_load_offset(nb));
     const int32_t* Slcp = Ssa + kPartRound;
-    __shared__ int bulk_s, shift_s, sab_s;
+    __shared__ int bulk_s, shift_s, sab_s, over_s;
     __shared__ long long bbase_s, bnj_s;          // batch round: its string's offset and length
     if (threadIdx.x == 0) {
         int bk = 0, shift = 0, sab = 0;
@@ -566,6 +595,7 @@ k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t
                 }
             }
         }
+        over_s = 0;
         bulk_s = bk;
         shift_s = shift;
         sab_s = sab;
@@ -616,28 +646,41 @@ k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t
     if (sab && !mbar_wait(&load_bar, 0)) landed = false;
     if (kBatch && bulk && landed && !mbar_wait(&load_bar2, 0)) landed = false;
     if (!landed && threadIdx.x == 0) report(s, kErrTimeout);
+    if (bulk) {
+        // four consecutive ranks per thread and group: sa by one 16-byte
+        // load, the five lcp words from the two 16-byte loads around them
+        const uint32_t lim = kBatch ? bnj : (uint32_t)n;      // positions of the round's string
 #pragma unroll
-    for (int j = 0; j < kPartPer; ++j) {
-        const long long r = r0 + (long long)j * kPartThreads + threadIdx.x;
-        if (bulk) {
-            const int x = j * kPartThreads + (int)threadIdx.x;
-            if (!landed) { p[j] = 0xffffffffu; L[j] = 0; continue; }
-            uint32_t pl = (uint32_t)Ssa[x];
-            const int32_t a = Slcp[shift + x], c = Slcp[shift + x + 1];
-            int32_t Lj = a > c ? a : c;
+        for (int g = 0; g < kPartPer / 4; ++g) {
+            const int x = (g * kPartThreads + (int)threadIdx.x) * 4;
+            const int4 sv = *reinterpret_cast<const int4*>(Ssa + x);
+            const int4 wa = *reinterpret_cast<const int4*>(Slcp + x), wb = *reinterpret_cast<const int4*>(Slcp + x + 4);
+            int32_t w0 = wa.x, w1 = wa.y, w2 = wa.z, w3 = wa.w, w4 = wb.x;
             if constexpr (kBatch) {
-                if (x == 0 && (long long)bbase == r0 && bnj != 0 && a != 0) bad = 1;   // lcp sentinel
-                if (pl >= bnj) { bad = 1; pl = 0xffffffffu; }
-                else if (Lj < 0 || (uint32_t)Lj > bnj - pl) { bad = 1; Lj = 0; }
-                p[j] = (pl == 0xffffffffu) ? pl : bbase + pl;
-            } else {
-                if (pl >= (uint32_t)n) { bad = 1; pl = 0xffffffffu; }
-                else if (Lj < 0 || (long long)Lj > (long long)n - pl) { bad = 1; Lj = 0; }
-                p[j] = pl;
+                if (shift == 1) { w0 = wa.y; w1 = wa.z; w2 = wa.w; w3 = wb.x; w4 = wb.y; }
+                else if (shift == 2) { w0 = wa.z; w1 = wa.w; w2 = wb.x; w3 = wb.y; w4 = wb.z; }
+                else if (shift == 3) { w0 = wa.w; w1 = wb.x; w2 = wb.y; w3 = wb.z; w4 = wb.w; }
+                if (x == 0 && (long long)bbase == r0 && bnj != 0 && w0 != 0) bad = 1;   // lcp sentinel
             }
-            L[j] = Lj;
-        } else if (r < n) {
-            if (sab && !landed) { p[j] = 0xffffffffu; L[j] = 0; continue; }
+            const uint32_t pl[4] = {(uint32_t)sv.x, (uint32_t)sv.y, (uint32_t)sv.z, (uint32_t)sv.w};
+            const int32_t Lv[4] = {max(w0, w1), max(w1, w2), max(w2, w3), max(w3, w4)};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                // negative lengths are too long as unsigned ones
+                const bool in = landed && pl[c] < lim, fit = (uint32_t)Lv[c] <= lim - pl[c];
+                if (!(in && fit)) bad = 1;
+                p[g * 4 + c] = in ? bbase + pl[c] : 0xffffffffu;
+                L[g * 4 + c] = fit ? Lv[c] : 0;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kPartPer; ++j) {
+            const long long r = r0 + (long long)j * kPartThreads + threadIdx.x;
+            p[j] = 0xffffffffu;
+            L[j] = 0;
+            if (r >= n) continue;
+            if (sab && !landed) continue;
             uint32_t pl = sab ? (uint32_t)Ssa[j * kPartThreads + (int)threadIdx.x] : (uint32_t)__ldcs(sa + r);
             long long base = 0, nj = n, lidx = r;
             if constexpr (kBatch) {
@@ -645,67 +688,36 @@ k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t
                 base = sv.at(hint);
                 nj = sv.at(hint + 1) - base;
                 lidx = r + hint;
-                if (base < 0 || nj < 1 || base + nj > n || r < base) {     // bad offset table
-                    bad = 1; p[j] = 0xffffffffu; L[j] = 0; continue;
-                }
+                if (base < 0 || nj < 1 || base + nj > n || r < base) { bad = 1; continue; }   // bad offset table
             }
             const int32_t a = __ldcs(lcp + lidx), c = __ldg(lcp + lidx + 1);
             if (kBatch && ((r == base && a != 0) || (r == base + nj - 1 && c != 0))) bad = 1;   // lcp sentinels
             int32_t Lj = a > c ? a : c;
-            if (pl >= (uint32_t)nj) { bad = 1; pl = 0xffffffffu; }
-            else if (Lj < 0 || (long long)Lj > nj - pl) { bad = 1; Lj = 0; }
-            p[j] = (pl == 0xffffffffu) ? pl : (uint32_t)(base + pl);
+            if (pl >= (uint32_t)nj) { bad = 1; continue; }
+            if (Lj < 0 || (long long)Lj > nj - pl) { bad = 1; Lj = 0; }
+            p[j] = (uint32_t)(base + pl);
             L[j] = Lj;
-        } else {
-            p[j] = 0xffffffffu; L[j] = 0;
         }
     }
     // the steps of level1_scatter, with one shared atomic per entry (pairs in
-    // rank order come in no runs), kept inline here (as a call they cost this
-    // kernel 3 %: more register spills)
+    // rank order come in no runs)
     uint32_t ent[kPartPer], key[kPartPer];          // key: bucket << 16 | slot, or ~0u
+    bool valid = true;
 #pragma unroll
     for (int j = 0; j < kPartPer; ++j) {
-        const long long r = r0 + (long long)j * kPartThreads + threadIdx.x;
-        key[j] = 0xffffffffu;
-        if (r >= n) continue;
         const uint32_t pj = p[j];
-        if (pj >= (uint32_t)n) { bad = 1; continue; }
+        key[j] = 0xffffffffu;
+        if (pj >= (uint32_t)n) { valid = false; continue; }
         const int32_t Lj = L[j];
         uint32_t field = (uint32_t)Lj;
         if (field >= kEsc12) { field = kEsc12; s.lbig[pj] = Lj; }
         if ((pj & (kBucket - 1)) == kBucket - 1) s.halo[(pj >> kBucketLog) + 1] = Lj;
         const uint32_t b1 = pj >> kSuperLog;
-        ent[j] = ((pj & (kSuper - 1)) << 12) | field;
+        ent[j] = (pj << 12) | field;
         key[j] = (b1 << 16) | atomicAdd(&P.hist[b1], 1u);
     }
-    __syncthreads();
-    const bool wscan = nb <= 8 * kWarp;
-    if (wscan) part_scan_w<8>(P, nb);
-    else part_reserve(P, nb, s.cursor1);
-    __syncthreads();
-    if (wscan) {
-        for (int b = threadIdx.x; b < nb; b += kPartThreads) {
-            const uint32_t c = P.loff[b + 1] - P.loff[b];
-            if (c) P.base[b] = atomicAdd(s.cursor1 + (size_t)b * kCursorStride, c);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kPartPer; ++j) {
-        if (key[j] == 0xffffffffu) continue;
-        const uint32_t b1 = key[j] >> 16;
-        const uint32_t o = P.loff[b1] + (key[j] & 0xffffu);
-        P.stage[o] = ent[j];
-        P.sbk[o] = (uint16_t)b1;
-    }
-    __syncthreads();
-    const uint32_t total = P.loff[nb];
-    for (uint32_t i = threadIdx.x; i < total; i += kPartThreads) {
-        const uint32_t b1 = P.sbk[i];
-        const uint32_t idx = P.base[b1] + (i - P.loff[b1]);
-        if (idx < (uint32_t)kSuper) s.ent1[((size_t)b1 << kSuperLog) + idx] = P.stage[i];
-        else bad = 1;                                   // more than 2^20 positions: sa is not a permutation
-    }
+    const bool all_valid = __syncthreads_and(valid) != 0;
+    bad |= level1_write(P, nb, s, ent, key, all_valid, &over_s);
     if (bad) report(s, kErrInput);
 }
 
@@ -728,6 +740,7 @@ __global__ void __launch_bounds__(kPartThreads, kPartBlocks)
 k_rank_win(const int32_t* __restrict__ rank, int32_t n, Scratch s, int tma) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned long long load_bar;
+    __shared__ int over_s;                            // not read: every window index is checked below
     const int nw = (int)s.nwins;                      // <= kMaxWins
     const PartSmem P = part_smem(smem_raw, nw);       // counters; the stage area is the 8-byte one below
     unsigned long long* stage = reinterpret_cast<unsigned long long*>(smem_raw + win_stage_offset(nw));
@@ -765,8 +778,8 @@ k_rank_win(const int32_t* __restrict__ rank, int32_t n, Scratch s, int tma) {
         key[j] = (w << 16) | atomicAdd(&P.hist[w], 1u);
     }
     __syncthreads();
-    if (nw <= 2 * kWarp) part_reserve_w<2>(P, nw, s.cursor_w);
-    else part_reserve(P, nw, s.cursor_w);
+    if (nw <= 2 * kWarp) part_reserve_w<2>(P, nw, nw, s.cursor_w, kWinLog, &over_s);
+    else part_reserve(P, nw, s.cursor_w, kWinLog, &over_s);
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kPartPer; ++j) {
@@ -779,10 +792,8 @@ k_rank_win(const int32_t* __restrict__ rank, int32_t n, Scratch s, int tma) {
     __syncthreads();
     const uint32_t total = P.loff[nw];
     for (uint32_t t = threadIdx.x; t < total; t += kPartThreads) {
-        const uint32_t w = sbk[t];
-        const uint32_t slot = P.base[w] + (t - P.loff[w]);
-        const long long idx = ((long long)w << kWinLog) + slot;
-        if (slot < (1u << kWinLog) && idx < n) s.went[idx] = stage[t];
+        const uint32_t w = sbk[t], idx = P.base[w] + t;
+        if (idx - (w << kWinLog) < (1u << kWinLog) && idx < (uint32_t)n) s.went[idx] = stage[t];
         else bad = 1;                                 // a window overflows: rank is not a permutation
     }
     if (bad) report(s, kErrInput);
@@ -799,6 +810,8 @@ k_part1_win(const int32_t* __restrict__ lcp, int32_t n, Scratch s) {
     const uint32_t fill = __ldcg(s.cursor_w + (size_t)w * kCursorStride);
     const long long wsize = ((long long)n - (w << kWinLog) < (1LL << kWinLog)) ? (long long)n - (w << kWinLog)
                                                                                 : (1LL << kWinLog);
+    __shared__ int over_s;
+    if (threadIdx.x == 0) over_s = 0;
     for (int b = threadIdx.x; b < nb; b += kPartThreads) P.hist[b] = 0;
     unsigned bad = 0;
     if (q == 0 && threadIdx.x == 0) {
@@ -834,116 +847,169 @@ k_part1_win(const int32_t* __restrict__ lcp, int32_t n, Scratch s) {
         if (Lj < 0 || (long long)Lj > (long long)n - i) { bad = 1; Lj = 0; }
         L[j] = Lj;
     }
-    bad |= level1_scatter(P, nb, s, n, p, L, cnt);
+    bad |= level1_scatter(P, nb, s, n, p, L, cnt, &over_s);
     if (bad) report(s, kErrInput);
 }
 
-// Level 2: each CTA takes kPartRound entries of one super-bucket and splits
-// them into its kSubPerSuper buckets, entries <position mod 2^15, field>
-// (field = L, or kEsc17 when L is in lbig), the same way as level 1.
+// Level 2: rounds of kPartRound entries of one super-bucket, split into its
+// kSubPerSuper buckets the same way.  The entries stay as they are: a
+// bucket's CTA reads the position mod 2^15 from them.  CTAs stay and take
+// every gridDim.x-th round; the next round's entries arrive by a bulk copy
+// while this one is counted, staged and written.
 // kRuns: slots by run_slot, for level-1 entries that come clustered by
 // bucket (those of the rank-window front end).
 template <bool kRuns>
 __global__ void __launch_bounds__(kPartThreads, kPartBlocks)
-k_part2(int32_t n, Scratch s) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const PartSmem P = part_smem(smem_raw, kSubPerSuper);
+k_part2(int32_t n, Scratch s, int rounds) {
+    __shared__ __align__(16) uint32_t load[kPartRound];
+    __shared__ __align__(16) uint32_t stage[kPartRound];
+    __shared__ uint32_t cnt_s[2][kSubPerSuper + 1];     // counts, then staging offsets, of this round and the next
+    __shared__ uint32_t base_s[kSubPerSuper];
+    __shared__ int over_s;
+    __shared__ unsigned long long load_bar;
     constexpr int kChunksPerSuper = kSuper / kPartRound;
-    const long long b1 = blockIdx.x / kChunksPerSuper;
-    const int q = blockIdx.x % kChunksPerSuper;
-    const uint32_t fill = __ldcg(s.cursor1 + (size_t)b1 * kCursorStride);
-    if (threadIdx.x < kSubPerSuper) P.hist[threadIdx.x] = 0;
-    if (q == 0 && threadIdx.x == 0) {
-        const long long want = ((long long)n - b1 * kSuper < kSuper) ? (long long)n - b1 * kSuper : kSuper;
-        if ((long long)fill != want) report(s, kErrInput);
+    const int tid = threadIdx.x;
+    int c = blockIdx.x;
+    if (c >= rounds) return;
+    uint32_t fill = __ldcg(s.cursor1 + (size_t)(c / kChunksPerSuper) * kCursorStride);
+    if (tid == 0) {
+        mbar_init(&load_bar, 1);
+        mbar_fence_init();
+        mbar_arrive_tx(&load_bar, kPartRound * 4);
+        bulk_g2s(load, s.ent1 + (size_t)c * kPartRound, kPartRound * 4, &load_bar);
     }
-    __syncthreads();
-    const uint32_t i0 = (uint32_t)q * kPartRound;
-    if (i0 >= fill) return;                             // uniform over the CTA
-    const uint32_t* src = s.ent1 + ((size_t)b1 << kSuperLog);
-    uint32_t ent[kPartPer], key[kPartPer];
-#pragma unroll
-    for (int j = 0; j < kPartPer; ++j) {
-        const uint32_t i = i0 + j * kPartThreads + threadIdx.x;
-        ent[j] = (i < fill) ? __ldcs(src + i) : 0xffffffffu;
-    }
-#pragma unroll
-    for (int j = 0; j < kPartPer; ++j) {
-        const uint32_t i = i0 + j * kPartThreads + threadIdx.x;
-        if constexpr (kRuns) {
-            const bool ok = i < fill;
-            uint32_t b2 = 0;
-            if (ok) {
-                const uint32_t low20 = ent[j] >> 12, f12 = ent[j] & kEsc12;
-                b2 = low20 >> kBucketLog;
-                ent[j] = ((low20 & (kBucket - 1)) << 17) | (f12 == kEsc12 ? kEsc17 : f12);
-            }
-            const uint32_t slot = run_slot(P.hist, b2, ok);
-            key[j] = ok ? ((b2 << 16) | slot) : 0xffffffffu;
-        } else {
-            key[j] = 0xffffffffu;
-            if (i >= fill) continue;
-            const uint32_t low20 = ent[j] >> 12, f12 = ent[j] & kEsc12;
-            const uint32_t b2 = low20 >> kBucketLog;
-            ent[j] = ((low20 & (kBucket - 1)) << 17) | (f12 == kEsc12 ? kEsc17 : f12);
-            key[j] = (b2 << 16) | atomicAdd(&P.hist[b2], 1u);
-        }
-    }
-    __syncthreads();
-    const long long bb = b1 * kSubPerSuper;
-    const int nsub = (int)((s.nbuckets - bb < kSubPerSuper) ? s.nbuckets - bb : kSubPerSuper);
-    part_reserve_w<1>(P, nsub, s.cursor2 + (size_t)bb * kCursorStride);
+    if (tid < 2 * (kSubPerSuper + 1)) cnt_s[0][tid] = 0;
     __syncthreads();
     unsigned bad = 0;
+    for (int it = 0; c < rounds; ++it) {
+        const int b1 = c / kChunksPerSuper, q = c % kChunksPerSuper, next = c + (int)gridDim.x;
+        const long long bb = (long long)b1 * kSubPerSuper;
+        const int nsub = (int)((s.nbuckets - bb < kSubPerSuper) ? s.nbuckets - bb : kSubPerSuper);
+        const uint32_t i0 = (uint32_t)q * kPartRound;
+        const bool full = i0 + kPartRound <= fill;
+        if (q == 0 && tid == 0) {
+            const long long want = ((long long)n - (long long)b1 * kSuper < kSuper) ? (long long)n - (long long)b1 * kSuper : kSuper;
+            if ((long long)fill != want) bad = 1;
+        }
+        PartSmem P;
+        P.hist = P.loff = cnt_s[it & 1];
+        P.base = base_s;
+        const bool landed = mbar_wait(&load_bar, it & 1);
+        uint32_t ent[kPartPer], slot[kPartPer];
+        if (full) {                                     // four consecutive entries per load
 #pragma unroll
-    for (int j = 0; j < kPartPer; ++j) {
-        if (key[j] == 0xffffffffu) continue;
-        const uint32_t b2 = key[j] >> 16;
-        if ((int)b2 >= nsub) { bad = 1; continue; }
-        const uint32_t o = P.loff[b2] + (key[j] & 0xffffu);
-        P.stage[o] = ent[j];
-        P.sbk[o] = (uint16_t)b2;
-    }
-    __syncthreads();
-    const uint32_t total = P.loff[nsub];
-    for (uint32_t i = threadIdx.x; i < total; i += kPartThreads) {
-        const uint32_t b2 = P.sbk[i];
-        const uint32_t idx = P.base[b2] + (i - P.loff[b2]);
-        if (idx < (uint32_t)kBucket) s.ent2[((size_t)(bb + b2) << kBucketLog) + idx] = P.stage[i];
-        else bad = 1;
+            for (int g = 0; g < kPartPer / 4; ++g) {
+                const uint4 v = reinterpret_cast<const uint4*>(load)[g * kPartThreads + tid];
+                ent[4 * g] = v.x; ent[4 * g + 1] = v.y; ent[4 * g + 2] = v.z; ent[4 * g + 3] = v.w;
+            }
+#pragma unroll
+            for (int j = 0; j < kPartPer; ++j)
+                slot[j] = kRuns ? run_slot(P.hist, ent[j] >> 27, true) : atomicAdd(&P.hist[ent[j] >> 27], 1u);
+        } else {
+#pragma unroll
+            for (int j = 0; j < kPartPer; ++j) {
+                const uint32_t i = j * kPartThreads + tid;
+                const bool in = i0 + i < fill;
+                ent[j] = in ? load[i] : 0u;
+                const bool ok = in && (int)(ent[j] >> 27) < nsub;   // a position at or past the last bucket: reported
+                if (in && !ok) bad = 1;
+                slot[j] = 0xffffffffu;
+                if (kRuns) {
+                    const uint32_t t = run_slot(P.hist, ent[j] >> 27, ok);
+                    if (ok) slot[j] = t;
+                } else if (ok) {
+                    slot[j] = atomicAdd(&P.hist[ent[j] >> 27], 1u);
+                }
+            }
+        }
+        if (__syncthreads_or(!landed)) {                // the copy never landed: reported, nothing more is loaded
+            if (tid == 0) report(s, kErrTimeout);
+            break;
+        }
+        if (tid == kPartThreads - 1 && next < rounds) {
+            fence_proxy_async_smem();
+            mbar_arrive_tx(&load_bar, kPartRound * 4);
+            bulk_g2s(load, s.ent1 + (size_t)next * kPartRound, kPartRound * 4, &load_bar);
+        }
+        if (next < rounds) fill = __ldcg(s.cursor1 + (size_t)(next / kChunksPerSuper) * kCursorStride);
+        if (tid < kWarp) {
+            if (tid == 0) over_s = 0;
+            __syncwarp();
+            if (full && tid >= nsub && P.hist[tid]) over_s = 1;
+        }
+        part_reserve_w<1>(P, kSubPerSuper, nsub, s.cursor2 + (size_t)bb * kCursorStride, kBucketLog, &over_s);
+        __syncthreads();
+        if (tid <= kSubPerSuper) cnt_s[(it & 1) ^ 1][tid] = 0;
+#pragma unroll
+        for (int j = 0; j < kPartPer; ++j)
+            if (full || slot[j] != 0xffffffffu) stage[P.loff[ent[j] >> 27] + slot[j]] = ent[j];
+        const uint32_t total = P.loff[kSubPerSuper];
+        __syncthreads();
+        uint32_t* dst = s.ent2 + ((size_t)bb << kBucketLog);
+        if (full && over_s == 0) {
+#pragma unroll
+            for (int j = 0; j < kPartPer; ++j) {
+                const uint32_t i = j * kPartThreads + tid;
+                const uint32_t e = stage[i];
+                dst[P.base[e >> 27] + i] = e;
+            }
+        } else {
+            for (uint32_t i = tid; i < total; i += kPartThreads) {
+                const uint32_t e = stage[i], b2 = e >> 27, idx = P.base[b2] + i;
+                if ((int)b2 < nsub && idx - (b2 << kBucketLog) < (uint32_t)kBucket) dst[idx] = e;
+                else bad = 1;
+            }
+        }
+        c = next;
     }
     if (bad) report(s, kErrInput);
 }
 
 // One bucket of kBucket positions per CTA: lengths scattered into shared
 // memory by position, usefulness flags (K1), compaction (K2) and the
-// bucket's place in LLRc by look-back (K3).  Each warp owns a contiguous
-// range of 64 runs of 32 positions, so L_{k-1} comes from the lane to the
-// left (or the previous run's last lane).
-constexpr uint16_t kUnset = 0xfffeu;                  // no length field takes this value
-constexpr uint32_t kUnset2 = 0xfffefffeu;
-__global__ void __launch_bounds__(kBucketThreads)
+// bucket's place in LLRc by look-back (K3).
+//
+// A position's word is the low half of its entry: the 12-bit length field
+// under the low four bits of the position.  XOR with those four bits (a
+// constant pattern per eight positions) leaves the plain field, and anything
+// else above bit 11 means that the position was never written (the words
+// start with the four bits inverted): sa gave another one twice.
+//
+// Each warp owns 2048 positions as eight chunks of 256, eight consecutive
+// positions per lane: one 16-byte load gives a lane its lengths, the flags
+// are sign bits shifted together, and the kept positions of a chunk are
+// listed in shared memory so that LLRc is written in whole runs.  2^26
+// positions of English take 114 us (67 M warp instructions); with a ballot
+// per run of 32 positions and one store per flagged lane it was 190 us
+// (156 M).
+constexpr int kBktChunk = 256;                                   // = kSeg: seg_cbase falls out of the chunk counts
+__device__ __forceinline__ uint32_t bucket_pattern(int x, int pair) {   // position bits of words x + 2 pair, x + 2 pair + 1
+    const uint32_t lo = (uint32_t)((x & 8) + 2 * pair);
+    return (lo << 12) | ((lo + 1) << 28);
+}
+__global__ void __launch_bounds__(kBucketThreads, 3)
 k_bucket_llr(int32_t n, Scratch s) {
-    constexpr int kChunks = kBucket / kWarp;                 // 1024 runs of 32 positions
+    constexpr int kChunks = kBucket / kBktChunk;             // 128
     constexpr int kWarps = kBucketThreads / kWarp;           // 16
-    constexpr int kRunsPerWarp = kChunks / kWarps;           // 64
+    constexpr int kPerWarp = kChunks / kWarps;               // 8
     constexpr int kTilesPerBucket = kBucket / kTile;         // 16
+    static_assert(kBktChunk == kSeg && kPerWarp * kBktChunk == kTile, "chunk, segment and tile sizes");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint16_t* sL = reinterpret_cast<uint16_t*>(smem_raw);                        // kBucket lengths
-    unsigned* cmask = reinterpret_cast<unsigned*>(smem_raw + kBucket * 2);       // kChunks flag masks
-    int32_t* ccnt = reinterpret_cast<int32_t*>(cmask + kChunks);                 // kChunks run offsets
-    __shared__ int32_t wsum[kWarps];
+    uint16_t* sL = reinterpret_cast<uint16_t*>(smem_raw);                        // kBucket words
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem_raw + kBucket * 2);        // kBktChunk kept positions per warp
+    __shared__ int32_t ccnt[kChunks];
     __shared__ long long b_s, base_s;
     __shared__ int32_t total_s;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) b_s = atomicAdd(&s.tickets[1], 1u);
-    {
-        // every length starts as kUnset: a position left unset after the
-        // scatter means sa gave another one twice
-        const uint4 u = make_uint4(kUnset2, kUnset2, kUnset2, kUnset2);
-        uint4* d = reinterpret_cast<uint4*>(sL);
-        for (int i = tid; i < kBucket / 8; i += kBucketThreads) d[i] = u;
+    for (int i = tid; i < kBucket / 8; i += kBucketThreads) {
+        uint4 u;
+        u.x = bucket_pattern(8 * i, 0) ^ 0xf000f000u;
+        u.y = bucket_pattern(8 * i, 1) ^ 0xf000f000u;
+        u.z = bucket_pattern(8 * i, 2) ^ 0xf000f000u;
+        u.w = bucket_pattern(8 * i, 3) ^ 0xf000f000u;
+        reinterpret_cast<uint4*>(sL)[i] = u;
     }
     __syncthreads();
     const long long b = b_s;
@@ -955,97 +1021,142 @@ k_bucket_llr(int32_t n, Scratch s) {
     const uint32_t fill = __ldcg(s.cursor2 + (size_t)b * kCursorStride);
     unsigned bad = fill != (uint32_t)cnt;
     const int nent = (int)(fill < (uint32_t)cnt ? fill : (uint32_t)cnt);
-    // eight loads in flight per thread before any of them is used
-    constexpr int kUnroll = 8;
-    for (int i0 = 0; i0 < nent; i0 += kBucketThreads * kUnroll) {
-        uint32_t e[kUnroll];
+    if (nent == kBucket) {
+        constexpr int kUnroll = 4;                           // loads of four entries in flight per thread
+        const uint4* src = reinterpret_cast<const uint4*>(ent) + tid;
+        for (int i0 = 0; i0 < kBucket / 4; i0 += kBucketThreads * kUnroll) {
+            uint4 e[kUnroll];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            const int i = i0 + u * kBucketThreads + tid;
-            e[u] = (i < nent) ? __ldcs(ent + i) : 0u;
+            for (int u = 0; u < kUnroll; ++u) e[u] = __ldcs(src + i0 + u * kBucketThreads);
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                sL[(e[u].x >> 12) & (kBucket - 1)] = (uint16_t)e[u].x;
+                sL[(e[u].y >> 12) & (kBucket - 1)] = (uint16_t)e[u].y;
+                sL[(e[u].z >> 12) & (kBucket - 1)] = (uint16_t)e[u].z;
+                sL[(e[u].w >> 12) & (kBucket - 1)] = (uint16_t)e[u].w;
+            }
         }
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-            if (i0 + u * kBucketThreads + tid >= nent) continue;
-            const uint32_t low = e[u] >> 17, f = e[u] & kEsc17;
-            if (low < (uint32_t)cnt) sL[low] = (uint16_t)(f == kEsc17 ? 0xffffu : f);
+    } else {
+        for (int i = tid; i < nent; i += kBucketThreads) {
+            const uint32_t e = __ldcs(ent + i), low = (e >> 12) & (kBucket - 1);
+            if (low < (uint32_t)cnt) sL[low] = (uint16_t)e;
             else bad = 1;
         }
     }
     __syncthreads();
-    auto len_at = [&](int x) -> int32_t {                    // L of position k0 + x, 0 <= x < cnt
-        const uint32_t f = sL[x];
-        return f == 0xffffu ? __ldcg(s.lbig + k0 + x) : (int32_t)f;
+    // L of position k0 + x, 0 <= x < cnt; a position never written counts as 0
+    auto len_at = [&](int x) -> int32_t {
+        const uint32_t f = (uint32_t)sL[x] ^ ((uint32_t)(x & 15) << 12);
+        return f < kEsc12 ? (int32_t)f : (f == kEsc12 ? __ldcg(s.lbig + k0 + x) : 0);
     };
 
-    // K1 flags, one ballot per run, runs of a warp contiguous
-    int32_t left = 0;                                        // L of the position before the run
+    // K1: the flags of a lane's eight positions per chunk, first position in the top bit
+    uint32_t flags[kPerWarp / 4] = {};                       // eight bits per chunk
+    uint32_t last = 0;                                       // field of the position before the chunk
     {
-        const int x0 = warp * kRunsPerWarp * kWarp;
-        left = (x0 == 0) ? ((k0 > 0) ? __ldcg(s.halo + b) : 0) : (x0 - 1 < cnt ? len_at(x0 - 1) : 0);
+        const int xw = warp * kTile;
+        if (xw > 0 && xw - 1 < cnt) last = min(((uint32_t)sL[xw - 1] ^ 0xf000u) & 0xffffu, kEsc12);
+        if (xw == 0 && k0 > 0) last = min((uint32_t)__ldcg(s.halo + b), kEsc12);
     }
-    for (int r = 0; r < kRunsPerWarp; ++r) {
-        const int c = warp * kRunsPerWarp + r;
-        const int x = c * kWarp + lane;
-        if (x < cnt && sL[x] == kUnset) bad = 1;
-        const int32_t L = (x < cnt) ? len_at(x) : 0;
-        int32_t prev = __shfl_up_sync(kFull, L, 1);
-        if (lane == 0) prev = left;
-        left = __shfl_sync(kFull, L, kWarp - 1);
-        const unsigned m = __ballot_sync(kFull, x < cnt && L > 0 && L >= prev);
-        if (lane == 0) { cmask[c] = m; ccnt[c] = __popc(m); }
+#pragma unroll
+    for (int q = 0; q < kPerWarp; ++q) {
+        const int x = warp * kTile + q * kBktChunk + lane * 8;
+        uint4 w = *reinterpret_cast<const uint4*>(sL + x);
+        w.x ^= bucket_pattern(x, 0);
+        w.y ^= bucket_pattern(x, 1);
+        w.z ^= bucket_pattern(x, 2);
+        w.w ^= bucket_pattern(x, 3);
+        const uint32_t m = __vmaxu2(__vmaxu2(w.x, w.y), __vmaxu2(w.z, w.w));
+        const bool odd = (m & 0xffffu) >= kEsc12 || (m >> 16) >= kEsc12;
+        uint32_t prev = __shfl_up_sync(kFull, w.w >> 16, 1);
+        if (lane == 0) prev = last;
+        last = min(__shfl_sync(kFull, w.w >> 16, kWarp - 1), kEsc12);
+        uint32_t f = 0;
+        if (__any_sync(kFull, odd)) {
+            // a length from lbig, a position never written or past the end
+            int32_t before = x > 0 ? (x - 1 < cnt ? len_at(x - 1) : 0) : (k0 > 0 ? __ldcg(s.halo + b) : 0);
+            for (int j = 0; j < 8; ++j) {
+                if (x + j < cnt && ((uint32_t)sL[x + j] ^ ((uint32_t)((x + j) & 15) << 12)) > kEsc12) bad = 1;
+                const int32_t l = x + j < cnt ? len_at(x + j) : 0;
+                f = 2 * f + (l > 0 && l >= before);
+                before = l;
+            }
+        } else {
+            const uint32_t l[8] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16,
+                                   w.z & 0xffffu, w.z >> 16, w.w & 0xffffu, w.w >> 16};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {                     // sign of l - max(prev, 1): 1 = dropped
+                f = __funnelshift_l(l[j] - max(prev, 1u), f, 1);
+                prev = l[j];
+            }
+            f ^= 0xffu;
+        }
+        flags[q / 4] |= (f & 0xffu) << (8 * (q % 4));
+        const int c = (int)__reduce_add_sync(kFull, (unsigned)__popc(f & 0xffu));
+        if (lane == 0) ccnt[warp * kPerWarp + q] = c;
     }
     if (bad) report(s, kErrInput);
     __syncthreads();
-    // exclusive scan of the 1024 run counts: 2 per thread
-    {
-        const int a0 = ccnt[2 * tid], a1 = ccnt[2 * tid + 1];
-        const int incl = warp_incl_scan(a0 + a1);
-        if (lane == kWarp - 1) wsum[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const int v = (lane < kWarps) ? wsum[lane] : 0;
-            const int wi = warp_incl_scan(v);
-            if (lane < kWarps) wsum[lane] = wi - v;
-            if (lane == kWarp - 1) total_s = wi;
-        }
-        __syncthreads();
-        const int ex = wsum[warp] + incl - a0 - a1;
-        ccnt[2 * tid] = ex;
-        ccnt[2 * tid + 1] = ex + a0;
-    }
-    __syncthreads();
+    // exclusive scan of the chunk counts and the bucket's place, by warp 0
     if (warp == 0) {
-        const long long ex = lookback_exclusive(s.status_b, b, total_s, s.err, s.qerr, s.spin_limit);
-        if (lane == 0) base_s = ex;
+        int a[kChunks / kWarp], sum = 0;
+#pragma unroll
+        for (int u = 0; u < kChunks / kWarp; ++u) { a[u] = ccnt[lane * (kChunks / kWarp) + u]; sum += a[u]; }
+        const int incl = warp_incl_scan(sum);
+        int ex = incl - sum;
+#pragma unroll
+        for (int u = 0; u < kChunks / kWarp; ++u) { ccnt[lane * (kChunks / kWarp) + u] = ex; ex += a[u]; }
+        const int total = __shfl_sync(kFull, incl, kWarp - 1);
+        const long long at = lookback_exclusive(s.status_b, b, total, s.err, s.qerr, s.spin_limit);
+        if (lane == 0) { base_s = at; total_s = total; }
     }
     __syncthreads();
     const long long base = base_s;
     // first LLRc entry of each tile and of each kSeg-position segment of the bucket
-    if (tid < kTilesPerBucket) {
-        const long long tile = b * kTilesPerBucket + tid;
-        if (tile < s.ntiles) s.tile_cbase[tile] = (int32_t)(base + ccnt[tid * (kTile / kWarp)]);
-        if (tile == s.ntiles - 1) s.tile_cbase[s.ntiles] = (int32_t)(base + total_s);
-    }
-    for (int j = tid; j < kBucket / kSeg; j += kBucketThreads) {
-        const long long sg = b * (kBucket / kSeg) + j;
-        if (sg < s.nsegs) s.seg_cbase[sg] = (int32_t)(base + ccnt[j * (kSeg / kWarp)]);
+    if (tid < kChunks) {
+        const long long sg = b * kChunks + tid;
+        const int32_t at = (int32_t)(base + ccnt[tid]);
+        if (sg < s.nsegs) s.seg_cbase[sg] = at;
         if (sg == s.nsegs - 1) s.seg_cbase[s.nsegs] = (int32_t)(base + total_s);
-    }
-    // K3: write the kept LLR's
-    for (int r = 0; r < kRunsPerWarp; ++r) {
-        const int c = warp * kRunsPerWarp + r;
-        const unsigned m = cmask[c];
-        if ((m >> lane) & 1u) {
-            const int x = c * kWarp + lane;
-            const long long o = base + ccnt[c] + __popc(m & ((1u << lane) - 1u));
-            s.cstart[o] = (int32_t)(k0 + x);
-            s.cend[o] = (int32_t)(k0 + x + len_at(x) - 1);
+        if (tid % kPerWarp == 0) {
+            const long long tile = b * kTilesPerBucket + tid / kPerWarp;
+            if (tile < s.ntiles) s.tile_cbase[tile] = at;
+            if (tile == s.ntiles - 1) s.tile_cbase[s.ntiles] = (int32_t)(base + total_s);
         }
+    }
+    // K3: list a chunk's kept positions, then write them
+    uint16_t* const mine = list + warp * kBktChunk;
+#pragma unroll
+    for (int q = 0; q < kPerWarp; ++q) {
+        const int x = warp * kTile + q * kBktChunk + lane * 8;
+        const uint32_t f = (flags[q / 4] >> (8 * (q % 4))) & 0xffu;
+        const int c = __popc(f);
+        const int incl = warp_incl_scan(c);
+        int o = incl - c;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (f & (0x80u >> j)) mine[o++] = (uint16_t)(x + j);
+        const int tot = __shfl_sync(kFull, incl, kWarp - 1);
+        __syncwarp();
+        const long long to = base + ccnt[warp * kPerWarp + q];
+        for (int i = lane; i < tot; i += kWarp) {
+            const int y = mine[i];
+            const int32_t k = (int32_t)(k0 + y);
+            s.cstart[to + i] = k;
+            s.cend[to + i] = k + len_at(y) - 1;
+        }
+        __syncwarp();
     }
 }
 
-size_t bucket_smem_bytes() { return (size_t)kBucket * 2 + (size_t)(kBucket / kWarp) * 8; }
+size_t bucket_smem_bytes() { return (size_t)kBucket * 2 + (size_t)(kBucketThreads / kWarp) * kBktChunk * 2; }
+
+template <bool kRuns>
+void launch_part2(int32_t n, const Scratch& s, cudaStream_t stream) {
+    const int rounds = (int)(((long long)n + kPartRound - 1) / kPartRound);   // the entries of every super-bucket but the last fill it
+    const int grid = rounds < kSms * kPartBlocks ? rounds : kSms * kPartBlocks;
+    k_part2<kRuns><<<grid, kPartThreads, 0, stream>>>(n, s, rounds);
+}
 
 void launch_partition(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                       cudaStream_t stream) {
@@ -1056,8 +1167,7 @@ void launch_partition(const int32_t* sa, const int32_t* lcp, int32_t n, const Sc
         k_part1<true><<<g1, kPartThreads, part_smem_bytes((int)s.nsupers), stream>>>(sa, lcp, n, s, segs, tma);
     else
         k_part1<false><<<g1, kPartThreads, part_smem_bytes((int)s.nsupers), stream>>>(sa, lcp, n, s, segs, tma);
-    const unsigned g2 = (unsigned)(s.nsupers * (kSuper / kPartRound));
-    k_part2<false><<<g2, kPartThreads, part2_smem_bytes(), stream>>>(n, s);
+    launch_part2<false>(n, s, stream);
 }
 
 void launch_rank_window_front(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s,
@@ -1067,8 +1177,7 @@ void launch_rank_window_front(const int32_t* rank, const int32_t* lcp, int32_t n
     k_rank_win<<<g0, kPartThreads, rank_win_smem_bytes((int)s.nwins), stream>>>(rank, n, s, tma);
     const unsigned g1 = (unsigned)(s.nwins * ((1 << kWinLog) / kPartRound));
     k_part1_win<<<g1, kPartThreads, part_scatter_smem_bytes((int)s.nsupers), stream>>>(lcp, n, s);
-    const unsigned g2 = (unsigned)(s.nsupers * (kSuper / kPartRound));
-    k_part2<true><<<g2, kPartThreads, part2_smem_bytes(), stream>>>(n, s);
+    launch_part2<true>(n, s, stream);
 }
 
 void launch_bucket_front(int32_t n, const Scratch& s, cudaStream_t stream) {
@@ -1087,11 +1196,7 @@ cudaError_t configure_front() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_part1_win, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)part_scatter_smem_bytes(2048));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_part2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part2_smem_bytes());
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_part2<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)part2_smem_bytes());
+    return e;
 }
 
 }  // namespace lr

@@ -29,8 +29,7 @@ constexpr int kPartThreads = 512;              // threads of a partition CTA
 constexpr int kPartBlocks = 4;                 // partition CTAs per SM (registers: 32 per thread)
 constexpr int kPartPer = 8;                    // entries per thread per partition CTA
 constexpr int kPartRound = kPartThreads * kPartPer;   // 4096 entries per partition CTA
-constexpr uint32_t kEsc12 = 0xfffu;            // 12-bit length field of level 1: value in lbig
-constexpr uint32_t kEsc17 = 0x1ffffu;          // 17-bit length field of level 2: value in lbig
+constexpr uint32_t kEsc12 = 0xfffu;            // 12-bit length field of the entries: value in lbig
 constexpr int kCursorStride = 32;              // one 128-byte line per partition cursor
 // Rank-window front end (rank without sa, one string): the pairs
 // <rank[i], i> partitioned by rank into windows of 2^22 ranks, so that the
@@ -56,7 +55,7 @@ struct Scratch {
     int32_t* cstart;               // n: compact LLR starts (ascending)
     int32_t* cend;                 // n: compact LLR ends   (ascending)
     uint32_t* ent1;                // nsupers x 2^20: level-1 entries <pos mod 2^20, min(L, 4095)>
-    uint32_t* ent2;                // nbuckets x 2^15: level-2 entries <pos mod 2^15, min(L, 2^17-1)>
+    uint32_t* ent2;                // nbuckets x 2^15: the same entries by bucket of 2^15 positions
     unsigned* cursor1;             // fill counts of ent1, one per kCursorStride words (cleared per query)
     unsigned* cursor2;             // fill counts of ent2, one per kCursorStride words (cleared per query)
     int32_t* lbig;                 // n: L of positions whose length field escaped
