@@ -20,14 +20,23 @@
 //    iff the strings and the first c * 2^r symbols are; a re-sorted suffix
 //    takes the rank of its old group's start plus the offset of its new
 //    group inside the old one;
-//  * rounds stop when all ranks differ; the suffix array is the positions
-//    sorted by rank (flattened index g holds the suffix of local rank
-//    g - off[j]);
-//  * lcp of each pair of sa neighbours: the round at which they parted
+//  * rounds stop when all ranks differ; the suffix array is kept from the
+//    first sort on: a re-sorted group's members move only within its range
+//    (flattened index g holds the suffix of local rank g - off[j]);
+//  * lcp of each pair of sa neighbours: pairs with different round-0 keys
+//    have it from the keys; of the others the round at which they parted
 //    gives it within a factor of two (first c * 2^(r-1) symbols equal, fewer
 //    than c * 2^r), binary lifting over the ranks of the earlier rounds
 //    (equal ranks at round q mean c * 2^q equal symbols) and fewer than c
 //    symbol comparisons give the rest.
+//
+// What bounds it: the radix sorts (CUB; two thirds of the time), then the
+// scattered rank stores and the lookups of k_lcp.  2^25 + 1 positions of
+// English take 7.9 ms and 2^28 73 ms; 10.5 and 89.7 ms with the suffix array
+// sorted once more from the final ranks, round 0's ranks sorted back to
+// position order at any size, separate marks, max-scans and updates, the
+// actives selected from all positions every round, keys of 32 + 26 instead of
+// 26 + 26 bits, and a thread per position coding all its symbols.
 #include <cuda_runtime.h>
 #include <cub/cub.cuh>
 #include <thrust/iterator/counting_iterator.h>
@@ -66,24 +75,68 @@ struct SymCodes {
     uint16_t code[256];
 };
 
-__global__ void k_keys0(const uint8_t* __restrict__ text, long long total, const int64_t* __restrict__ off,
-                        long long num, int csyms, int bps, SymCodes codes, uint64_t* __restrict__ key,
-                        int32_t* __restrict__ val, int32_t* __restrict__ end) {
+// Round-0 keys: a block's symbols are coded once into shared memory, a thread
+// rolls the keys of eight consecutive positions out of them (one symbol in,
+// one shifted out), and the keys leave through shared memory in order.  With
+// one thread per position reading and coding all its symbols itself 2^25
+// positions of English took 386 us.
+constexpr int kKeyThreads = 256, kKeyPer = 8, kKeyTile = kKeyThreads * kKeyPer;
+constexpr int kMaxSyms = 63;                             // one bit per symbol at least
+__global__ void __launch_bounds__(kKeyThreads)
+k_keys0(const uint8_t* __restrict__ text, long long total, const int64_t* __restrict__ off, long long num, int csyms,
+        int bps, SymCodes codes, uint64_t* __restrict__ key, int32_t* __restrict__ val, int32_t* __restrict__ end) {
     __shared__ uint16_t sc[256];
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) sc[t] = codes.code[t];
+    __shared__ __align__(16) uint16_t cd[kKeyTile + ((kMaxSyms + 7) & ~7) + 8];
+    __shared__ uint64_t out[kKeyTile + kKeyTile / kKeyPer];   // one word of padding per thread's keys
+    const int tid = threadIdx.x;
+    for (int t = tid; t < 256; t += kKeyThreads) sc[t] = codes.code[t];
     __syncthreads();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const long long j = string_of(off, num, i);
-    const long long e = __ldg(off + j + 1);
-    uint64_t k = (uint64_t)j;
-    for (int t = 0; t < csyms; ++t) {
-        const uint32_t c = (i + t < e) ? (uint32_t)sc[__ldg(text + i + t)] : 0u;
-        k = (k << bps) | c;
+    const long long g0 = (long long)blockIdx.x * kKeyTile;
+    const int need = kKeyTile + ((csyms + 7) & ~7) + 8;
+    for (int t = tid; t < need; t += kKeyThreads) cd[t] = g0 + t < total ? sc[__ldg(text + g0 + t)] : (uint16_t)0;
+    __syncthreads();
+    const long long i = g0 + (long long)tid * kKeyPer;
+    const int kbits = csyms * bps;
+    const uint64_t mask = (1ull << kbits) - 1;           // kbits <= 63
+    if (i < total) {
+        long long j = string_of(off, num, i), e = __ldg(off + j + 1);
+        uint64_t* o = out + tid * (kKeyPer + 1);
+        if (num == 1 || i + kKeyPer + csyms <= e) {      // (past the end of the text the codes are 0)
+            const uint64_t top = (uint64_t)j << kbits;
+            uint64_t k = 0;
+            for (int t0 = 0; t0 < csyms + kKeyPer - 1; t0 += 8) {
+                const uint4 w = *reinterpret_cast<const uint4*>(cd + tid * kKeyPer + t0);
+                const uint32_t c[8] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16,
+                                       w.z & 0xffffu, w.z >> 16, w.w & 0xffffu, w.w >> 16};
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    k = ((k << bps) | c[u]) & mask;
+                    const int q = t0 + u - (csyms - 1);  // the symbol completes the key of position i + q
+                    if (q >= 0 && q < kKeyPer) o[q] = top | k;
+                }
+            }
+            if (end)
+                for (int q = 0; q < kKeyPer; ++q)
+                    if (i + q < total) end[i + q] = (int32_t)e;
+        } else {                                         // across strings: each position by itself
+            for (int q = 0; q < kKeyPer && i + q < total; ++q) {
+                while (i + q >= e) { ++j; e = __ldg(off + j + 1); }
+                uint64_t k = (uint64_t)j;
+                for (int t = 0; t < csyms; ++t) k = (k << bps) | (i + q + t < e ? (uint64_t)cd[tid * kKeyPer + q + t] : 0ull);
+                o[q] = k;
+                if (end) end[i + q] = (int32_t)e;
+            }
+        }
     }
-    key[i] = k;
-    val[i] = (int32_t)i;
-    end[i] = (int32_t)e;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kKeyPer; ++u) {
+        const int x = u * kKeyThreads + tid;
+        if (g0 + x < total) {
+            key[g0 + x] = out[x + x / kKeyPer];
+            val[g0 + x] = (int32_t)(g0 + x);
+        }
+    }
 }
 
 // A rank word holds the rank in bits 0..30 and, in bit 31, whether the
@@ -95,15 +148,17 @@ constexpr uint32_t kRankMask = 0x7fffffffu;
 // Round r >= 1 keys of the suffixes still in groups of two or more (act[0..A),
 // ascending positions): (rank(i), rank(i + h) + 1, or 0 past the end of i's
 // string).
+// `end` (null for one string: `total`) holds the ends of the positions'
+// strings; the halves take sb bits each.
 __global__ void k_keys_act(const int32_t* __restrict__ act, long long A, const int32_t* __restrict__ rank,
-                           long long h, const int32_t* __restrict__ end, uint64_t* __restrict__ key,
-                           int32_t* __restrict__ val) {
+                           long long h, const int32_t* __restrict__ end, long long total, int sb,
+                           uint64_t* __restrict__ key, int32_t* __restrict__ val) {
     const long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= A) return;
     const long long i = __ldg(act + a);
-    const uint32_t second =
-        (i + h < __ldg(end + i)) ? ((uint32_t)__ldg(rank + i + h) & kRankMask) + 1u : 0u;
-    key[a] = ((uint64_t)((uint32_t)__ldg(rank + i) & kRankMask) << 32) | second;
+    const long long e = end ? (long long)__ldg(end + i) : total;
+    const uint32_t second = (i + h < e) ? ((uint32_t)__ldg(rank + i + h) & kRankMask) + 1u : 0u;
+    key[a] = ((uint64_t)((uint32_t)__ldg(rank + i) & kRankMask) << sb) | second;
     val[a] = (int32_t)i;
 }
 
@@ -113,134 +168,205 @@ struct ActiveAt {
     __device__ __forceinline__ bool operator()(int32_t i) const { return ((uint32_t)__ldg(rank + i) & kActiveBit) != 0; }
 };
 
-// Round 0, over all sorted keys: head[g] = g where key g starts a group of
-// equal keys, else 0; the number of groups is added to *groups; sep[g] = 0
-// where g starts a group; flags[g] = 1 where g is in a group of two or
-// more.  A block takes kHeadsPer x 256 consecutive keys and adds its count
-// with one atomic: adds on the one counter serialise (one per 256 keys cost
-// ~5 ms at n = 256 Mi).
-constexpr int kHeadsThreads = 256;
-constexpr int kHeadsPer = 16;
-__global__ void __launch_bounds__(kHeadsThreads)
-k_heads(const uint64_t* __restrict__ key, long long total, int32_t* __restrict__ head,
-        unsigned long long* __restrict__ groups, uint8_t* __restrict__ sep, uint8_t* __restrict__ flags) {
-    __shared__ int wsum[kHeadsThreads / 32];
-    const long long g0 = (long long)blockIdx.x * (kHeadsThreads * kHeadsPer) + threadIdx.x;
-    int cnt = 0;
-#pragma unroll 4
-    for (int u = 0; u < kHeadsPer; ++u) {
-        const long long g = g0 + (long long)u * kHeadsThreads;
-        if (g < total) {
-            const uint64_t k = __ldg(key + g);
-            const bool h = (g == 0) || (k != __ldg(key + g - 1));
-            head[g] = h ? (int32_t)g : 0;
-            cnt += h;
-            if (h) sep[g] = 0;
-            flags[g] = !h || (g + 1 < total && __ldg(key + g + 1) == k);
+// Groups of equal sorted keys, a tile of kGrpTile per block: a bitmap of the
+// elements that start one, the last start before each of its words, and the
+// start of the group that runs into the tile (found from its first element by
+// doubling steps back, then halving: a few steps for the usual group).
+constexpr int kGrpThreads = 256, kGrpPer = 8, kGrpTile = kGrpThreads * kGrpPer;
+struct GroupMap {
+    unsigned bits[kGrpTile / 32 + 1];                    // the extra word: bit 0 = the element after the tile
+    int32_t last[kGrpTile / 32];                         // last start before the word, -1: before the tile
+    long long first;                                     // start of the group of the tile's first element
+};
+
+// The start of the run of elements equal (key >> shift) to element g.
+__device__ __forceinline__ long long run_start(const uint64_t* __restrict__ key, long long g, int shift) {
+    const uint64_t k = __ldg(key + g) >> shift;
+    long long step = 1, lo = -1;                         // lo: an element known to differ (or -1)
+    while (true) {
+        if (g - step < 0) break;
+        if ((__ldg(key + g - step) >> shift) != k) { lo = g - step; break; }
+        g -= step;
+        step *= 2;
+    }
+    while (g - lo > 1) {                                 // g is equal, lo is not
+        const long long mid = lo + (g - lo) / 2;
+        if ((__ldg(key + mid) >> shift) == k) g = mid; else lo = mid;
+    }
+    return g;
+}
+
+// One warp: last starts before the words.
+__device__ __forceinline__ void group_lasts(GroupMap& m) {
+    constexpr int kPer = kGrpTile / 32 / 32;             // 2
+    const int lane = threadIdx.x & 31;
+    int own[kPer], x = -1;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int w = lane * kPer + u;
+        const unsigned b = m.bits[w];
+        own[u] = b ? w * 32 + 31 - __clz(b) : -1;
+        x = max(x, own[u]);
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x = max(x, y);
+    }
+    int run = __shfl_up_sync(0xffffffffu, x, 1);
+    if (lane == 0) run = -1;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        m.last[lane * kPer + u] = run;
+        run = max(run, own[u]);
+    }
+}
+
+// The start of the group of element x of the tile at t0.
+__device__ __forceinline__ long long group_start(const GroupMap& m, long long t0, int x) {
+    const unsigned b = m.bits[x >> 5] & ((2u << (x & 31)) - 1u);
+    const int at = b ? (x & ~31) + 31 - __clz(b) : m.last[x >> 5];
+    return at >= 0 ? t0 + at : m.first;
+}
+
+__device__ __forceinline__ bool starts_group(const GroupMap& m, int x) { return (m.bits[x >> 5] >> (x & 31)) & 1u; }
+
+// Round 0, over all sorted keys: the rank word of each suffix (the start of
+// its group, with the active bit in groups of two or more) goes to its
+// position (kScatter) or stays in sorted order, sa takes the sorted
+// positions, sep is 0 where a group starts, and the lcp of neighbours in
+// different groups is the number of equal leading symbols of their keys.
+template <bool kScatter>
+__global__ void __launch_bounds__(kGrpThreads)
+k_rank0(const uint64_t* __restrict__ key, const int32_t* __restrict__ val, long long total, int kbits, int bps,
+        int32_t* __restrict__ rank, int32_t* __restrict__ sa, uint8_t* __restrict__ sep, int32_t* __restrict__ lcp) {
+    __shared__ GroupMap m;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long t0 = (long long)blockIdx.x * kGrpTile;
+#pragma unroll
+    for (int u = 0; u < kGrpPer; ++u) {
+        const int x = u * kGrpThreads + tid;
+        const long long g = t0 + x;
+        const uint64_t k = g < total ? __ldg(key + g) : 0;
+        uint64_t p = __shfl_up_sync(0xffffffffu, k, 1);
+        if (lane == 0 && g > 0 && g < total) p = __ldg(key + g - 1);
+        const bool head = g < total && (g == 0 || k != p);
+        const unsigned b = __ballot_sync(0xffffffffu, head || g >= total);
+        if (lane == 0) m.bits[u * (kGrpThreads / 32) + warp] = b;
+        if (head) {
+            const long long j = (long long)(k >> kbits);
+            const bool same = g > 0 && (long long)(p >> kbits) == j;
+            lcp[g + j] = same ? __clzll((long long)((k ^ p) << (64 - kbits))) / bps : 0;
         }
+        if (g < total) sep[g] = head ? 0 : 0xff;
     }
-    cnt = __reduce_add_sync(0xffffffffu, (unsigned)cnt);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = cnt;
+    if (tid == 0) {
+        const long long g = t0 + kGrpTile;
+        m.bits[kGrpTile / 32] = g >= total || __ldg(key + g) != __ldg(key + g - 1);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int w = 0; w < kHeadsThreads / 32; ++w) t += (unsigned long long)wsum[w];
-        if (t) atomicAdd(groups, t);
+    if (warp == 0) group_lasts(m);
+    if (tid == 32) m.first = (m.bits[0] & 1u) ? t0 : run_start(key, t0, 0);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kGrpPer; ++u) {
+        const int x = u * kGrpThreads + tid;
+        const long long g = t0 + x;
+        if (g >= total) break;
+        const bool act = !(starts_group(m, x) && starts_group(m, x + 1));
+        const int32_t word = (int32_t)((uint32_t)group_start(m, t0, x) | (act ? kActiveBit : 0u));
+        const int32_t v = __ldg(val + g);
+        if (kScatter) rank[v] = word; else rank[g] = word;
+        sa[g] = v;
     }
 }
 
-__global__ void k_scatter_rank(const int32_t* __restrict__ sorted, const int32_t* __restrict__ hp, long long total,
-                               int32_t* __restrict__ rank) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g < total) rank[sorted[g]] = hp[g];
-}
-
-// Round r >= 1, over the re-sorted keys key[0..A): mh[a] = a where key a
-// starts a new group, mo[a] = a where it starts a group of the previous
-// round (its first half, the old rank, changes); else 0.
-__global__ void k_marks(const uint64_t* __restrict__ key, long long A, int32_t* __restrict__ mh,
-                        int32_t* __restrict__ mo) {
-    const long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= A) return;
-    const uint64_t k = __ldg(key + a);
-    bool nh = true, oh = true;
-    if (a > 0) {
-        const uint64_t p = __ldg(key + a - 1);
-        nh = k != p;
-        oh = (k >> 32) != (p >> 32);
+// Round r >= 1, over the re-sorted keys key[0..A) (halves of sb bits): an old
+// group (rank g0 = its first sorted index) holds its re-sorted members at
+// a0 .. a0 + size - 1, so member a sits at sorted index g0 + a - a0 and its
+// new rank is the index of its new group's first member, g0 + ah - a0, with
+// the active bit when the new group has two or more members.  New group
+// starts inside an old group take sep = r.
+__global__ void __launch_bounds__(kGrpThreads)
+k_update(const uint64_t* __restrict__ key, const int32_t* __restrict__ val, long long A, int sb,
+         int32_t* __restrict__ rank, int32_t* __restrict__ sa, uint8_t* __restrict__ sep, int round) {
+    __shared__ GroupMap nm, om;                          // new and old groups
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long t0 = (long long)blockIdx.x * kGrpTile;
+    uint32_t old[kGrpPer];
+#pragma unroll
+    for (int u = 0; u < kGrpPer; ++u) {
+        const long long a = t0 + u * kGrpThreads + tid;
+        const uint64_t k = a < A ? __ldg(key + a) : 0;
+        uint64_t p = __shfl_up_sync(0xffffffffu, k, 1);
+        if (lane == 0 && a > 0 && a < A) p = __ldg(key + a - 1);
+        const bool nh = a >= A || a == 0 || k != p, oh = a >= A || a == 0 || (k >> sb) != (p >> sb);
+        const unsigned nb = __ballot_sync(0xffffffffu, nh), ob = __ballot_sync(0xffffffffu, oh);
+        if (lane == 0) {
+            nm.bits[u * (kGrpThreads / 32) + warp] = nb;
+            om.bits[u * (kGrpThreads / 32) + warp] = ob;
+        }
+        old[u] = (uint32_t)(k >> sb);
     }
-    mh[a] = nh ? (int32_t)a : 0;
-    mo[a] = oh ? (int32_t)a : 0;
+    if (tid == 0) {
+        const long long a = t0 + kGrpTile;
+        nm.bits[kGrpTile / 32] = a >= A || __ldg(key + a) != __ldg(key + a - 1);
+    }
+    __syncthreads();
+    if (warp == 0) group_lasts(nm);
+    if (warp == 1) group_lasts(om);
+    if (tid == 64) nm.first = (nm.bits[0] & 1u) ? t0 : run_start(key, t0, 0);
+    if (tid == 96) om.first = (om.bits[0] & 1u) ? t0 : run_start(key, t0, sb);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kGrpPer; ++u) {
+        const int x = u * kGrpThreads + tid;
+        const long long a = t0 + x;
+        if (a >= A) break;
+        const long long g0 = old[u], s0 = group_start(om, t0, x), hh = group_start(nm, t0, x);
+        const bool nh = starts_group(nm, x), act = !(nh && starts_group(nm, x + 1));
+        const int32_t v = __ldg(val + a);
+        rank[v] = (int32_t)((uint32_t)(g0 + (hh - s0)) | (act ? kActiveBit : 0u));
+        sa[g0 + (a - s0)] = v;
+        if (nh && s0 != a) sep[g0 + (a - s0)] = (uint8_t)round;
+    }
 }
 
-// Round r >= 1: an old group (rank g0 = its first sorted index) holds its
-// re-sorted members at a0 .. a0 + size - 1, so member a sits at sorted index
-// g0 + a - a0 and its new rank is the index of its new group's first member,
-// g0 + ah - a0 (ah, a0: max-scans of the marks), with the active bit when
-// the new group has two or more members.  New group starts inside an old
-// group take sep = r.
-__global__ void k_update(const uint64_t* __restrict__ key, const int32_t* __restrict__ val,
-                         const int32_t* __restrict__ ah, const int32_t* __restrict__ a0, long long A,
-                         int32_t* __restrict__ rank, uint8_t* __restrict__ sep, int round) {
-    const long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= A) return;
-    const uint64_t k = __ldg(key + a);
-    const long long g0 = (long long)(k >> 32), s0 = __ldg(a0 + a), hh = __ldg(ah + a);
-    const bool act = (a > 0 && __ldg(key + a - 1) == k) || (a + 1 < A && __ldg(key + a + 1) == k);
-    rank[__ldg(val + a)] = (int32_t)((uint32_t)(g0 + (hh - s0)) | (act ? kActiveBit : 0u));
-    if (hh == a && s0 != a) sep[g0 + (a - s0)] = (uint8_t)round;
-}
-
-// Round 0: the active bit on the ranks (in sorted order) of keys in groups
-// of two or more.
-__global__ void k_mark_active(int32_t* __restrict__ hp, const uint8_t* __restrict__ flags, long long total) {
+// String-local suffix array of a batch: index g lies in string j's range.
+__global__ void k_local_sa(int32_t* __restrict__ sa, long long total, const int64_t* __restrict__ off, long long num) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g < total && flags[g]) hp[g] = (int32_t)((uint32_t)hp[g] | kActiveBit);
+    if (g < total) sa[g] -= (int32_t)__ldg(off + string_of(off, num, g));
 }
 
-__global__ void k_iota(int32_t* __restrict__ v, long long total) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < total) v[i] = (int32_t)i;
-}
-
-// lcp of sorted neighbours g - 1, g of one string, written in the layout the
-// queries take (string j's n_j + 1 entries at off[j] + j), and the string-
-// local sa and rank (index g read as a rank for sa, as a position for rank:
-// both lie in string j's range [off[j], off[j+1])).  The two suffixes parted
-// at round r = sep[g]: their first csyms * 2^(r-1) symbols are equal (none
-// for r = 0) and fewer than csyms * 2^r are; the rest is found by binary
+// lcp of sorted neighbours g - 1, g that share their round-0 key, written in
+// the layout the queries take (string j's n_j + 1 entries at off[j] + j), and
+// the string-local rank.  The two suffixes parted at round r = sep[g] >= 1
+// (k_rank0 wrote the others): their first csyms * 2^(r-1) symbols are equal
+// and fewer than csyms * 2^r are; the rest is found by binary
 // lifting over the ranks of rounds r - 2 .. 0 (equal ranks at round q mean
 // csyms * 2^q more equal symbols, longest first), then fewer than csyms
 // symbol comparisons.
 __global__ void k_lcp(const uint8_t* __restrict__ text, long long total, const int64_t* __restrict__ off,
                       long long num, const int32_t* __restrict__ sorted, const int32_t* __restrict__ levels,
                       int rounds, int csyms, const uint8_t* __restrict__ sep, const int32_t* __restrict__ frank,
-                      int32_t* __restrict__ sa, int32_t* __restrict__ rank, int32_t* __restrict__ lcp) {
+                      int32_t* __restrict__ rank, int32_t* __restrict__ lcp) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= total) return;
     const long long j = string_of(off, num, g);
     const long long a = __ldg(off + j), e = __ldg(off + j + 1);
-    sa[g] = (int32_t)(sorted[g] - a);
     rank[g] = (int32_t)(frank[g] - a);
-    int32_t out = 0;
-    if (g > a) {
-        long long x = sorted[g - 1], y = sorted[g], l = 0;
-        int r = sep[g];
-        r = r < rounds ? r : rounds - 1;               // every index parts by the last round
-        if (r > 0) {
-            l = (long long)csyms << (r - 1);
-            x += l;
-            y += l;
-        }
-        for (int q = r - 2; q >= 0; --q) {
-            const long long len = (long long)csyms << q;
-            const int32_t* R = levels + (size_t)q * (size_t)total;
-            if (x < e && y < e && __ldg(R + x) == __ldg(R + y)) { l += len; x += len; y += len; }
-        }
-        for (int t = 0; t < csyms && x < e && y < e && __ldg(text + x) == __ldg(text + y); ++t) { ++l; ++x; ++y; }
-        out = (int32_t)l;
+    int r = sep[g];
+    if (r == 0) return;
+    r = r < rounds ? r : rounds - 1;                       // every index parts by the last round
+    long long l = (long long)csyms << (r - 1);
+    long long x = sorted[g - 1] + l, y = sorted[g] + l;
+    for (int q = r - 2; q >= 0; --q) {
+        const long long len = (long long)csyms << q;
+        const int32_t* R = levels + (size_t)q * (size_t)total;
+        if (x < e && y < e && __ldg(R + x) == __ldg(R + y)) { l += len; x += len; y += len; }
     }
-    lcp[g + j] = out;                                  // lcp[0] of string j is 0 (g == a)
+    for (int t = 0; t < csyms && x < e && y < e && __ldg(text + x) == __ldg(text + y); ++t) { ++l; ++x; ++y; }
+    lcp[g + j] = (int32_t)l;
 }
 
 // The closing sentinel lcp[n_j] = 0 of every string (and the only entry of
@@ -261,26 +387,31 @@ __global__ void k_check_off(const int64_t* __restrict__ off, long long num, long
     if (b) atomicOr(bad, 1ull);
 }
 
-struct MaxOp {
-    __device__ __forceinline__ int32_t operator()(int32_t a, int32_t b) const { return a > b ? a : b; }
-};
-
 inline unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 size_t sort_temp_bytes(long long n) {
-    size_t a = 0, b = 0, c = 0;
+    size_t a = 0, c = 0;
     cub::DoubleBuffer<uint64_t> keys(nullptr, nullptr);
     cub::DoubleBuffer<int32_t> vals(nullptr, nullptr), pos(nullptr, nullptr);
     cub::DeviceRadixSort::SortPairs(nullptr, a, keys, vals, (int)n, 0, 64, (cudaStream_t)0);
-    cub::DeviceScan::InclusiveScan(nullptr, b, (int32_t*)nullptr, (int32_t*)nullptr, MaxOp{}, (int)n, (cudaStream_t)0);
     cub::DeviceRadixSort::SortPairs(nullptr, c, pos, vals, (int)n, 0, 32, (cudaStream_t)0);
     size_t d = 0;
     cub::DeviceSelect::If(nullptr, d, thrust::counting_iterator<int32_t>(0), (int32_t*)nullptr,
                           (unsigned long long*)nullptr, (int)n, ActiveAt{nullptr}, (cudaStream_t)0);
-    if (b > a) a = b;
+    if (d > a) a = d;
+    d = 0;
+    cub::DeviceSelect::If(nullptr, d, (const int32_t*)nullptr, (int32_t*)nullptr, (unsigned long long*)nullptr, (int)n,
+                          ActiveAt{nullptr}, (cudaStream_t)0);
     if (d > a) a = d;
     return (c > a ? c : a) + 256;
 }
+
+// Positions up to which round 0's ranks are scattered straight to position
+// order, while most of their 4-byte array stays in the 129 MB L2: at 2^25
+// positions the build takes 7.85 ms this way and 8.03 ms with the sort by
+// position; scattered 4-byte stores past L2 run at 27 G/s (10 ms for 2^28,
+// the sort 5).
+constexpr long long kScatterMax = 40LL << 20;
 
 inline size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -369,114 +500,88 @@ cudaError_t build_arrays_batch(const uint8_t* text, long long total, const int64
     while (bits < 31 && (1ll << bits) <= total) ++bits;
     cub::DoubleBuffer<uint64_t> keys(w.k0, w.k1);
     cub::DoubleBuffer<int32_t> vals(w.v0, w.v1);
-    e = cudaMemsetAsync(w.sep, 0xff, nn, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.misc, 0, 24, stream);
-    if (e != cudaSuccess) return e;
     // round 0: every suffix by its string and first csyms symbols
-    k_keys0<<<blocks(total, 256), 256, 0, stream>>>(text, total, off, num, csyms, bps, codes, keys.Current(),
-                                                    vals.Current(), w.end);
+    const bool one = num == 1;
+    k_keys0<<<blocks(total, kKeyTile), kKeyThreads, 0, stream>>>(text, total, off, num, csyms, bps, codes, keys.Current(),
+                                                                vals.Current(), one ? nullptr : w.end);
     size_t tb = w.tmp_bytes;
     e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, keys, vals, (int)total, 0, jobbits + bps * csyms, stream);
     if (e != cudaSuccess) return e;
-    uint8_t* flags = reinterpret_cast<uint8_t*>(keys.Alternate());
-    k_heads<<<blocks(total, kHeadsThreads * kHeadsPer), kHeadsThreads, 0, stream>>>(keys.Current(), total, w.head,
-                                                                                  w.misc, w.sep, flags);
+    // The suffix array is kept in sa (flattened) from here on.  The ranks go
+    // back to position order by scattered stores while their array fits L2,
+    // else by a radix sort keyed by position (streaming passes)
+    if (total <= kScatterMax) {
+        k_rank0<true><<<blocks(total, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), total,
+                                                                          bps * csyms, bps, w.levels, sa, w.sep, lcp);
+    } else {
+        k_rank0<false><<<blocks(total, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), total,
+                                                                           bps * csyms, bps, w.hp, sa, w.sep, lcp);
+        cub::DoubleBuffer<int32_t> pos(vals.Current(), vals.Alternate());
+        cub::DoubleBuffer<int32_t> rnk(w.hp, w.levels);
+        tb = w.tmp_bytes;
+        e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, pos, rnk, (int)total, 0, bits, stream);
+        if (e == cudaSuccess && rnk.Current() != w.levels)
+            e = cudaMemcpyAsync(w.levels, rnk.Current(), nn * 4, cudaMemcpyDeviceToDevice, stream);
+        if (e != cudaSuccess) return e;
+    }
+    // the active positions, ascending (their rank words are then read in
+    // order); only the suffixes in groups of two or more are sorted again
+    int32_t *act = w.head, *spare = w.hp;
     tb = w.tmp_bytes;
-    e = cub::DeviceScan::InclusiveScan(w.tmp, tb, w.head, w.hp, MaxOp{}, (int)total, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&w.groups_host, w.misc, 8, cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    e = cub::DeviceSelect::If(w.tmp, tb, thrust::counting_iterator<int32_t>(0), act, w.misc + 2, (int)total,
+                              ActiveAt{w.levels}, stream);
     if (e != cudaSuccess) return e;
     int rounds = 1;
-    const int32_t* sorted = nullptr;                       // the suffix array (flattened) at the end
-    if (w.groups_host == (unsigned long long)total) {
-        // all first keys differ: the sorted positions are the suffix array
-        k_scatter_rank<<<blocks(total, 256), 256, 0, stream>>>(vals.Current(), w.hp, total, w.levels);
-        sorted = vals.Current();
-    } else {
-        // the suffixes in groups of two or more (act, in w.head) are the only
-        // ones sorted again; then the ranks go back to position order by a
-        // radix sort keyed by position (streaming passes instead of one random
-        // 4-byte store per position)
-        long long A = 0;
-        k_mark_active<<<blocks(total, 256), 256, 0, stream>>>(w.hp, flags, total);
-        {
-            cub::DoubleBuffer<int32_t> pos(vals.Current(), vals.Alternate());
-            cub::DoubleBuffer<int32_t> rnk(w.hp, w.levels);
-            tb = w.tmp_bytes;
-            e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, pos, rnk, (int)total, 0, bits, stream);
-            if (e == cudaSuccess && rnk.Current() != w.levels)
-                e = cudaMemcpyAsync(w.levels, rnk.Current(), nn * 4, cudaMemcpyDeviceToDevice, stream);
-            if (e != cudaSuccess) return e;
-        }
-        // the active positions, ascending (their rank words are then read in order)
-        tb = w.tmp_bytes;
-        e = cub::DeviceSelect::If(w.tmp, tb, thrust::counting_iterator<int32_t>(0), w.head, w.misc + 2, (int)total,
-                                  ActiveAt{w.levels}, stream);
+    for (int r = 1;; ++r) {
+        e = cudaMemcpyAsync(&w.groups_host, w.misc + 2, 8, cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
         if (e != cudaSuccess) return e;
-        for (int r = 1;; ++r) {
-            e = cudaMemcpyAsync(&w.groups_host, w.misc + 2, 8, cudaMemcpyDeviceToHost, stream);
+        const long long A = (long long)w.groups_host;
+        if (A == 0) { rounds = r; break; }
+        if (r >= 40 || A > total) return cudaErrorUnknown;
+        if (r >= w.cap_rounds) {                          // more rounds than the level store holds
+            if (!grow) return cudaErrorMemoryAllocation;
+            IndexWork bigger;
+            e = bigger.alloc(w.cap_n, w.cap_rounds * 2);
+            if (e != cudaSuccess) return e;
+            e = cudaMemcpyAsync(bigger.levels, w.levels, (size_t)w.cap_rounds * nn * 4, cudaMemcpyDeviceToDevice,
+                                stream);
+            if (e == cudaSuccess && !one) e = cudaMemcpyAsync(bigger.end, w.end, nn * 4, cudaMemcpyDeviceToDevice, stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(bigger.sep, w.sep, nn, cudaMemcpyDeviceToDevice, stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(bigger.head, act, (size_t)A * 4, cudaMemcpyDeviceToDevice,
+                                                      stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-            if (e != cudaSuccess) return e;
-            A = (long long)w.groups_host;
-            if (A == 0) { rounds = r; break; }
-            if (r >= 40 || A > total) return cudaErrorUnknown;
-            if (r >= w.cap_rounds) {                          // more rounds than the level store holds
-                if (!grow) return cudaErrorMemoryAllocation;
-                IndexWork bigger;
-                e = bigger.alloc(w.cap_n, w.cap_rounds * 2);
-                if (e != cudaSuccess) return e;
-                e = cudaMemcpyAsync(bigger.levels, w.levels, (size_t)w.cap_rounds * nn * 4, cudaMemcpyDeviceToDevice,
-                                    stream);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(bigger.end, w.end, nn * 4, cudaMemcpyDeviceToDevice, stream);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(bigger.sep, w.sep, nn, cudaMemcpyDeviceToDevice, stream);
-                if (e == cudaSuccess) e = cudaMemcpyAsync(bigger.head, w.head, (size_t)A * 4, cudaMemcpyDeviceToDevice,
-                                                          stream);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-                if (e != cudaSuccess) { bigger.release(); return e; }
-                w.release();
-                w = bigger;
-                bigger.base = nullptr;                        // owned by w now
-                keys = cub::DoubleBuffer<uint64_t>(w.k0, w.k1);
-                vals = cub::DoubleBuffer<int32_t>(w.v0, w.v1);
-            }
-            const int32_t* prev = w.levels + (size_t)(r - 1) * nn;
-            int32_t* level = w.levels + (size_t)r * nn;
-            e = cudaMemcpyAsync(level, prev, nn * 4, cudaMemcpyDeviceToDevice, stream);   // settled ranks stay
-            if (e != cudaSuccess) return e;
-            const long long h = (long long)csyms << (r - 1);
-            k_keys_act<<<blocks(A, 256), 256, 0, stream>>>(w.head, A, prev, h, w.end, keys.Current(), vals.Current());
-            tb = w.tmp_bytes;
-            e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, keys, vals, (int)A, 0, 32 + bits, stream);
-            if (e != cudaSuccess) return e;
-            int32_t* mh = reinterpret_cast<int32_t*>(keys.Alternate());
-            int32_t* mo = mh + nn;
-            int32_t* a0 = vals.Alternate();
-            k_marks<<<blocks(A, 256), 256, 0, stream>>>(keys.Current(), A, mh, mo);
-            tb = w.tmp_bytes;
-            e = cub::DeviceScan::InclusiveScan(w.tmp, tb, mh, w.hp, MaxOp{}, (int)A, stream);
-            tb = w.tmp_bytes;
-            if (e == cudaSuccess) e = cub::DeviceScan::InclusiveScan(w.tmp, tb, mo, a0, MaxOp{}, (int)A, stream);
-            if (e != cudaSuccess) return e;
-            k_update<<<blocks(A, 256), 256, 0, stream>>>(keys.Current(), vals.Current(), w.hp, a0, A, level, w.sep, r);
-            tb = w.tmp_bytes;
-            e = cub::DeviceSelect::If(w.tmp, tb, thrust::counting_iterator<int32_t>(0), w.head, w.misc + 2,
-                                      (int)total, ActiveAt{level}, stream);
-            if (e != cudaSuccess) return e;
+            if (e != cudaSuccess) { bigger.release(); return e; }
+            w.release();
+            w = bigger;
+            bigger.base = nullptr;                        // owned by w now
+            keys = cub::DoubleBuffer<uint64_t>(w.k0, w.k1);
+            vals = cub::DoubleBuffer<int32_t>(w.v0, w.v1);
+            act = w.head;
+            spare = w.hp;
         }
-        // the suffix array: positions sorted by their final (distinct) ranks
-        int32_t* kk = reinterpret_cast<int32_t*>(w.k0);
-        e = cudaMemcpyAsync(kk, w.levels + (size_t)(rounds - 1) * nn, nn * 4, cudaMemcpyDeviceToDevice, stream);
+        const int32_t* prev = w.levels + (size_t)(r - 1) * nn;
+        int32_t* level = w.levels + (size_t)r * nn;
+        e = cudaMemcpyAsync(level, prev, nn * 4, cudaMemcpyDeviceToDevice, stream);   // settled ranks stay
         if (e != cudaSuccess) return e;
-        k_iota<<<blocks(total, 256), 256, 0, stream>>>(w.v0, total);
-        cub::DoubleBuffer<int32_t> fk(kk, kk + nn);
-        cub::DoubleBuffer<int32_t> fv(w.v0, w.v1);
+        const long long h = (long long)csyms << (r - 1);
+        k_keys_act<<<blocks(A, 256), 256, 0, stream>>>(act, A, prev, h, one ? nullptr : w.end, total, bits,
+                                                       keys.Current(), vals.Current());
         tb = w.tmp_bytes;
-        e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, fk, fv, (int)total, 0, bits, stream);
+        e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, keys, vals, (int)A, 0, 2 * bits, stream);
         if (e != cudaSuccess) return e;
-        sorted = fv.Current();
+        k_update<<<blocks(A, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), A, bits, level, sa, w.sep,
+                                                                  r);
+        tb = w.tmp_bytes;
+        e = cub::DeviceSelect::If(w.tmp, tb, (const int32_t*)act, spare, w.misc + 2, (int)A, ActiveAt{level}, stream);
+        if (e != cudaSuccess) return e;
+        int32_t* t = act;
+        act = spare;
+        spare = t;
     }
-    k_lcp<<<blocks(total, 256), 256, 0, stream>>>(text, total, off, num, sorted, w.levels, rounds, csyms, w.sep,
-                                                  w.levels + (size_t)(rounds - 1) * nn, sa, rank, lcp);
+    k_lcp<<<blocks(total, 256), 256, 0, stream>>>(text, total, off, num, sa, w.levels, rounds, csyms, w.sep,
+                                                  w.levels + (size_t)(rounds - 1) * nn, rank, lcp);
+    if (!one) k_local_sa<<<blocks(total, 256), 256, 0, stream>>>(sa, total, off, num);
     if (rounds_out) *rounds_out = rounds;
     return cudaGetLastError();
 }
