@@ -124,6 +124,7 @@ void carve(unsigned char* b, long long cap_n, long long n, unsigned* d_err, lr::
     s->cstart = (int32_t*)(b + L.off_cstart);
     s->cend = (int32_t*)(b + L.off_cend);
     s->ent1 = (uint32_t*)(b + L.off_ent1);
+    s->dense = (uint16_t*)(b + L.off_ent1);
     s->ent2 = (uint32_t*)(b + L.off_ent2);
     s->lbig = (int32_t*)(b + L.off_lbig);
     s->halo = (int32_t*)(b + L.off_halo);
@@ -156,6 +157,7 @@ lr_status get_scratch(lr_ctx* ctx, long long n, lr::Scratch* s) {
     carve(ctx->scratch, ctx->scratch_n, n, ctx->d_err, s);
     s->spin_limit = ctx->spin_limit;
     s->hold_tile = ctx->hold_tile;
+    s->one_tile = ctx->hold_tile < 0;              // the test hook needs the look-back
     ctx->last_n = n;
     return LR_OK;
 }

@@ -269,6 +269,187 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
     }
 }
 
+// From the staged entries to the outputs of the tile (whole CTA, after the
+// barrier that completes the staging; sm.bmap, rec[0], nx, ttot and far are
+// initialised).  Staged entries nlow + 1 .. MS of sm.ent reach the tile.
+// kOne: the tile is the whole string, so there is nothing to look back to.
+template <bool kAll, int TP, bool kOne>
+__device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, const Scratch& s, long long tile, int32_t k0,
+                                              int32_t MS, int32_t nlow, int32_t* __restrict__ lr_len,
+                                              int32_t* __restrict__ lr_start, int64_t* __restrict__ offsets,
+                                              int32_t* __restrict__ starts, long long capacity) {
+    constexpr int kCoverTile = Cfg<TP>::kTileC;
+    constexpr int kCoverThreads = Cfg<TP>::kThr;
+    constexpr int kWarps = Cfg<TP>::kWarps;
+    constexpr int kChunksPerWarp = Cfg<TP>::kChunksPerWarp;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // Per entry: the positions of the tile [hs, he) where it is a holder, the
+    // holders where they begin and those left where it ends.
+    uint8_t* const nx = reinterpret_cast<uint8_t*>(sm.nx);
+    const int32_t k1 = k0 > 0x7fffffff - kCoverTile ? 0x7fffffff : k0 + kCoverTile;   // the tile's end (no entry ends past n)
+    int32_t held = 0;                                         // positions x holders of this thread's entries
+    for (int v0 = nlow + 1 + warp * kWarp; v0 <= MS; v0 += kCoverThreads) {
+        const int v = v0 + lane;
+        const bool in = v <= MS;                              // other lanes take the outer entries and stop at once
+        const int2 me = sm.ent[in ? v : 0];
+        const int32_t L = me.y, e1 = me.x + L;                // one past its end
+        const int32_t a = me.x > k0 ? me.x : k0;
+        const int32_t b1 = e1 < k1 ? e1 : k1;
+        // to the left, over the entries that still cover a: those of length L
+        // before a longer one are holders wherever v begins to be one
+        int32_t left = v, eq = 1, qe;
+        bool go;
+        int u = in ? v : 1;
+        do {
+            const int2 q = sm.ent[--u];
+            qe = q.x + q.y;
+            go = (qe > a) & (q.y <= L);
+            if (go & (q.y == L)) { ++eq; left = u; }
+        } while (go);
+        const int32_t hs = qe > a ? qe : a;
+        // to the right, over the entries that start by e1, up to a longer one
+        // (unless v is never the longest in this tile)
+        int32_t first = MS + 1, feq = 0, qs;
+        u = hs < b1 ? v : MS;
+        do {
+            const int2 q = sm.ent[++u];
+            qs = q.x;
+            go = (qs <= e1) & (q.y <= L);
+            if (go & (q.y == L)) { first = min(first, u); ++feq; }
+        } while (go);
+        const int32_t he = qs < b1 ? qs : b1;
+        if (hs < he) {
+            held += he - hs;
+            if constexpr (kAll) {
+                if (feq > 0) {
+                    nx[v] = (uint8_t)(first - v < 255 ? first - v : 255);
+                    if (first - v >= 255) sm.far = 1;
+                }
+            }
+            if (sm.ent[first].x > hs) {                       // else the next of length L begins at hs too
+                const int32_t x = hs - k0;
+                sm.rec[x] = (uint32_t)left | ((uint32_t)eq << 16);
+                atomicOr(&sm.bmap[x >> 5], 1u << (x & 31));
+            }
+            // where v ends with no longer entry begun: the remaining holders
+            // of length L, if any; nothing, if no entry starts by then; else
+            // the best shorter entry begins there
+            if (qs > e1 && e1 < k1 && (feq > 0 || u == v + 1)) {
+                const int32_t x = e1 - k0;
+                sm.rec[x] = feq > 0 ? ((uint32_t)first | ((uint32_t)feq << 16)) : 0u;
+                atomicOr(&sm.bmap[x >> 5], 1u << (x & 31));
+            }
+        }
+        __syncwarp();
+    }
+    if constexpr (kAll) {
+        held = (int32_t)__reduce_add_sync(kFull, (unsigned)held);
+        if (lane == 0 && held) atomicAdd(&sm.ttot, held);
+    }
+    __syncthreads();
+    if constexpr (kAll) {
+        if (!kOne && tid == 0 && tile != s.hold_tile) publish(s.status_o, tile, tile == 0 ? kPrefix : kAggregate, sm.ttot);
+    }
+
+    // Per position: its record is the one of the last boundary at or before it.
+    const unsigned below = (1u << lane) - 1u;
+    const unsigned upto = below | (1u << lane);
+    const int c0 = warp * kChunksPerWarp;
+    int pb = 0;                                               // last boundary before the warp's current run
+    for (int w0 = c0; w0 > 0; w0 -= kWarp) {
+        const int w = w0 - 1 - lane;
+        const unsigned word = w >= 0 ? sm.bmap[w] : 0u;
+        const unsigned m = __ballot_sync(kFull, word != 0u);
+        if (m) {
+            const int l = __ffs(m) - 1;
+            pb = (w0 - 1 - l) * kWarp + 31 - __clz(__shfl_sync(kFull, word, l));
+            break;
+        }
+    }
+    uint32_t pk[kChunksPerWarp];                              // the positions' records
+    int32_t sum = 0;
+#pragma unroll
+    for (int q = 0; q < kChunksPerWarp; ++q) {
+        const int x0 = (c0 + q) * kWarp;
+        const unsigned word = sm.bmap[c0 + q];
+        const unsigned m = word & upto;
+        const uint32_t r = sm.rec[m ? x0 + 31 - __clz(m) : pb];
+        if (word) pb = x0 + 31 - __clz(word);
+        const int2 h = sm.ent[r & 0xffffu];
+        const int32_t k = k0 + x0 + lane;
+        pk[q] = r;
+        if (k < n) {
+            __stcs(lr_len + k, h.y);
+            __stcs(lr_start + k, h.x);
+            sum += (int32_t)(r >> 16);
+        } else {
+            pk[q] = 0;
+        }
+    }
+    if constexpr (kAll) {
+        sum = (int32_t)__reduce_add_sync(kFull, (unsigned)sum);
+        if (lane == 0) sm.wtot[warp] = sum;
+        if (kOne) {
+            if (tid == 0) { sm.obase = 0; offsets[n] = sm.ttot; }
+        } else if (warp == kWarps - 1) {
+            const long long ex = place_tile(s, tile, num_cover_tiles(n, TP), n, sm.ttot, offsets);
+            if (lane == 0) sm.obase = ex;
+        }
+        __syncthreads();
+        long long o0 = sm.obase;
+        {
+            const int32_t t = lane < warp ? sm.wtot[lane < kWarps ? lane : 0] : 0;
+            o0 += (int32_t)__reduce_add_sync(kFull, (unsigned)t);
+        }
+        // starts[o0 ..]: 32-bit indices from here; entries past the capacity are not written
+        const long long room = capacity - o0;
+        const int32_t lim = room < 0 ? 0 : (room > 0x7fffffff ? 0x7fffffff : (int32_t)room);
+        int32_t* out = starts + o0;
+        const bool far = sm.far != 0;
+        int32_t run = 0;
+#pragma unroll
+        for (int q = 0; q < kChunksPerWarp; ++q) {
+            const int32_t k = k0 + (c0 + q) * kWarp + lane;
+            const int32_t cq = (int32_t)(pk[q] >> 16);
+            const unsigned two = __ballot_sync(kFull, cq > 1);
+            const unsigned one = __ballot_sync(kFull, cq & 1);
+            int tot = __popc(one);
+            int32_t o = run + __popc(one & below);
+            if (two) {
+                if (__ballot_sync(kFull, cq > 3) == 0u) {
+                    tot += 2 * __popc(two);
+                    o += 2 * __popc(two & below);
+                } else {
+                    const int incl = warp_incl_scan(cq);
+                    tot = __shfl_sync(kFull, incl, kWarp - 1);
+                    o = run + incl - cq;
+                }
+            }
+            run += tot;
+            if (k < n) __stcs(reinterpret_cast<long long*>(offsets) + k, o0 + o);
+            // every compact LLR of the longest length over k, ascending
+            int32_t left = cq < lim - o ? cq : lim - o;
+            int v = (int)(pk[q] & 0xffffu);
+            int32_t* p = out + o;
+            if (left > 0) __stcs(p, sm.ent[v].x);
+            if (two) {
+                while (--left > 0) {
+                    const int32_t d = nx[v];
+                    if (far && d == 255) {
+                        const int32_t L = sm.ent[v].y;
+                        v += d;
+                        while (v <= MS && sm.ent[v].y != L) ++v;
+                    } else {
+                        v += d;
+                    }
+                    __stcs(++p, sm.ent[v].x);
+                }
+                __syncwarp();
+            }
+        }
+    }
+}
+
 }  // namespace
 
 template <bool kAll, int TP>
@@ -278,9 +459,7 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
     constexpr int kCoverTile = Cfg<TP>::kTileC;
     constexpr int kCoverThreads = Cfg<TP>::kThr;
     constexpr int kCoverTilesPer = TP;
-    constexpr int kWarps = Cfg<TP>::kWarps;
     constexpr int kChunks = Cfg<TP>::kChunks;
-    constexpr int kChunksPerWarp = Cfg<TP>::kChunksPerWarp;
     extern __shared__ __align__(16) unsigned char cover_smem[];
     CoverSmem<TP>& sm = *reinterpret_cast<CoverSmem<TP>*>(cover_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -350,170 +529,104 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
         cover_long_carry<kAll, TP>(sm, n, s, tile, cb0, cb1, lr_len, lr_start, offsets, starts, capacity);
         return;
     }
+    cover_entries<kAll, TP, false>(sm, n, s, tile, k0, MS, nlow, lr_len, lr_start, offsets, starts, capacity);
+}
 
-    // Per entry: the positions of the tile [hs, he) where it is a holder, the
-    // holders where they begin and those left where it ends.
-    uint8_t* const nx = reinterpret_cast<uint8_t*>(sm.nx);
-    const int32_t k1 = k0 > 0x7fffffff - kCoverTile ? 0x7fffffff : k0 + kCoverTile;   // the tile's end (no entry ends past n)
-    int32_t held = 0;                                         // positions x holders of this thread's entries
-    for (int v0 = nlow + 1 + warp * kWarp; v0 <= MS; v0 += kCoverThreads) {
-        const int v = v0 + lane;
-        const bool in = v <= MS;                              // other lanes take the outer entries and stop at once
-        const int2 me = sm.ent[in ? v : 0];
-        const int32_t L = me.y, e1 = me.x + L;                // one past its end
-        const int32_t a = me.x > k0 ? me.x : k0;
-        const int32_t b1 = e1 < k1 ? e1 : k1;
-        // to the left, over the entries that still cover a: those of length L
-        // before a longer one are holders wherever v begins to be one
-        int32_t left = v, eq = 1, qe;
-        bool go;
-        int u = in ? v : 1;
-        do {
-            const int2 q = sm.ent[--u];
-            qe = q.x + q.y;
-            go = (qe > a) & (q.y <= L);
-            if (go & (q.y == L)) { ++eq; left = u; }
-        } while (go);
-        const int32_t hs = qe > a ? qe : a;
-        // to the right, over the entries that start by e1, up to a longer one
-        // (unless v is never the longest in this tile)
-        int32_t first = MS + 1, feq = 0, qs;
-        u = hs < b1 ? v : MS;
-        do {
-            const int2 q = sm.ent[++u];
-            qs = q.x;
-            go = (qs <= e1) & (q.y <= L);
-            if (go & (q.y == L)) { first = min(first, u); ++feq; }
-        } while (go);
-        const int32_t he = qs < b1 ? qs : b1;
-        if (hs < he) {
-            held += he - hs;
-            if constexpr (kAll) {
-                if (feq > 0) {
-                    nx[v] = (uint8_t)(first - v < 255 ? first - v : 255);
-                    if (first - v >= 255) sm.far = 1;
-                }
-            }
-            if (sm.ent[first].x > hs) {                       // else the next of length L begins at hs too
-                const int32_t x = hs - k0;
-                sm.rec[x] = (uint32_t)left | ((uint32_t)eq << 16);
-                atomicOr(&sm.bmap[x >> 5], 1u << (x & 31));
-            }
-            // where v ends with no longer entry begun: the remaining holders
-            // of length L, if any; nothing, if no entry starts by then; else
-            // the best shorter entry begins there
-            if (qs > e1 && e1 < k1 && (feq > 0 || u == v + 1)) {
-                const int32_t x = e1 - k0;
-                sm.rec[x] = feq > 0 ? ((uint32_t)first | ((uint32_t)feq << 16)) : 0u;
-                atomicOr(&sm.bmap[x >> 5], 1u << (x & 31));
-            }
-        }
-        __syncwarp();
+// A string of at most one tile of 8192 positions: the whole query in one CTA
+// and one launch (Lemma 1 from sa or rank into shared memory by position,
+// flags, compaction, cover), with nothing to clear before it.  What bounds a
+// query of this size is launches and the chains between them: 4099
+// positions of DNA took 74 us with five launches, and 42 us with this one.
+constexpr int kOneTP = 4;
+static_assert(Cfg<kOneTP>::kTileC == kOneTileMax, "one-tile strings");
+
+template <bool kAll, bool kSa>
+__global__ void __launch_bounds__(Cfg<kOneTP>::kThr, 1)
+k_one_tile(const int32_t* __restrict__ in, const int32_t* __restrict__ lcp, int32_t n, Scratch s,
+           int32_t* __restrict__ lr_len, int32_t* __restrict__ lr_start, int64_t* __restrict__ offsets,
+           int32_t* __restrict__ starts, long long capacity) {
+    constexpr int TP = kOneTP, kThr = Cfg<TP>::kThr, kChunks = Cfg<TP>::kChunks, kPer = Cfg<TP>::kTileC / kThr;
+    extern __shared__ __align__(16) unsigned char cover_smem[];
+    CoverSmem<TP>& sm = *reinterpret_cast<CoverSmem<TP>*>(cover_smem);
+    int32_t* const D = reinterpret_cast<int32_t*>(cover_smem + sizeof(CoverSmem<TP>));   // L by position, -1 where none came
+    __shared__ int32_t wsum[kThr / kWarp];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        sm.ttot = 0;
+        sm.far = 0;
+        sm.rec[0] = 0;
+        *s.qerr = 0;
     }
+    if (tid < kChunks) sm.bmap[tid] = tid == 0 ? 1u : 0u;
     if constexpr (kAll) {
-        held = (int32_t)__reduce_add_sync(kFull, (unsigned)held);
-        if (lane == 0 && held) atomicAdd(&sm.ttot, held);
+        for (int i = tid; i < CoverSmem<TP>::kNxWords; i += kThr) sm.nx[i] = 0;
+    }
+    // all loads in flight before the first is used
+    int32_t v[kPer], a[kPer], b[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int r = j * kThr + tid;
+        v[j] = r < n ? __ldg(in + r) : 0;
+        if (kSa) { a[j] = r < n ? __ldg(lcp + r) : 0; b[j] = r < n ? __ldg(lcp + r + 1) : 0; }
+        D[r] = -1;
+    }
+    bool bad = false;
+    if (tid == 0 && (__ldg(lcp) != 0 || __ldg(lcp + n) != 0)) bad = true;
+    if (!kSa) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int k = j * kThr + tid;
+            if (k < n && (uint32_t)v[j] >= (uint32_t)n) { bad = true; v[j] = 0; }
+            a[j] = k < n ? __ldg(lcp + v[j]) : 0;
+            b[j] = k < n ? __ldg(lcp + v[j] + 1) : 0;
+        }
     }
     __syncthreads();
-    if constexpr (kAll) {
-        if (tid == 0 && tile != s.hold_tile) publish(s.status_o, tile, tile == 0 ? kPrefix : kAggregate, sm.ttot);
-    }
-
-    // Per position: its record is the one of the last boundary at or before it.
-    const unsigned below = (1u << lane) - 1u;
-    const unsigned upto = below | (1u << lane);
-    const int c0 = warp * kChunksPerWarp;
-    int pb = 0;                                               // last boundary before the warp's current run
-    for (int w0 = c0; w0 > 0; w0 -= kWarp) {
-        const int w = w0 - 1 - lane;
-        const unsigned word = w >= 0 ? sm.bmap[w] : 0u;
-        const unsigned m = __ballot_sync(kFull, word != 0u);
-        if (m) {
-            const int l = __ffs(m) - 1;
-            pb = (w0 - 1 - l) * kWarp + 31 - __clz(__shfl_sync(kFull, word, l));
-            break;
-        }
-    }
-    uint32_t pk[kChunksPerWarp];                              // the positions' records
-    int32_t sum = 0;
 #pragma unroll
-    for (int q = 0; q < kChunksPerWarp; ++q) {
-        const int x0 = (c0 + q) * kWarp;
-        const unsigned word = sm.bmap[c0 + q];
-        const unsigned m = word & upto;
-        const uint32_t r = sm.rec[m ? x0 + 31 - __clz(m) : pb];
-        if (word) pb = x0 + 31 - __clz(word);
-        const int2 h = sm.ent[r & 0xffffu];
-        const int32_t k = k0 + x0 + lane;
-        pk[q] = r;
-        if (k < n) {
-            __stcs(lr_len + k, h.y);
-            __stcs(lr_start + k, h.x);
-            sum += (int32_t)(r >> 16);
-        } else {
-            pk[q] = 0;
-        }
+    for (int j = 0; j < kPer; ++j) {
+        const int r = j * kThr + tid;
+        if (r >= n) continue;
+        const uint32_t p = kSa ? (uint32_t)v[j] : (uint32_t)r;
+        if (p >= (uint32_t)n) { bad = true; continue; }
+        int32_t L = a[j] > b[j] ? a[j] : b[j];
+        if ((uint32_t)L > (uint32_t)n - p) { bad = true; L = 0; }   // negative ones too
+        D[p] = L;
     }
-    if constexpr (kAll) {
-        sum = (int32_t)__reduce_add_sync(kFull, (unsigned)sum);
-        if (lane == 0) sm.wtot[warp] = sum;
-        if (warp == kWarps - 1) {
-            const long long ex = place_tile(s, tile, num_cover_tiles(n, TP), n, sm.ttot, offsets);
-            if (lane == 0) sm.obase = ex;
-        }
-        __syncthreads();
-        long long o0 = sm.obase;
-        {
-            const int32_t t = lane < warp ? sm.wtot[lane < kWarps ? lane : 0] : 0;
-            o0 += (int32_t)__reduce_add_sync(kFull, (unsigned)t);
-        }
-        // starts[o0 ..]: 32-bit indices from here; entries past the capacity are not written
-        const long long room = capacity - o0;
-        const int32_t lim = room < 0 ? 0 : (room > 0x7fffffff ? 0x7fffffff : (int32_t)room);
-        int32_t* out = starts + o0;
-        const bool far = sm.far != 0;
-        int32_t run = 0;
+    __syncthreads();
+    // flags and compaction: eight consecutive positions per thread
+    static_assert(kPer == 8, "positions per thread");
+    const int x = tid * kPer;
+    int32_t l[kPer], prev = x > 0 ? max(D[x - 1], 0) : 0;
+    unsigned f = 0;
 #pragma unroll
-        for (int q = 0; q < kChunksPerWarp; ++q) {
-            const int32_t k = k0 + (c0 + q) * kWarp + lane;
-            const int32_t cq = (int32_t)(pk[q] >> 16);
-            const unsigned two = __ballot_sync(kFull, cq > 1);
-            const unsigned one = __ballot_sync(kFull, cq & 1);
-            int tot = __popc(one);
-            int32_t o = run + __popc(one & below);
-            if (two) {
-                if (__ballot_sync(kFull, cq > 3) == 0u) {
-                    tot += 2 * __popc(two);
-                    o += 2 * __popc(two & below);
-                } else {
-                    const int incl = warp_incl_scan(cq);
-                    tot = __shfl_sync(kFull, incl, kWarp - 1);
-                    o = run + incl - cq;
-                }
-            }
-            run += tot;
-            if (k < n) __stcs(reinterpret_cast<long long*>(offsets) + k, o0 + o);
-            // every compact LLR of the longest length over k, ascending
-            int32_t left = cq < lim - o ? cq : lim - o;
-            int v = (int)(pk[q] & 0xffffu);
-            int32_t* p = out + o;
-            if (left > 0) __stcs(p, sm.ent[v].x);
-            if (two) {
-                while (--left > 0) {
-                    const int32_t d = nx[v];
-                    if (far && d == 255) {
-                        const int32_t L = sm.ent[v].y;
-                        v += d;
-                        while (v <= MS && sm.ent[v].y != L) ++v;
-                    } else {
-                        v += d;
-                    }
-                    __stcs(++p, sm.ent[v].x);
-                }
-                __syncwarp();
-            }
-        }
+    for (int j = 0; j < kPer; ++j) {
+        l[j] = D[x + j];
+        if (x + j < n && l[j] < 0) bad = true;                // sa gave another position twice
+        l[j] = max(l[j], 0);
+        if (l[j] > 0 && l[j] >= prev) f |= 1u << j;           // 0 past the end
+        prev = l[j];
     }
+    if (bad) {
+        atomicOr(s.err, kErrInput);
+        atomicOr(s.qerr, kErrInput);
+    }
+    const int c = __popc(f), incl = warp_incl_scan(c);
+    if (lane == kWarp - 1) wsum[warp] = incl;
+    __syncthreads();
+    const int w = wsum[lane];                                 // kThr / kWarp = 32 totals
+    static_assert(kThr / kWarp == kWarp, "one total per lane");
+    int o = incl - c + (int)__reduce_add_sync(kFull, lane < warp ? (unsigned)w : 0u);
+    const int32_t m = (int32_t)__reduce_add_sync(kFull, (unsigned)w);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+        if ((f >> j) & 1u) sm.ent[++o] = make_int2(x + j, l[j]);
+    if (tid == 0) {
+        sm.ent[0] = make_int2(-1, 0);
+        sm.ent[m + 1] = make_int2(0x7fffffff, 0);
+        s.tile_cbase[s.ntiles] = m;
+    }
+    __syncthreads();
+    cover_entries<kAll, TP, true>(sm, n, s, 0, 0, m, 0, lr_len, lr_start, offsets, starts, capacity);
 }
 
 namespace {
@@ -538,8 +651,41 @@ cudaError_t set_cover_smem() {
 
 }  // namespace
 
+namespace {
+constexpr size_t kOneSmem = sizeof(CoverSmem<kOneTP>) + (size_t)Cfg<kOneTP>::kTileC * 4;
+
+template <bool kAll, bool kSa>
+cudaError_t set_one_smem() {
+    return cudaFuncSetAttribute(k_one_tile<kAll, kSa>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneSmem);
+}
+
+template <bool kAll, bool kSa>
+void launch_one_t(const int32_t* in, const int32_t* lcp, int32_t n, const Scratch& s, int32_t* lr_len, int32_t* lr_start,
+                  int64_t* offsets, int32_t* starts, long long capacity, cudaStream_t stream) {
+    k_one_tile<kAll, kSa><<<1, Cfg<kOneTP>::kThr, kOneSmem, stream>>>(in, lcp, n, s, lr_len, lr_start, offsets, starts,
+                                                                      capacity);
+}
+}  // namespace
+
+void launch_one_tile(const int32_t* sa, const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s,
+                     int32_t* lr_len, int32_t* lr_start, int64_t* offsets, int32_t* starts, long long capacity, bool all,
+                     cudaStream_t stream) {
+    if (!all) { offsets = nullptr; starts = nullptr; capacity = 0; }
+    if (sa) {
+        if (all) launch_one_t<true, true>(sa, lcp, n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+        else launch_one_t<false, true>(sa, lcp, n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+    } else {
+        if (all) launch_one_t<true, false>(rank, lcp, n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+        else launch_one_t<false, false>(rank, lcp, n, s, lr_len, lr_start, offsets, starts, capacity, stream);
+    }
+}
+
 cudaError_t configure_cover() {
-    cudaError_t e = set_cover_smem<1>();
+    cudaError_t e = set_one_smem<true, true>();
+    if (e == cudaSuccess) e = set_one_smem<true, false>();
+    if (e == cudaSuccess) e = set_one_smem<false, true>();
+    if (e == cudaSuccess) e = set_one_smem<false, false>();
+    if (e == cudaSuccess) e = set_cover_smem<1>();
     if (e == cudaSuccess) e = set_cover_smem<2>();
     if (e == cudaSuccess) e = set_cover_smem<4>();
     return e;

@@ -7,7 +7,7 @@
 // index of its first LLRc entry (tile_cbase, seg_cbase), which the cover
 // kernels start from.
 //
-// Two front ends compute the same LLRc:
+// Three front ends compute the same LLRc:
 //
 //  * rank-order (the default when the suffix array is given).  Lemma 1 read
 //    in rank order is L_{sa[r]} = max(lcp[r], lcp[r+1]): sa and lcp are then
@@ -19,11 +19,15 @@
 //    CTA, scatters its lengths into shared memory by position, and flags
 //    and compacts them.
 //
+//  * dense (the suffix array given, up to a few million positions): the
+//    lengths are stored straight at their positions (k_scatter) and compacted
+//    tile by tile (k_compact).
+//
 //  * rank gather (when only rank is given, as in the paper's data flow of
 //    Sec. 4): k_gather_llr reads rank coalesced and gathers the two lcp
 //    words of each position, then flags and compacts one tile.
 //
-// Both place their entries in LLRc with a decoupled look-back over the
+// All place their entries in LLRc with a decoupled look-back over the
 // per-CTA counts (tiles handed out in order by an atomic ticket).
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -965,35 +969,178 @@ k_part2(int32_t n, Scratch s, int rounds) {
     if (bad) report(s, kErrInput);
 }
 
+// K1 (Sec. 4.2.1) on 2-byte length words: each warp owns kPerWarp chunks of
+// 256 consecutive positions from position x0 on, eight consecutive positions
+// per lane.  One 16-byte load gives a lane its words, the flags are sign bits
+// shifted together (first position in the top bit).  W gives plain words:
+// load8(x) for positions x .. x + 7 and at(x); below W::kEsc a word is the
+// length, W::kEsc itself stands for a longer one (in lbig), anything above
+// for a position that got no length (reported: sa gave another one twice).
+// `halo`: the length of the position before 0 (used where x0 is 0).
+constexpr int kBktChunk = 256;                                   // = kSeg: seg_cbase falls out of the chunk counts
+static_assert(kBktChunk == kSeg, "chunk and segment sizes");
+
+// L of position x of a tile, 0 <= x < cnt; a position without a length counts as 0
+template <class W>
+__device__ __forceinline__ int32_t llr_len(const W& words, int x, const int32_t* lbig) {
+    const uint32_t f = words.at(x);
+    return f < W::kEsc ? (int32_t)f : (f == W::kEsc ? __ldcg(lbig + x) : 0);
+}
+
+template <int kPerWarp, class W>
+__device__ __forceinline__ void llr_flags(const W& words, int x0, int cnt, int32_t halo, const int32_t* lbig,
+                                          uint32_t (&flags)[(kPerWarp + 3) / 4], int32_t* counts, unsigned& bad) {
+    const int lane = lane_id();
+    uint32_t last = 0;                                       // word of the position before the chunk
+    if (x0 == 0) last = min((uint32_t)halo, W::kEsc);
+    else if (x0 - 1 < cnt) last = min(words.at(x0 - 1), W::kEsc);
+#pragma unroll
+    for (int q = 0; q < kPerWarp; ++q) {
+        const int x = x0 + q * kBktChunk + lane * 8;
+        const uint4 w = words.load8(x);
+        const uint32_t m = __vmaxu2(__vmaxu2(w.x, w.y), __vmaxu2(w.z, w.w));
+        const bool odd = (m & 0xffffu) >= W::kEsc || (m >> 16) >= W::kEsc;
+        uint32_t prev = __shfl_up_sync(kFull, w.w >> 16, 1);
+        if (lane == 0) prev = last;
+        last = min(__shfl_sync(kFull, w.w >> 16, kWarp - 1), W::kEsc);
+        uint32_t f = 0;
+        if (__any_sync(kFull, odd || x + 8 > cnt)) {
+            // a length from lbig, a position without one or past the end
+            int32_t before = x > 0 ? (x - 1 < cnt ? llr_len(words, x - 1, lbig) : 0) : halo;
+            for (int j = 0; j < 8; ++j) {
+                const bool in = x + j < cnt;
+                if (in && words.at(x + j) > W::kEsc) bad = 1;
+                const int32_t l = in ? llr_len(words, x + j, lbig) : 0;
+                f = 2 * f + (l > 0 && l >= before);
+                before = l;
+            }
+        } else {
+            const uint32_t l[8] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16,
+                                   w.z & 0xffffu, w.z >> 16, w.w & 0xffffu, w.w >> 16};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {                     // sign of l - max(prev, 1): 1 = dropped
+                f = __funnelshift_l(l[j] - max(prev, 1u), f, 1);
+                prev = l[j];
+            }
+            f ^= 0xffu;
+        }
+        flags[q / 4] |= (f & 0xffu) << (8 * (q % 4));
+        const int c = (int)__reduce_add_sync(kFull, (unsigned)__popc(f & 0xffu));
+        if (lane == 0) counts[q] = c;
+    }
+}
+
+// K3: a chunk's kept positions are listed in shared memory (mine, kBktChunk
+// entries per warp) and then written to LLRc in one run.
+template <int kPerWarp, class W>
+__device__ __forceinline__ void llr_write(const W& words, int x0, long long k0, const int32_t* lbig,
+                                          const uint32_t (&flags)[(kPerWarp + 3) / 4], const int32_t* offs, long long base,
+                                          uint16_t* mine, const Scratch& s) {
+    const int lane = lane_id();
+#pragma unroll
+    for (int q = 0; q < kPerWarp; ++q) {
+        const int x = x0 + q * kBktChunk + lane * 8;
+        const uint32_t f = (flags[q / 4] >> (8 * (q % 4))) & 0xffu;
+        const int c = __popc(f);
+        const int incl = warp_incl_scan(c);
+        int o = incl - c;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (f & (0x80u >> j)) mine[o++] = (uint16_t)(x + j);
+        const int tot = __shfl_sync(kFull, incl, kWarp - 1);
+        __syncwarp();
+        const long long to = base + offs[q];
+        for (int i = lane; i < tot; i += kWarp) {
+            const int y = mine[i];
+            const int32_t k = (int32_t)(k0 + y);
+            s.cstart[to + i] = k;
+            s.cend[to + i] = k + llr_len(words, y, lbig) - 1;
+        }
+        __syncwarp();
+    }
+}
+
+// Exclusive scan of a tile's kChunks chunk counts and the tile's place in
+// LLRc (K2, look-back), by one warp; *total the tile's count.
+template <int kChunks>
+__device__ __forceinline__ long long llr_place(int32_t* counts, unsigned long long* status, long long tile,
+                                               const Scratch& s, int32_t* total) {
+    const int lane = lane_id();
+    constexpr int kPer = (kChunks + kWarp - 1) / kWarp;
+    int a[kPer], sum = 0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int i = lane * kPer + u;
+        a[u] = i < kChunks ? counts[i] : 0;
+        sum += a[u];
+    }
+    const int incl = warp_incl_scan(sum);
+    int ex = incl - sum;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int i = lane * kPer + u;
+        if (i < kChunks) counts[i] = ex;
+        ex += a[u];
+    }
+    *total = __shfl_sync(kFull, incl, kWarp - 1);
+    return lookback_exclusive(status, tile, *total, s.err, s.qerr, s.spin_limit);
+}
+
+// First LLRc entry of each tile of kTile positions and of each segment of
+// kSeg positions of a tile of kChunks chunks (whole CTA).
+template <int kChunks>
+__device__ __forceinline__ void llr_bases(long long tile, const int32_t* offs, long long base, int32_t total,
+                                          const Scratch& s) {
+    const int i = threadIdx.x;
+    if (i >= kChunks) return;
+    const long long sg = tile * kChunks + i;
+    const int32_t at = (int32_t)(base + offs[i]);
+    if (sg < s.nsegs) s.seg_cbase[sg] = at;
+    if (sg == s.nsegs - 1) s.seg_cbase[s.nsegs] = (int32_t)(base + total);
+    constexpr int kPerTile = kTile / kBktChunk;
+    if (i % kPerTile == 0) {
+        const long long t = sg / kPerTile;
+        if (t < s.ntiles) s.tile_cbase[t] = at;
+        if (t == s.ntiles - 1) s.tile_cbase[s.ntiles] = (int32_t)(base + total);
+    }
+}
+
 // One bucket of kBucket positions per CTA: lengths scattered into shared
-// memory by position, usefulness flags (K1), compaction (K2) and the
-// bucket's place in LLRc by look-back (K3).
+// memory by position, then flags (K1), compaction (K2) and the bucket's place
+// in LLRc by look-back (K3).
 //
 // A position's word is the low half of its entry: the 12-bit length field
 // under the low four bits of the position.  XOR with those four bits (a
 // constant pattern per eight positions) leaves the plain field, and anything
 // else above bit 11 means that the position was never written (the words
-// start with the four bits inverted): sa gave another one twice.
+// start with the four bits inverted).
 //
-// Each warp owns 2048 positions as eight chunks of 256, eight consecutive
-// positions per lane: one 16-byte load gives a lane its lengths, the flags
-// are sign bits shifted together, and the kept positions of a chunk are
-// listed in shared memory so that LLRc is written in whole runs.  2^26
-// positions of English take 114 us (67 M warp instructions); with a ballot
-// per run of 32 positions and one store per flagged lane it was 190 us
+// 2^26 positions of English take 114 us (67 M warp instructions); with a
+// ballot per run of 32 positions and one store per flagged lane it was 190 us
 // (156 M).
-constexpr int kBktChunk = 256;                                   // = kSeg: seg_cbase falls out of the chunk counts
 __device__ __forceinline__ uint32_t bucket_pattern(int x, int pair) {   // position bits of words x + 2 pair, x + 2 pair + 1
     const uint32_t lo = (uint32_t)((x & 8) + 2 * pair);
     return (lo << 12) | ((lo + 1) << 28);
 }
+struct BucketWords {
+    static constexpr uint32_t kEsc = kEsc12;
+    const uint16_t* sL;
+    __device__ __forceinline__ uint32_t at(int x) const { return (uint32_t)sL[x] ^ ((uint32_t)(x & 15) << 12); }
+    __device__ __forceinline__ uint4 load8(int x) const {
+        uint4 w = *reinterpret_cast<const uint4*>(sL + x);
+        w.x ^= bucket_pattern(x, 0);
+        w.y ^= bucket_pattern(x, 1);
+        w.z ^= bucket_pattern(x, 2);
+        w.w ^= bucket_pattern(x, 3);
+        return w;
+    }
+};
+
 __global__ void __launch_bounds__(kBucketThreads, 3)
 k_bucket_llr(int32_t n, Scratch s) {
     constexpr int kChunks = kBucket / kBktChunk;             // 128
     constexpr int kWarps = kBucketThreads / kWarp;           // 16
     constexpr int kPerWarp = kChunks / kWarps;               // 8
-    constexpr int kTilesPerBucket = kBucket / kTile;         // 16
-    static_assert(kBktChunk == kSeg && kPerWarp * kBktChunk == kTile, "chunk, segment and tile sizes");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint16_t* sL = reinterpret_cast<uint16_t*>(smem_raw);                        // kBucket words
     uint16_t* list = reinterpret_cast<uint16_t*>(smem_raw + kBucket * 2);        // kBktChunk kept positions per warp
@@ -1044,109 +1191,153 @@ k_bucket_llr(int32_t n, Scratch s) {
         }
     }
     __syncthreads();
-    // L of position k0 + x, 0 <= x < cnt; a position never written counts as 0
-    auto len_at = [&](int x) -> int32_t {
-        const uint32_t f = (uint32_t)sL[x] ^ ((uint32_t)(x & 15) << 12);
-        return f < kEsc12 ? (int32_t)f : (f == kEsc12 ? __ldcg(s.lbig + k0 + x) : 0);
-    };
-
-    // K1: the flags of a lane's eight positions per chunk, first position in the top bit
-    uint32_t flags[kPerWarp / 4] = {};                       // eight bits per chunk
-    uint32_t last = 0;                                       // field of the position before the chunk
-    {
-        const int xw = warp * kTile;
-        if (xw > 0 && xw - 1 < cnt) last = min(((uint32_t)sL[xw - 1] ^ 0xf000u) & 0xffffu, kEsc12);
-        if (xw == 0 && k0 > 0) last = min((uint32_t)__ldcg(s.halo + b), kEsc12);
-    }
-#pragma unroll
-    for (int q = 0; q < kPerWarp; ++q) {
-        const int x = warp * kTile + q * kBktChunk + lane * 8;
-        uint4 w = *reinterpret_cast<const uint4*>(sL + x);
-        w.x ^= bucket_pattern(x, 0);
-        w.y ^= bucket_pattern(x, 1);
-        w.z ^= bucket_pattern(x, 2);
-        w.w ^= bucket_pattern(x, 3);
-        const uint32_t m = __vmaxu2(__vmaxu2(w.x, w.y), __vmaxu2(w.z, w.w));
-        const bool odd = (m & 0xffffu) >= kEsc12 || (m >> 16) >= kEsc12;
-        uint32_t prev = __shfl_up_sync(kFull, w.w >> 16, 1);
-        if (lane == 0) prev = last;
-        last = min(__shfl_sync(kFull, w.w >> 16, kWarp - 1), kEsc12);
-        uint32_t f = 0;
-        if (__any_sync(kFull, odd)) {
-            // a length from lbig, a position never written or past the end
-            int32_t before = x > 0 ? (x - 1 < cnt ? len_at(x - 1) : 0) : (k0 > 0 ? __ldcg(s.halo + b) : 0);
-            for (int j = 0; j < 8; ++j) {
-                if (x + j < cnt && ((uint32_t)sL[x + j] ^ ((uint32_t)((x + j) & 15) << 12)) > kEsc12) bad = 1;
-                const int32_t l = x + j < cnt ? len_at(x + j) : 0;
-                f = 2 * f + (l > 0 && l >= before);
-                before = l;
-            }
-        } else {
-            const uint32_t l[8] = {w.x & 0xffffu, w.x >> 16, w.y & 0xffffu, w.y >> 16,
-                                   w.z & 0xffffu, w.z >> 16, w.w & 0xffffu, w.w >> 16};
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {                     // sign of l - max(prev, 1): 1 = dropped
-                f = __funnelshift_l(l[j] - max(prev, 1u), f, 1);
-                prev = l[j];
-            }
-            f ^= 0xffu;
-        }
-        flags[q / 4] |= (f & 0xffu) << (8 * (q % 4));
-        const int c = (int)__reduce_add_sync(kFull, (unsigned)__popc(f & 0xffu));
-        if (lane == 0) ccnt[warp * kPerWarp + q] = c;
-    }
+    const BucketWords words{sL};
+    const int32_t* lbig = s.lbig + k0;
+    const int x0 = warp * kPerWarp * kBktChunk;
+    const int32_t halo = (x0 == 0 && k0 > 0) ? __ldcg(s.halo + b) : 0;
+    uint32_t flags[(kPerWarp + 3) / 4] = {};
+    llr_flags<kPerWarp>(words, x0, cnt, halo, lbig, flags, ccnt + warp * kPerWarp, bad);
     if (bad) report(s, kErrInput);
     __syncthreads();
-    // exclusive scan of the chunk counts and the bucket's place, by warp 0
     if (warp == 0) {
-        int a[kChunks / kWarp], sum = 0;
-#pragma unroll
-        for (int u = 0; u < kChunks / kWarp; ++u) { a[u] = ccnt[lane * (kChunks / kWarp) + u]; sum += a[u]; }
-        const int incl = warp_incl_scan(sum);
-        int ex = incl - sum;
-#pragma unroll
-        for (int u = 0; u < kChunks / kWarp; ++u) { ccnt[lane * (kChunks / kWarp) + u] = ex; ex += a[u]; }
-        const int total = __shfl_sync(kFull, incl, kWarp - 1);
-        const long long at = lookback_exclusive(s.status_b, b, total, s.err, s.qerr, s.spin_limit);
+        int32_t total;
+        const long long at = llr_place<kChunks>(ccnt, s.status_b, b, s, &total);
         if (lane == 0) { base_s = at; total_s = total; }
     }
     __syncthreads();
-    const long long base = base_s;
-    // first LLRc entry of each tile and of each kSeg-position segment of the bucket
-    if (tid < kChunks) {
-        const long long sg = b * kChunks + tid;
-        const int32_t at = (int32_t)(base + ccnt[tid]);
-        if (sg < s.nsegs) s.seg_cbase[sg] = at;
-        if (sg == s.nsegs - 1) s.seg_cbase[s.nsegs] = (int32_t)(base + total_s);
-        if (tid % kPerWarp == 0) {
-            const long long tile = b * kTilesPerBucket + tid / kPerWarp;
-            if (tile < s.ntiles) s.tile_cbase[tile] = at;
-            if (tile == s.ntiles - 1) s.tile_cbase[s.ntiles] = (int32_t)(base + total_s);
+    llr_bases<kChunks>(b, ccnt, base_s, total_s, s);
+    llr_write<kPerWarp>(words, x0, k0, lbig, flags, ccnt + warp * kPerWarp, base_s, list + warp * kBktChunk, s);
+}
+
+// ---------------------------------------------------------------------------
+// dense front end
+// ---------------------------------------------------------------------------
+
+// Up to kDenseMaxN positions with sa, the lengths go straight to a 2-byte
+// array in text order: k_scatter stores L_{sa[r]} at sa[r] (scattered stores
+// into an array that stays in L2, where partial writes merge), k_compact reads
+// it back tile by tile, flags and compacts it.  The array is preset to
+// kDenseNone; a position that still has it afterwards means that sa gave
+// another one twice.
+constexpr uint32_t kDenseEsc = 0xfffeu;           // longer: the length is in lbig
+constexpr uint32_t kDenseNone = 0xffffu;
+
+template <bool kBatch>
+__global__ void __launch_bounds__(kThreads) k_scatter(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp,
+                                                      int32_t n, Scratch s, Segs segs) {
+    constexpr int kPer = kTile / kThreads;
+    __shared__ long long seg_sh[kBatch ? kSegCap + 1 : 1];
+    const int tid = threadIdx.x;
+    const long long r0 = (long long)blockIdx.x * kTile;
+    // the round's string, where it lies inside one (else looked up per entry)
+    long long base = 0, nj = n, lbase = 0, hint = 0;
+    bool direct = true;
+    SegView sv{};
+    if constexpr (kBatch) {
+        const long long r1 = (r0 + kTile < n) ? r0 + kTile : n;
+        sv.stage(segs, s, r0, r1, seg_sh);
+        hint = sv.find(r0, sv.j0);
+        base = sv.at(hint);
+        const long long end = sv.at(hint + 1);
+        nj = end - base;
+        lbase = hint;
+        direct = base >= 0 && base <= r0 && r1 <= end && end <= (long long)n;
+    }
+    unsigned bad = 0;
+    if (!kBatch && blockIdx.x == 0 && tid == 0 && (__ldg(lcp) != 0 || __ldg(lcp + n) != 0)) bad = 1;
+    auto put = [&](uint32_t pl, int32_t a, int32_t b, long long at, long long len) {
+        int32_t L = a > b ? a : b;
+        if ((long long)pl >= len) { bad = 1; return; }
+        if (L < 0 || (long long)L > len - (long long)pl) { bad = 1; L = 0; }
+        const long long p = at + pl;
+        uint32_t w = (uint32_t)L;
+        if (w >= kDenseEsc) { w = kDenseEsc; s.lbig[p] = L; }
+        s.dense[p] = (uint16_t)w;
+    };
+    if (direct) {
+        uint32_t v[kPer];
+        int32_t a[kPer], b[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const long long r = r0 + j * kThreads + tid;
+            v[j] = r < n ? (uint32_t)__ldcs(sa + r) : 0u;
+            a[j] = r < n ? __ldg(lcp + lbase + r) : 0;
+            b[j] = r < n ? __ldg(lcp + lbase + r + 1) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const long long r = r0 + j * kThreads + tid;
+            if (r >= n) continue;
+            if (kBatch && ((r == base && a[j] != 0) || (r == base + nj - 1 && b[j] != 0))) bad = 1;   // lcp sentinels
+            put(v[j], a[j], b[j], base, nj);
+        }
+    } else {
+        for (int j = 0; j < kPer; ++j) {
+            const long long r = r0 + j * kThreads + tid;
+            if (r >= n) continue;
+            hint = sv.find(r, hint);
+            const long long at = sv.at(hint), len = sv.at(hint + 1) - at;
+            if (at < 0 || len < 1 || at + len > n || r < at) { bad = 1; continue; }   // bad offset table
+            const int32_t a = __ldg(lcp + r + hint), b = __ldg(lcp + r + hint + 1);
+            if ((r == at && a != 0) || (r == at + len - 1 && b != 0)) bad = 1;        // lcp sentinels
+            put((uint32_t)__ldcs(sa + r), a, b, at, len);
         }
     }
-    // K3: list a chunk's kept positions, then write them
-    uint16_t* const mine = list + warp * kBktChunk;
-#pragma unroll
-    for (int q = 0; q < kPerWarp; ++q) {
-        const int x = warp * kTile + q * kBktChunk + lane * 8;
-        const uint32_t f = (flags[q / 4] >> (8 * (q % 4))) & 0xffu;
-        const int c = __popc(f);
-        const int incl = warp_incl_scan(c);
-        int o = incl - c;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            if (f & (0x80u >> j)) mine[o++] = (uint16_t)(x + j);
-        const int tot = __shfl_sync(kFull, incl, kWarp - 1);
-        __syncwarp();
-        const long long to = base + ccnt[warp * kPerWarp + q];
-        for (int i = lane; i < tot; i += kWarp) {
-            const int y = mine[i];
-            const int32_t k = (int32_t)(k0 + y);
-            s.cstart[to + i] = k;
-            s.cend[to + i] = k + len_at(y) - 1;
-        }
-        __syncwarp();
+    if (bad) report(s, kErrInput);
+}
+
+struct DenseWords {
+    static constexpr uint32_t kEsc = kDenseEsc;
+    const uint16_t* d;                            // of the tile's first position
+    __device__ __forceinline__ uint32_t at(int x) const { return __ldg(d + x); }
+    __device__ __forceinline__ uint4 load8(int x) const { return __ldg(reinterpret_cast<const uint4*>(d + x)); }
+};
+
+constexpr int kCompactThreads = 512;
+__global__ void __launch_bounds__(kCompactThreads) k_compact(int32_t n, Scratch s) {
+    constexpr int kChunks = kCompactTile / kBktChunk;        // 32
+    constexpr int kWarps = kCompactThreads / kWarp;          // 16
+    constexpr int kPerWarp = kChunks / kWarps;               // 2
+    __shared__ uint16_t list[kWarps * kBktChunk];
+    __shared__ int32_t ccnt[kChunks];
+    __shared__ long long t_s, base_s;
+    __shared__ int32_t total_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) t_s = atomicAdd(&s.tickets[1], 1u);
+    __syncthreads();
+    const long long t = t_s, k0 = t * kCompactTile;
+    const int cnt = (int)(((long long)n - k0 < kCompactTile) ? (long long)n - k0 : kCompactTile);
+    const DenseWords words{s.dense + k0};
+    const int32_t* lbig = s.lbig + k0;
+    const int x0 = warp * kPerWarp * kBktChunk;
+    const int32_t halo = (x0 == 0 && k0 > 0) ? llr_len(words, -1, lbig) : 0;
+    unsigned bad = 0;
+    uint32_t flags[1] = {};
+    llr_flags<kPerWarp>(words, x0, cnt, halo, lbig, flags, ccnt + warp * kPerWarp, bad);
+    if (bad) report(s, kErrInput);
+    __syncthreads();
+    if (warp == 0) {
+        int32_t total;
+        const long long at = llr_place<kChunks>(ccnt, s.status_g, t, s, &total);
+        if (lane == 0) { base_s = at; total_s = total; }
     }
+    __syncthreads();
+    llr_bases<kChunks>(t, ccnt, base_s, total_s, s);
+    llr_write<kPerWarp>(words, x0, k0, lbig, flags, ccnt + warp * kPerWarp, base_s, list + warp * kBktChunk, s);
+}
+
+void launch_scatter(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
+                    cudaStream_t stream) {
+    cudaMemsetAsync(s.dense, 0xff, (size_t)n * 2, stream);   // kDenseNone everywhere
+    if (segs.num > 0)
+        k_scatter<true><<<(unsigned)s.ntiles, kThreads, 0, stream>>>(sa, lcp, n, s, segs);
+    else
+        k_scatter<false><<<(unsigned)s.ntiles, kThreads, 0, stream>>>(sa, lcp, n, s, segs);
+}
+
+void launch_compact(int32_t n, const Scratch& s, cudaStream_t stream) {
+    const unsigned grid = (unsigned)(((long long)n + kCompactTile - 1) / kCompactTile);
+    k_compact<<<grid, kCompactThreads, 0, stream>>>(n, s);
 }
 
 size_t bucket_smem_bytes() { return (size_t)kBucket * 2 + (size_t)(kBucketThreads / kWarp) * kBktChunk * 2; }

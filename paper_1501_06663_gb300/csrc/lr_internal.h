@@ -39,6 +39,22 @@ constexpr int kWinLog = 22;
 constexpr int kMaxWins = 512;                  // n < 2^31
 constexpr long long kRankWinMinN = 1LL << 24;
 
+// A string of at most this many positions takes one CTA and one launch
+// (4099 positions: 74 -> 42 us; above, one CTA would work alone for longer
+// than the launches of the other paths take: 20 000 positions need 67 us there).
+constexpr int kOneTileMax = 8192;
+
+// Up to this many positions (one string, or a batch) the lengths of Lemma 1
+// go straight to a dense array in text order (2 bytes each, scattered stores
+// that merge in L2) instead of through the radix partition.  Where the lines
+// lie: front end DNA 2 x 10^5 positions 23 us against 37 us with the
+// partition, 2^20 30 and 40 us, 3 x 10^6 51 and 50 us, 8 x 10^6 99 and 83 us
+// (scattered stores run at 110 G/s whatever the size, the partition gains
+// with it); a batch of 10^7 131 and 136 us (its partition looks strings up).
+constexpr long long kDenseMaxN = 1LL << 20;
+constexpr long long kDenseMaxBatch = 12LL << 20;
+constexpr int kCompactTile = 8192;             // positions per CTA that compacts the dense array
+
 // Polls of a look-back status word before the wait is declared lost (a
 // few seconds at most; the kernel then reports kErrTimeout and finishes).
 constexpr int kSpinLimit = 1 << 23;
@@ -58,6 +74,7 @@ struct Scratch {
     uint32_t* ent2;                // nbuckets x 2^15: the same entries by bucket of 2^15 positions
     unsigned* cursor1;             // fill counts of ent1, one per kCursorStride words (cleared per query)
     unsigned* cursor2;             // fill counts of ent2, one per kCursorStride words (cleared per query)
+    uint16_t* dense;               // n: lengths in text order of the dense front end (in the ent1 region)
     int32_t* lbig;                 // n: L of positions whose length field escaped
     int32_t* halo;                 // nbuckets + 1: L of the position before each bucket
     int32_t* tile_seg;             // ntiles: first string overlapping each tile (batched queries)
@@ -73,6 +90,7 @@ struct Scratch {
                                    // per query); null where the scratch has no room for the rank-window front
     unsigned long long* went = nullptr;   // n: rank-window entries rank << 32 | i (in the cstart / cend region)
     long long nwins = 0;
+    bool one_tile = false;         // short strings may take the one-tile kernel (nothing is cleared before it)
     int spin_limit = kSpinLimit;   // polls of one look-back wait before it gives up
     long long hold_tile = -1;      // test hook: this cover tile never publishes its look-back word
 };
@@ -125,6 +143,14 @@ void launch_gather_front(const int32_t* rank, const int32_t* lcp, int32_t n, con
                          cudaStream_t stream);
 void launch_partition(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                       cudaStream_t stream);
+// the dense front end: k_scatter, k_compact
+void launch_scatter(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
+                    cudaStream_t stream);
+void launch_compact(int32_t n, const Scratch& s, cudaStream_t stream);
+// k_one_tile: the whole query of a string of at most kOneTileMax positions
+void launch_one_tile(const int32_t* sa, const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s,
+                     int32_t* lr_len, int32_t* lr_start, int64_t* offsets, int32_t* starts, long long capacity, bool all,
+                     cudaStream_t stream);
 void launch_bucket_front(int32_t n, const Scratch& s, cudaStream_t stream);
 // k_rank_win, k_part1_win and k_part2 (the rank-window front end up to the bucket kernel)
 void launch_rank_window_front(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s,
