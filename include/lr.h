@@ -20,13 +20,15 @@
  * takes sa or rank (at least one; when both are given, sa is used unless
  * lr_autotune chose the rank front end for queries of that size):
  *   - with sa, the lengths are computed in rank order (sa and lcp read
- *     once, coalesced) and radix-partitioned back to text order;
+ *     once, coalesced) and radix-partitioned back to text order, or, up to a
+ *     few million positions, stored straight at their positions;
  *   - with rank only, each position gathers its two lcp words, the paper's
  *     own data flow (Sec. 4): one random 32-byte sector per position.  For
  *     one string of 2^24 positions or more (not a batch, not the static
  *     call), the pairs <rank[i], i> are first partitioned into windows of
  *     2^22 ranks, so that each window's gathers hit L2, and then join the
  *     sa path's partition.
+ * A string of at most 8192 positions is answered by one kernel.
  * All give identical results.  sa must be a permutation of [0, n) and rank
  * its inverse; a violation that the kernels detect is reported as
  * LR_ERR_SENTINEL, and no input ever makes a kernel access memory out of
@@ -429,8 +431,10 @@ lr_status lr_test_hold_lookback(lr_ctx* ctx, int64_t tile, int32_t spin_limit);
 
 /*
  * Kernels launched by the most recent query of this context (for the
- * benchmark's launch accounting): 4 with sa, 2 with rank only, one more for
- * a batch; 2 for the raw-LLR variant, 4 for lr_walk_stats.
+ * benchmark's launch accounting): 1 for a string of at most 8192 positions;
+ * else 4 with sa (one more for a batch that takes the partition), 2 with
+ * rank only (5 through the rank windows), one more for a batch; 2 for the
+ * raw-LLR variant, 4 for lr_walk_stats.
  */
 int32_t lr_last_launch_count(lr_ctx* ctx);
 
@@ -441,8 +445,10 @@ int32_t lr_last_launch_count(lr_ctx* ctx);
  * the duration in milliseconds of each of its phases, in launch order, into
  * ms[0 .. cap); it returns the number of phases of that query, or -1 if
  * timing was off or an event failed.  The phases are: with sa, the
- * partition (two kernels), the bucket front end and the cover kernel;
- * with rank only, the gather front end and the cover kernel.
+ * partition (two kernels), the bucket front end and the cover kernel, or, up
+ * to a few million positions, the dense array, its compaction and the cover
+ * kernel; with rank only, the gather front end and the cover kernel; one
+ * phase for a string of at most 8192 positions.
  */
 lr_status lr_set_phase_timing(lr_ctx* ctx, int32_t enable);
 int32_t lr_phase_times(lr_ctx* ctx, float* ms, int32_t cap);

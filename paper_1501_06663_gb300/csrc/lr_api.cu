@@ -20,7 +20,7 @@ struct lr_ctx {
     unsigned char* scratch = nullptr;     // lr::Scratch storage
     size_t scratch_bytes = 0;
     long long scratch_n = 0;              // positions the scratch is laid out for
-    long long* h_pinned = nullptr;        // [0] total, [1] error bits
+    long long* h_pinned = nullptr;        // [0], [1] Readback, [2] compact size
     unsigned char* hostpath = nullptr;    // device buffers of lr_query_all_host
     size_t hostpath_bytes = 0;
     int sms = 0;                          // SM count of the device
@@ -42,9 +42,8 @@ struct lr_plan {
     unsigned* d_err = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    const int64_t* d_total = nullptr;     // d_offsets + total
     int64_t capacity = 0;
-    long long* h_pinned = nullptr;        // 2 words: total, error bits
+    long long* h_pinned = nullptr;        // 2 words: Readback
 };
 
 namespace {
@@ -72,6 +71,9 @@ lr_status cuda_fail(lr_ctx* ctx, cudaError_t e) {
     ctx->last_cuda_error = (int)e;
     return e == cudaErrorMemoryAllocation ? LR_ERR_NOMEM : LR_ERR_CUDA;
 }
+
+// The word of an error block that takes the total (see Readback).
+inline long long* total_word(unsigned* d_err) { return reinterpret_cast<long long*>(d_err + 2); }
 
 struct Layout {
     size_t off_status_g, off_status_b, off_status_o, off_status_w, off_cursor1, off_cursor2, off_cursor_w, zero_end;
@@ -157,6 +159,7 @@ lr_status get_scratch(lr_ctx* ctx, long long n, lr::Scratch* s) {
     carve(ctx->scratch, ctx->scratch_n, n, ctx->d_err, s);
     s->spin_limit = ctx->spin_limit;
     s->hold_tile = ctx->hold_tile;
+    s->total_out = total_word(ctx->d_err);
     s->one_tile = ctx->hold_tile < 0;              // the test hook needs the look-back
     ctx->last_n = n;
     return LR_OK;
@@ -220,8 +223,6 @@ lr_status device_bits_to_status(unsigned bits) {
     return LR_OK;
 }
 
-// Copies the total (offsets[n]) and the error bits to the host, waits, and
-// clears the error word.
 }  // namespace
 
 namespace lr {
@@ -230,15 +231,32 @@ lr_status status_of_bits(unsigned bits) { return device_bits_to_status(bits); }
 
 namespace {
 
-lr_status sync_total(lr_ctx* ctx, cudaStream_t stream, const int64_t* d_total, int64_t* h_total) {
-    cudaError_t e = cudaSuccess;
-    if (d_total) e = cudaMemcpyAsync(&ctx->h_pinned[0], d_total, 8, cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&ctx->h_pinned[1], ctx->d_err, 4, cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_err, 0, 4, stream);
+// What a synchronising call reads back: the error word and, eight bytes on,
+// the last query's total (Scratch::total_out), in one copy.
+struct Readback {
+    unsigned bits, pad;
+    long long total;
+};
+
+// Waits for the stream and returns the status of the error bits, which are
+// cleared; *h_total (when non-null) receives the total.
+lr_status read_back(cudaStream_t stream, unsigned* d_err, Readback* h, int64_t* h_total, cudaError_t* err) {
+    cudaError_t e = cudaMemcpyAsync(h, d_err, sizeof(Readback), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e);
-    if (h_total && d_total) *h_total = ctx->h_pinned[0];
-    return device_bits_to_status((unsigned)(ctx->h_pinned[1] & 0xffffffffu));
+    if (e == cudaSuccess && h->bits) {
+        e = cudaMemsetAsync(d_err, 0, 4, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    }
+    *err = e;
+    if (e != cudaSuccess) return LR_ERR_CUDA;
+    if (h_total) *h_total = h->total;
+    return device_bits_to_status(h->bits);
+}
+
+lr_status sync_total(lr_ctx* ctx, cudaStream_t stream, int64_t* h_total) {
+    cudaError_t e;
+    const lr_status st = read_back(stream, ctx->d_err, reinterpret_cast<Readback*>(ctx->h_pinned), h_total, &e);
+    return e == cudaSuccess ? st : cuda_fail(ctx, e);
 }
 
 }  // namespace
@@ -373,7 +391,7 @@ lr_status lr_device_status(lr_ctx* ctx, lr_stream_t stream) {
     if (!ctx) return LR_ERR_ARG;
     DeviceGuard g(ctx->device);
     if (!g.ok) return cuda_fail(ctx, cudaErrorInvalidDevice);
-    return sync_total(ctx, (cudaStream_t)stream, nullptr, nullptr);
+    return sync_total(ctx, (cudaStream_t)stream, nullptr);
 }
 
 lr_status lr_query_leftmost(lr_ctx* ctx, lr_stream_t stream, const int32_t* d_sa, const int32_t* d_rank,
@@ -413,7 +431,7 @@ lr_status lr_query_all(lr_ctx* ctx, lr_stream_t stream, const int32_t* d_sa, con
                                      lr::Segs{nullptr, 0}, shape);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     if (!h_total) return LR_OK;
-    st = sync_total(ctx, (cudaStream_t)stream, d_offsets + n, h_total);
+    st = sync_total(ctx, (cudaStream_t)stream, h_total);
     if (st != LR_OK) return st;
     return (*h_total > starts_capacity) ? LR_ERR_CAPACITY : LR_OK;
 }
@@ -464,7 +482,7 @@ lr_status lr_query_all_host(lr_ctx* ctx, lr_stream_t stream, const int32_t* h_sa
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_lr_start, d_start, nn * 4, cudaMemcpyDeviceToHost, strm);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_offsets, d_off, (nn + 1) * 8, cudaMemcpyDeviceToHost, strm);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
-    st = sync_total(ctx, strm, d_off + n, h_total);
+    st = sync_total(ctx, strm, h_total);
     if (st != LR_OK) return st;
     const int64_t tot = *h_total;
     const int64_t copy = tot < starts_capacity ? tot : starts_capacity;
@@ -593,7 +611,7 @@ lr_status lr_query_all_raw(lr_ctx* ctx, lr_stream_t stream, const int32_t* d_ran
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     ctx->last_launches = 2;
     if (!h_total) return LR_OK;
-    st = sync_total(ctx, (cudaStream_t)stream, d_offsets + n, h_total);
+    st = sync_total(ctx, (cudaStream_t)stream, h_total);
     if (st != LR_OK) return st;
     return (*h_total > starts_capacity) ? LR_ERR_CAPACITY : LR_OK;
 }
@@ -633,7 +651,7 @@ lr_status lr_walk_stats(lr_ctx* ctx, lr_stream_t stream, const int32_t* d_rank, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(&m, s.tile_cbase + s.ntiles, 4, cudaMemcpyDeviceToHost, strm);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     ctx->last_launches = 4;
-    st = sync_total(ctx, strm, nullptr, nullptr);
+    st = sync_total(ctx, strm, nullptr);
     if (st != LR_OK) return st;
     const int32_t* w = reinterpret_cast<const int32_t*>(hs + 2);
     h_summary->n = n;
@@ -683,7 +701,7 @@ lr_status lr_batch_query_all(lr_ctx* ctx, lr_stream_t stream, const lr_batch_des
     st = batch_launch(ctx, (cudaStream_t)stream, batch, tuned_code(ctx, batch->total, batch->num), d_lr_len,
                       d_lr_start, d_offsets, d_starts, starts_capacity);
     if (st != LR_OK || !h_total) return st;
-    st = sync_total(ctx, (cudaStream_t)stream, d_offsets + batch->total, h_total);
+    st = sync_total(ctx, (cudaStream_t)stream, h_total);
     if (st != LR_OK) return st;
     return (*h_total > starts_capacity) ? LR_ERR_CAPACITY : LR_OK;
 }
@@ -722,7 +740,7 @@ lr_status lr_autotune(lr_ctx* ctx, lr_stream_t stream, const lr_batch_desc* batc
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != LR_OK) return st;
-    st = sync_total(ctx, strm, nullptr, nullptr);
+    st = sync_total(ctx, strm, nullptr);
     if (st != LR_OK) return st;
     ctx->tuned[shape_class(batch->total, batch->num)] = best;
     *choice = best;
@@ -761,7 +779,6 @@ lr_status lr_plan_create(lr_ctx* ctx, const lr_batch_desc* batch, int32_t* d_lr_
     lr_plan* plan = new (std::nothrow) lr_plan();
     if (!plan) return LR_ERR_NOMEM;
     plan->device = ctx->device;
-    plan->d_total = d_offsets + batch->total;
     plan->capacity = starts_capacity;
     const Layout L = layout_for(batch->total);
     cudaStream_t cs = nullptr;
@@ -773,6 +790,7 @@ lr_status lr_plan_create(lr_ctx* ctx, const lr_batch_desc* batch, int32_t* d_lr_
     if (e == cudaSuccess) {
         lr::Scratch s;
         carve(plan->scratch, batch->total, batch->total, plan->d_err, &s);
+        s.total_out = total_word(plan->d_err);
         const int code = tuned_code(ctx, batch->total, batch->num);
         const bool use_rank = (code & 2) && batch->d_rank;
         const int32_t* sa = use_rank ? nullptr : batch->d_sa;
@@ -809,15 +827,13 @@ lr_status lr_plan_result(lr_plan* plan, lr_stream_t stream, int64_t* h_total) {
     DeviceGuard g(plan->device);
     if (!g.ok) return LR_ERR_CUDA;
     cudaStream_t strm = (cudaStream_t)stream;
-    cudaError_t e = cudaMemcpyAsync(&plan->h_pinned[0], plan->d_total, 8, cudaMemcpyDeviceToHost, strm);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&plan->h_pinned[1], plan->d_err, 4, cudaMemcpyDeviceToHost, strm);
-    if (e == cudaSuccess) e = cudaMemsetAsync(plan->d_err, 0, 4, strm);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(strm);
+    cudaError_t e;
+    int64_t total = 0;
+    const lr_status st = read_back(strm, plan->d_err, reinterpret_cast<Readback*>(plan->h_pinned), &total, &e);
     if (e != cudaSuccess) { cudaGetLastError(); return LR_ERR_CUDA; }
-    if (h_total) *h_total = plan->h_pinned[0];
-    lr_status st = device_bits_to_status((unsigned)(plan->h_pinned[1] & 0xffffffffu));
+    if (h_total) *h_total = total;
     if (st != LR_OK) return st;
-    return plan->h_pinned[0] > plan->capacity ? LR_ERR_CAPACITY : LR_OK;
+    return total > plan->capacity ? LR_ERR_CAPACITY : LR_OK;
 }
 
 lr_status lr_plan_destroy(lr_plan* plan) {

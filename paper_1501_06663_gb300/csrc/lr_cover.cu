@@ -159,7 +159,10 @@ __device__ __forceinline__ long long place_tile(const Scratch& s, long long tile
     const long long ex = (tile == 0) ? 0 : lookback(s.status_o, tile, s.err, s.qerr, s.spin_limit);
     if (lane_id() == 0) {
         if (tile != 0 && tile != s.hold_tile) publish(s.status_o, tile, kPrefix, ex + tot);
-        if (tile == ntiles - 1) offsets[n] = ex + tot;
+        if (tile == ntiles - 1) {
+            offsets[n] = ex + tot;
+            if (s.total_out) *s.total_out = ex + tot;
+        }
     }
     return ex;
 }
@@ -172,7 +175,7 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
                                               int32_t cb1, int32_t* __restrict__ lr_len, int32_t* __restrict__ lr_start,
                                               int64_t* __restrict__ offsets, int32_t* __restrict__ starts,
                                               long long capacity) {
-    constexpr int kCoverTile = Cfg<TP>::kTileC, kCoverThreads = Cfg<TP>::kThr, kWarps = Cfg<TP>::kWarps;
+    constexpr int kCoverTile = Cfg<TP>::kTileC, kCoverThreads = Cfg<TP>::kThr;
     constexpr int kChunks = Cfg<TP>::kChunks, kChunksPerWarp = Cfg<TP>::kChunksPerWarp;
     static_assert(sizeof(LongSmem<TP>) <= sizeof(sm.ent), "the bitmaps replace the staged entries");
     LongSmem<TP>& lm = *reinterpret_cast<LongSmem<TP>*>(sm.ent);
@@ -183,7 +186,7 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
         int32_t t = cb0;
         while (t > 0) {
             const int32_t idx = t - 1 - lane;
-            const bool reach = idx >= 0 && __ldg(s.cend + idx) >= k0;
+            const bool reach = idx >= 0 && s.cend[idx] >= k0;
             const unsigned m = __ballot_sync(kFull, reach);
             if (m == kFull) { t -= kWarp; continue; }
             t -= __ffs(~m) - 1;
@@ -194,7 +197,7 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
     __syncthreads();
     const int32_t lo = sm.lo, C = cb0 - lo, M = cb1 - lo;
     for (int i = tid; i < M; i += kCoverThreads) {
-        const int32_t cs = __ldg(s.cstart + lo + i), ce = __ldg(s.cend + lo + i);
+        const int32_t cs = s.cstart[lo + i], ce = s.cend[lo + i];
         const uint32_t xs = (uint32_t)(cs - k0), xe = (uint32_t)(ce - k0);
         if (i >= C && xs < (uint32_t)kCoverTile) atomicOr(&lm.smap[xs >> 5], 1u << (xs & 31));
         if (xe < (uint32_t)kCoverTile) atomicOr(&lm.emap[xe >> 5], 1u << (xe & 31));
@@ -215,7 +218,7 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
     auto best_of = [&](int32_t lw, int32_t hi, int32_t& b, int32_t& vb, int32_t& ct) {
         b = 0; vb = -1; ct = 0;
         for (int32_t v = lw; v <= hi; ++v) {
-            const int32_t len = __ldg(gce + v) - __ldg(gcs + v) + 1;
+            const int32_t len = gce[v] - gcs[v] + 1;
             const bool gt = len > b;
             ct = gt ? 1 : ct + (len == b);
             vb = gt ? v : vb;
@@ -232,7 +235,7 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
         best_of(lw, hi, b, vb, ct);
         if (k < n) {
             __stcs(lr_len + k, b);
-            __stcs(lr_start + k, b > 0 ? __ldg(gcs + vb) : -1);
+            __stcs(lr_start + k, b > 0 ? gcs[vb] : -1);
         }
         pk[q] = k < n ? ct : 0;
         if constexpr (kAll) {
@@ -261,8 +264,8 @@ __device__ __noinline__ void cover_long_carry(CoverSmem<TP>& sm, int32_t n, cons
             window(c, lw, hi);
             best_of(lw, hi, b, vb, ct);
             for (int32_t v = vb; v <= hi; ++v) {
-                if (__ldg(gce + v) - __ldg(gcs + v) + 1 != b) continue;
-                if (o < capacity) __stcs(starts + o, __ldg(gcs + v));
+                if (gce[v] - gcs[v] + 1 != b) continue;
+                if (o < capacity) __stcs(starts + o, gcs[v]);
                 ++o;
             }
         }
@@ -280,7 +283,6 @@ __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, cons
                                               int32_t* __restrict__ starts, long long capacity) {
     constexpr int kCoverTile = Cfg<TP>::kTileC;
     constexpr int kCoverThreads = Cfg<TP>::kThr;
-    constexpr int kWarps = Cfg<TP>::kWarps;
     constexpr int kChunksPerWarp = Cfg<TP>::kChunksPerWarp;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // Per entry: the positions of the tile [hs, he) where it is a holder, the
@@ -390,15 +392,19 @@ __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, cons
         sum = (int32_t)__reduce_add_sync(kFull, (unsigned)sum);
         if (lane == 0) sm.wtot[warp] = sum;
         if (kOne) {
-            if (tid == 0) { sm.obase = 0; offsets[n] = sm.ttot; }
-        } else if (warp == kWarps - 1) {
+            if (tid == 0) {
+                sm.obase = 0;
+                offsets[n] = sm.ttot;
+                if (s.total_out) *s.total_out = sm.ttot;
+            }
+        } else if (warp == Cfg<TP>::kWarps - 1) {
             const long long ex = place_tile(s, tile, num_cover_tiles(n, TP), n, sm.ttot, offsets);
             if (lane == 0) sm.obase = ex;
         }
         __syncthreads();
         long long o0 = sm.obase;
         {
-            const int32_t t = lane < warp ? sm.wtot[lane < kWarps ? lane : 0] : 0;
+            const int32_t t = lane < warp ? sm.wtot[lane] : 0;
             o0 += (int32_t)__reduce_add_sync(kFull, (unsigned)t);
         }
         // starts[o0 ..]: 32-bit indices from here; entries past the capacity are not written
@@ -456,6 +462,7 @@ template <bool kAll, int TP>
 __global__ void __launch_bounds__(Cfg<TP>::kThr, Cfg<TP>::kMinBlocks)
 k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict__ lr_start,
         int64_t* __restrict__ offsets, int32_t* __restrict__ starts, long long capacity) {
+    begin_last();
     constexpr int kCoverTile = Cfg<TP>::kTileC;
     constexpr int kCoverThreads = Cfg<TP>::kThr;
     constexpr int kCoverTilesPer = TP;
@@ -499,8 +506,8 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const int i = i0 + u * kCoverThreads + tid;
-            cs[u] = i < MS ? __ldg(s.cstart + sbase + i) : 0;
-            ce[u] = i < MS ? __ldg(s.cend + sbase + i) : 0;
+            cs[u] = i < MS ? __ldcg(s.cstart + sbase + i) : 0;
+            ce[u] = i < MS ? __ldcg(s.cend + sbase + i) : 0;
         }
         if (i0 == 0 && warp < kSpec / kWarp) {
             const unsigned m = __ballot_sync(kFull, tid < nspec && ce[0] < k0);
@@ -635,8 +642,8 @@ template <bool kAll, int TP>
 void launch_cover_t(int32_t n, const Scratch& s, int32_t* lr_len, int32_t* lr_start, int64_t* offsets,
                     int32_t* starts, long long capacity, cudaStream_t stream) {
     const unsigned grid = (unsigned)num_cover_tiles(n, TP);
-    k_cover<kAll, TP><<<grid, Cfg<TP>::kThr, sizeof(CoverSmem<TP>), stream>>>(n, s, lr_len, lr_start, offsets, starts,
-                                                                              capacity);
+    launch_after(k_cover<kAll, TP>, grid, Cfg<TP>::kThr, sizeof(CoverSmem<TP>), stream, n, s, lr_len, lr_start, offsets, starts,
+                 capacity);
 }
 
 template <int TP>

@@ -85,10 +85,10 @@ struct Range {
     const int32_t* cs;
     const int32_t* ce;                       // staged: lengths; in place: ends
     __device__ __forceinline__ int32_t s(int32_t v) const {
-        if constexpr (kStaged) return cs[v]; else return __ldg(cs + v);
+        if constexpr (kStaged) return cs[v]; else return cs[v];
     }
     __device__ __forceinline__ int32_t len(int32_t v) const {
-        if constexpr (kStaged) return ce[v]; else return __ldg(ce + v) - __ldg(cs + v) + 1;
+        if constexpr (kStaged) return ce[v]; else return ce[v] - cs[v] + 1;
     }
 };
 
@@ -157,7 +157,7 @@ __device__ __forceinline__ bool stage_segment(const Scratch& s, WarpStage& W, in
     for (int32_t i0 = 0; i0 < M; i0 += kWarp) {
         const int32_t i = i0 + (int32_t)lane;
         if (i < M) {
-            const int32_t cs = __ldg(s.cstart + lo + i), ce = __ldg(s.cend + lo + i);
+            const int32_t cs = __ldcg(s.cstart + lo + i), ce = __ldcg(s.cend + lo + i);
             const int32_t len = ce - cs + 1;
             if (fits) { W.cs[i] = cs; W.cl[i] = len; }
             longlen |= len >= (1 << 27);
@@ -330,6 +330,7 @@ template <bool kAll>
 __global__ void __launch_bounds__(kSegThreads, 3)
 k_cover_w(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict__ lr_start,
           int64_t* __restrict__ offsets, int32_t* __restrict__ starts, long long capacity) {
+    begin_last();
     extern __shared__ __align__(16) unsigned char wsm_raw[];
     CoverWSmem& sm = *reinterpret_cast<CoverWSmem*>(wsm_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -355,7 +356,7 @@ k_cover_w(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restric
         lo = c0;
         while (lo > 0) {
             const int32_t idx = lo - 1 - lane;
-            const bool reach = idx >= 0 && __ldg(s.cend + idx) >= p0;
+            const bool reach = idx >= 0 && s.cend[idx] >= p0;
             const unsigned mk = __ballot_sync(kFull, reach);
             if (mk == kFull) { lo -= kWarp; continue; }
             lo -= __ffs(~mk) - 1;
@@ -390,7 +391,10 @@ k_cover_w(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restric
         const long long ex = (tile == 0) ? 0 : lookback(s.status_w, tile, s.err, s.qerr, s.spin_limit);
         if (lane == 0) {
             if (tile != 0 && !held) publish(s.status_w, tile, kPrefix, ex + tile_tot);
-            if ((tile + 1) * kSegWarps >= s.nsegs) offsets[n] = ex + tile_tot;
+            if ((tile + 1) * kSegWarps >= s.nsegs) {
+                offsets[n] = ex + tile_tot;
+                if (s.total_out) *s.total_out = ex + tile_tot;
+            }
             sm.tile_ex = ex;
         }
     }
@@ -406,9 +410,9 @@ void launch_cover_w(int32_t n, const Scratch& s, int32_t* lr_len, int32_t* lr_st
     const unsigned grid = (unsigned)((s.nsegs + kSegWarps - 1) / kSegWarps);
     const size_t smem = sizeof(CoverWSmem);
     if (all)
-        k_cover_w<true><<<grid, kSegThreads, smem, stream>>>(n, s, lr_len, lr_start, offsets, starts, capacity);
+        launch_after(k_cover_w<true>, grid, kSegThreads, smem, stream, n, s, lr_len, lr_start, offsets, starts, capacity);
     else
-        k_cover_w<false><<<grid, kSegThreads, smem, stream>>>(n, s, lr_len, lr_start, nullptr, nullptr, 0);
+        launch_after(k_cover_w<false>, grid, kSegThreads, smem, stream, n, s, lr_len, lr_start, nullptr, nullptr, 0);
 }
 
 cudaError_t configure_cover_w() {

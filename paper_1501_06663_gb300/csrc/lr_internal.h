@@ -47,11 +47,11 @@ constexpr int kOneTileMax = 8192;
 // Up to this many positions (one string, or a batch) the lengths of Lemma 1
 // go straight to a dense array in text order (2 bytes each, scattered stores
 // that merge in L2) instead of through the radix partition.  Where the lines
-// lie: front end DNA 2 x 10^5 positions 23 us against 37 us with the
-// partition, 2^20 30 and 40 us, 3 x 10^6 51 and 50 us, 8 x 10^6 99 and 83 us
+// lie: whole queries, dense and partition, DNA: 2 x 10^5 positions 59 and
+// 78 us, 2^20 84 and 101 us, 4 x 10^6 134 and 141 us, 8 x 10^6 202 and 193 us
 // (scattered stores run at 110 G/s whatever the size, the partition gains
-// with it); a batch of 10^7 131 and 136 us (its partition looks strings up).
-constexpr long long kDenseMaxN = 1LL << 20;
+// with it); a batch of 10^7 248 and 264 us (its partition looks strings up).
+constexpr long long kDenseMaxN = 5LL << 20;
 constexpr long long kDenseMaxBatch = 12LL << 20;
 constexpr int kCompactTile = 8192;             // positions per CTA that compacts the dense array
 
@@ -90,6 +90,7 @@ struct Scratch {
                                    // per query); null where the scratch has no room for the rank-window front
     unsigned long long* went = nullptr;   // n: rank-window entries rank << 32 | i (in the cstart / cend region)
     long long nwins = 0;
+    long long* total_out = nullptr;   // also receives the number of LR starts, where set
     bool one_tile = false;         // short strings may take the one-tile kernel (nothing is cleared before it)
     int spin_limit = kSpinLimit;   // polls of one look-back wait before it gives up
     long long hold_tile = -1;      // test hook: this cover tile never publishes its look-back word
@@ -130,6 +131,22 @@ struct Shape {
     int cover_tiles_per = 1;       // its tile = kTile x this (1, 2 or 4)
 };
 
+// Launch of a kernel that begins with begin_after().
+template <typename... P, typename... A>
+inline void launch_after(void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, (P)args...);     // errors: the launch sequence's cudaGetLastError
+}
+
 // Launches the whole query on `stream`: the front end (rank-order when sa is
 // non-null, else the rank gather) and the cover kernel.
 cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s,
@@ -143,7 +160,9 @@ void launch_gather_front(const int32_t* rank, const int32_t* lcp, int32_t n, con
                          cudaStream_t stream);
 void launch_partition(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                       cudaStream_t stream);
-// the dense front end: k_scatter, k_compact
+// the dense front end: k_prep, k_scatter, k_compact
+// k_prep clears what the dense path needs cleared and, for a batch, does k_seg_index's work
+void launch_prep(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream);
 void launch_scatter(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                     cudaStream_t stream);
 void launch_compact(int32_t n, const Scratch& s, cudaStream_t stream);

@@ -37,13 +37,16 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
         if (events) events->count = k;
         return cudaGetLastError();
     }
-    cudaError_t e = cudaMemsetAsync(s.zero_base, 0, s.zero_bytes, stream);
-    if (e != cudaSuccess) return e;
-    if (segs.num > 0) launch_seg_index(n, s, segs, stream);                     // k_seg_index
-    const bool rankwin = !sa && segs.num == 0 && s.cursor_w && (long long)n >= kRankWinMinN;
     const bool dense = sa && (long long)n <= (segs.num > 0 ? kDenseMaxBatch : kDenseMaxN);
+    if (!dense) {
+        cudaError_t e = cudaMemsetAsync(s.zero_base, 0, s.zero_bytes, stream);
+        if (e != cudaSuccess) return e;
+        if (segs.num > 0) launch_seg_index(n, s, segs, stream);                 // k_seg_index
+    }
+    const bool rankwin = !sa && segs.num == 0 && s.cursor_w && (long long)n >= kRankWinMinN;
     if (dense) {
         mark();
+        launch_prep(n, s, segs, stream);                    // k_prep
         launch_scatter(sa, lcp, n, s, segs, stream);        // k_scatter
         mark();
         launch_compact(n, s, stream);                       // k_compact
@@ -67,7 +70,7 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
     else
         launch_cover_w(n, s, lr_len, lr_start, offsets, starts, capacity, all, stream);
     if (timed) cudaEventRecord(events->ev[k], stream);
-    if (launches) *launches = (dense ? 3 : (sa ? 4 : (rankwin ? 5 : 2))) + (segs.num > 0 ? 1 : 0);
+    if (launches) *launches = dense ? 4 : (sa ? 4 : (rankwin ? 5 : 2)) + (segs.num > 0 ? 1 : 0);
     if (events) events->count = k;
     return cudaGetLastError();
 }

@@ -114,7 +114,10 @@ __global__ void __launch_bounds__(kRawThreads) k_rawwalk(int32_t n, const int32_
             const long long ex = lookback_exclusive(s.status_o, tile, tot, s.err, s.qerr, s.spin_limit);
             if (lane == 0) {
                 obase_s = ex;
-                if (k0 + kRawTile >= n) offsets[n] = ex + tot;
+                if (k0 + kRawTile >= n) {
+                    offsets[n] = ex + tot;
+                    if (s.total_out) *s.total_out = ex + tot;
+                }
             }
         }
         __syncthreads();
