@@ -528,7 +528,9 @@ def single_leg(lr, dev, stream, name: str, steps: int, warmup: int):
     inputs_mb = (8 * n + 4) / 1e6
     return {"workload": name, "n": n, "ms_per_step": round(ms, 4), "value": round(n / (ms * 1e-3) / 1e9, 3),
             "unit": UNIT, "steps": steps, "total_lr_starts": total,
-            "kernel_ms": {nm: round(p, 4) for nm, p in zip(["partition", "bucket_llr", "cover"], phases or [])},
+            # up to 5 x 2^20 positions the lengths go to a dense array instead of through the partition
+            "kernel_ms": {nm: round(p, 4) for nm, p in zip(["partition", "bucket_llr", "cover"] if n > 5 << 20 else
+                                                           ["scatter", "compact", "cover"], phases or [])},
             "path_roofline": {"achieved": round(path_bytes / (ms * 1e-3) / 1e9, 1), "peak": peak, "unit": "GB/s",
                               "frac": round(path_bytes / (ms * 1e-3) / 1e9 / peak, 4), "peak_kind": peak_kind},
             "l2": "inputs %.0f MB: %s" % (inputs_mb, "larger than the 129 MB L2" if inputs_mb > 129 else
@@ -627,8 +629,9 @@ def run_ours(args):
     torch.cuda.synchronize(dev)
     gather_ms = g0.elapsed_time(g1) / gsteps
     per_gather = phase_avg(sa=None, rank=d_rank)
-    rank_front = "rank windows" if len(per_gather) == 3 else "rank gather"
-    rank_names = ["rank_windows_partition", "bucket_llr", "cover"] if len(per_gather) == 3 else ["gather_llr", "cover"]
+    rank_front = "rank windows" if n >= 1 << 24 else "rank gather"
+    rank_names = (["rank_windows_partition", "bucket_llr", "cover"] if n >= 1 << 24 else
+                  ["gather", "compact", "cover"] if len(per_gather) == 3 else ["one_tile"])
     # the paper's data flow itself (rank + a random gather of lcp), run as a
     # batch of one string, which always takes the gather
     paper_gather = None
@@ -647,7 +650,7 @@ def run_ours(args):
         pg = lr.lr_phase_times(ctx)
         lr.lr_set_phase_timing(ctx, False)
         paper_gather = {"ms_per_step": round(pg_ms, 4), "value": round(whole_job_rate(ws, n, pg_ms), 3),
-                        "kernel_ms": {nm: round(t, 4) for nm, t in zip(["gather_llr", "cover"], pg)},
+                        "kernel_ms": {nm: round(t, 4) for nm, t in zip(["gather", "compact", "cover"], pg)},
                         "how": "one-string batch (lr_batch_query_all), rank only"}
 
     # the leftmost-only query (Algorithm 2's output, no CSR pass), same front end

@@ -390,7 +390,7 @@ lr_status lr_server_stop(lr_server* server);
  * allocation would synchronise the whole device and stall unrelated work),
  * or services that fix their memory budget once at start-up.  It needs no
  * context and allocates nothing: its working memory is one array of about
- * 8 MB compiled into this library's device image, which every GPU that
+ * 10 MB compiled into this library's device image, which every GPU that
  * loads the library keeps until the process exits.
  *
  * Same inputs and outputs as lr_query_all with rank (the rank-gather front
@@ -432,9 +432,8 @@ lr_status lr_test_hold_lookback(lr_ctx* ctx, int64_t tile, int32_t spin_limit);
 /*
  * Kernels launched by the most recent query of this context (for the
  * benchmark's launch accounting): 1 for a string of at most 8192 positions;
- * else 4 with sa (one more for a batch that takes the partition), 2 with
- * rank only (5 through the rank windows), one more for a batch; 2 for the
- * raw-LLR variant, 4 for lr_walk_stats.
+ * else 4 (5 through the rank windows, one more for a batch that takes the
+ * partition); 2 for the raw-LLR variant, 6 for lr_walk_stats.
  */
 int32_t lr_last_launch_count(lr_ctx* ctx);
 
@@ -444,11 +443,10 @@ int32_t lr_last_launch_count(lr_ctx* ctx);
  * launches.  lr_phase_times() waits for the last query's events and writes
  * the duration in milliseconds of each of its phases, in launch order, into
  * ms[0 .. cap); it returns the number of phases of that query, or -1 if
- * timing was off or an event failed.  The phases are: with sa, the
- * partition (two kernels), the bucket front end and the cover kernel, or, up
- * to a few million positions, the dense array, its compaction and the cover
- * kernel; with rank only, the gather front end and the cover kernel; one
- * phase for a string of at most 8192 positions.
+ * timing was off or an event failed.  The phases are the lengths by
+ * position (the partition, two kernels, the dense array, two, or the rank
+ * windows, three), their compaction and the cover kernel; one phase for a
+ * string of at most 8192 positions.
  */
 lr_status lr_set_phase_timing(lr_ctx* ctx, int32_t enable);
 int32_t lr_phase_times(lr_ctx* ctx, float* ms, int32_t cap);

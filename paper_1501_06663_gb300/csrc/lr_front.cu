@@ -24,8 +24,8 @@
 //    tile by tile (k_compact).
 //
 //  * rank gather (when only rank is given, as in the paper's data flow of
-//    Sec. 4): k_gather_llr reads rank coalesced and gathers the two lcp
-//    words of each position, then flags and compacts one tile.
+//    Sec. 4): k_gather reads rank coalesced, gathers the two lcp words of each
+//    position and stores the lengths in the same dense array.
 //
 // All place their entries in LLRc with a decoupled look-back over the
 // per-CTA counts (tiles handed out in order by an atomic ticket).
@@ -41,16 +41,6 @@ namespace {
 __device__ __forceinline__ void report(const Scratch& s, unsigned bits) {
     atomicOr(s.err, bits);
     atomicOr(s.qerr, bits);
-}
-
-// Exclusive scan of 64 ints by one warp (two per lane); returns the total.
-__device__ __forceinline__ int warp_scan64(int32_t* a) {
-    const int lane = lane_id();
-    const int x = a[2 * lane], y = a[2 * lane + 1];
-    const int incl = warp_incl_scan(x + y);
-    a[2 * lane] = incl - x - y;
-    a[2 * lane + 1] = incl - y;
-    return __shfl_sync(kFull, incl, kWarp - 1);
 }
 
 // The strings of a batched query that overlap one CTA's flattened range
@@ -123,171 +113,6 @@ __global__ void k_seg_index(int32_t n, Scratch s, Segs segs) {
 
 void launch_seg_index(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream) {
     k_seg_index<<<(unsigned)((s.ntiles + 255) / 256), 256, 0, stream>>>(n, s, segs);
-}
-
-// ---------------------------------------------------------------------------
-// rank gather front end
-// ---------------------------------------------------------------------------
-
-template <bool kBatch>
-__global__ void __launch_bounds__(kThreads)
-k_gather_llr(const int32_t* __restrict__ rank, const int32_t* __restrict__ lcp, int32_t n, Scratch s, Segs segs) {
-    begin_after();
-    constexpr int kChunks = kTile / kWarp;          // 64 runs of 32 positions
-    constexpr int kWarps = kThreads / kWarp;        // 8
-    __shared__ int32_t Ls[kTile + 1];               // Ls[0] = L_{k0-1}, Ls[1+x] = L_{k0+x}
-    __shared__ int32_t chunk[kChunks];
-    __shared__ int32_t c_s[kTile];
-    __shared__ int32_t c_e[kTile];
-    __shared__ long long tile_s, base_s;
-    __shared__ int32_t total_s;
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) tile_s = atomicAdd(&s.tickets[0], 1u);
-    __syncthreads();
-    const long long tile = tile_s;
-    const long long k0 = tile * kTile;
-
-    // Lemma 1.  rank is streamed; the lcp pair goes through L1 (one sector
-    // for 7 of 8 rank values).  Invalid input is reported and clamped so
-    // every access stays in bounds.  In a batch, position k of string j has
-    // its local rank at rank[k] and the string's lcp at lcp[off[j] + j ..].
-    unsigned bad = 0;
-    __shared__ long long seg_sh[kBatch ? kSegCap + 1 : 1];
-    SegView sv{};
-    if constexpr (kBatch) {
-        const long long g1 = (k0 + kTile < n) ? k0 + kTile : n;
-        sv.stage(segs, s, k0 > 0 ? k0 - 1 : 0, g1, seg_sh);
-    }
-    long long hint = kBatch ? sv.j0 : 0;
-    auto llr = [&](long long k) -> int32_t {
-        uint32_t r = (uint32_t)__ldcs(rank + k);
-        long long base = 0, nj = n, lbase = 0;
-        if constexpr (kBatch) {
-            hint = sv.find(k, hint);
-            base = sv.at(hint);
-            nj = sv.at(hint + 1) - base;
-            lbase = base + hint;
-            if (base < 0 || nj < 1 || base + nj > n || k < base) { bad = 1; return 0; }   // bad offset table
-        }
-        if (r >= (uint32_t)nj) { bad = 1; r = 0; }
-        const int32_t a = __ldg(lcp + lbase + r), b = __ldg(lcp + lbase + r + 1);
-        if (kBatch && ((r == 0 && a != 0) || ((long long)r == nj - 1 && b != 0))) bad = 1;   // lcp sentinels
-        int32_t L = a > b ? a : b;
-        if (L < 0 || (long long)L > nj - (k - base)) { bad = 1; L = 0; }
-        return L;
-    };
-    if (tid == 0) {
-        Ls[0] = (k0 > 0) ? llr(k0 - 1) : 0;
-        if (!kBatch && tile == 0 && (__ldg(lcp) != 0 || __ldg(lcp + n) != 0)) bad = 1;
-    }
-    hint = kBatch ? sv.j0 : 0;
-    // All rank loads, then all lcp loads, then the lengths: every load of a
-    // thread is in flight before the first one is used.  A batch tile that
-    // lies inside one string does the same with that string's offsets and
-    // checks; other batch tiles look each position's string up.
-    long long sbase = 0, snj = n, slbase = 0;
-    bool direct = true;
-    if constexpr (kBatch) {
-        const long long g1 = (k0 + kTile < n) ? k0 + kTile : n;
-        const long long jk = sv.find(k0, sv.j0);
-        const long long b0 = sv.at(jk), b1 = sv.at(jk + 1);
-        direct = b0 >= 0 && b0 <= k0 && g1 <= b1 && b1 <= (long long)n;
-        sbase = b0;
-        snj = b1 - b0;
-        slbase = b0 + jk;
-    }
-    if (direct) {
-        constexpr int kPer = kTile / kThreads;
-        uint32_t r[kPer];
-        int32_t a[kPer], c[kPer];
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const long long k = k0 + j * kThreads + tid;
-            r[j] = (k < n) ? (uint32_t)__ldcs(rank + k) : 0u;
-        }
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const long long k = k0 + j * kThreads + tid;
-            if (k < n && (long long)r[j] >= snj) { bad = 1; r[j] = 0; }
-            a[j] = (k < n) ? __ldg(lcp + slbase + r[j]) : 0;
-            c[j] = (k < n) ? __ldg(lcp + slbase + r[j] + 1) : 0;
-        }
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int x = j * kThreads + tid;
-            const long long k = k0 + x;
-            int32_t L = a[j] > c[j] ? a[j] : c[j];
-            if (k < n) {
-                if (kBatch && ((r[j] == 0 && a[j] != 0) || ((long long)r[j] == snj - 1 && c[j] != 0))) bad = 1;
-                if (L < 0 || (long long)L > snj - (k - sbase)) { bad = 1; L = 0; }
-            }
-            Ls[1 + x] = (k < n) ? L : 0;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < kTile / kThreads; ++j) {
-            const int x = j * kThreads + tid;
-            Ls[1 + x] = (k0 + x < n) ? llr(k0 + x) : 0;
-        }
-    }
-    if (bad) report(s, kErrInput);
-    __syncthreads();
-
-    // K1 flags by warp ballots over runs of 32 positions, K2 within the tile.
-    unsigned masks[kChunks / kWarps];
-#pragma unroll
-    for (int q = 0; q < kChunks / kWarps; ++q) {
-        const int c = q * kWarps + warp;
-        const int x = c * kWarp + lane;
-        const int32_t L = Ls[1 + x], prev = Ls[x];
-        masks[q] = __ballot_sync(kFull, (k0 + x < n) && L > 0 && L >= prev);
-        if (lane == 0) chunk[c] = __popc(masks[q]);
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const int tot = warp_scan64(chunk);
-        if (lane == 0) total_s = tot;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kChunks / kWarps; ++q) {
-        const int c = q * kWarps + warp;
-        const int x = c * kWarp + lane;
-        if ((masks[q] >> lane) & 1u) {
-            const int o = chunk[c] + __popc(masks[q] & ((1u << lane) - 1u));
-            c_s[o] = (int32_t)(k0 + x);
-            c_e[o] = (int32_t)(k0 + x + Ls[1 + x] - 1);
-        }
-    }
-    // K3: the tile's place in LLRc.
-    if (warp == 0) {
-        const long long ex = lookback_exclusive(s.status_g, tile, total_s, s.err, s.qerr, s.spin_limit);
-        if (lane == 0) {
-            base_s = ex;
-            s.tile_cbase[tile] = (int32_t)ex;
-            if (tile == s.ntiles - 1) s.tile_cbase[s.ntiles] = (int32_t)(ex + total_s);
-        }
-    }
-    __syncthreads();
-    const long long base = base_s;
-    const int total = total_s;
-    // first LLRc entry of each kSeg-position segment of the tile
-    if (tid < kTile / kSeg) {
-        const long long sg = tile * (kTile / kSeg) + tid;
-        if (sg < s.nsegs) s.seg_cbase[sg] = (int32_t)(base + chunk[tid * (kSeg / kWarp)]);
-        if (sg == s.nsegs - 1) s.seg_cbase[s.nsegs] = (int32_t)(base + total);
-    }
-    for (int i = tid; i < total; i += kThreads) {
-        s.cstart[base + i] = c_s[i];
-        s.cend[base + i] = c_e[i];
-    }
-}
-
-void launch_gather_front(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
-                         cudaStream_t stream) {
-    if (segs.num > 0) launch_after(k_gather_llr<true>, (unsigned)s.ntiles, kThreads, 0, stream, rank, lcp, n, s, segs);
-    else k_gather_llr<false><<<(unsigned)s.ntiles, kThreads, 0, stream>>>(rank, lcp, n, s, segs);
 }
 
 // ---------------------------------------------------------------------------
@@ -734,7 +559,7 @@ k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t
 
 // Rank-window front end (rank without sa, one string of 2^24 positions or
 // more).  Lemma 1 in text order, max(lcp[rank[i]], lcp[rank[i] + 1]), makes
-// k_gather_llr read one random lcp sector per position from HBM.  Here
+// k_gather read one random lcp sector per position from HBM.  Here
 // k_rank_win first partitions the pairs <rank[i], i> by rank into windows
 // of 2^22 ranks (8-byte entries rank << 32 | i, in the compact LLR region,
 // which is idle until k_bucket_llr).  k_part1_win then takes kPartRound
@@ -1254,7 +1079,7 @@ constexpr uint32_t kDenseNone = 0xffffu;
 // What must be clear before the dense path: tickets and look-back words of
 // this n, and the dense array (kDenseNone); a batch's tile index as well.
 // One launch instead of two memsets and k_seg_index.
-__global__ void __launch_bounds__(256) k_prep(int32_t n, Scratch s, Segs segs) {
+__global__ void __launch_bounds__(256) k_prep(int32_t n, Scratch s, Segs segs, int fill) {
     begin_after();
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
     if (i0 < 8) s.tickets[i0] = 0;                // tickets and the query's error bits
@@ -1265,13 +1090,14 @@ __global__ void __launch_bounds__(256) k_prep(int32_t n, Scratch s, Segs segs) {
     }
     constexpr uint32_t kTwo = kDenseNone | (kDenseNone << 16);
     const uint4 none = make_uint4(kTwo, kTwo, kTwo, kTwo);
-    for (long long i = i0; i < ((long long)n + 7) / 8; i += step) reinterpret_cast<uint4*>(s.dense)[i] = none;
+    if (fill)
+        for (long long i = i0; i < ((long long)n + 7) / 8; i += step) reinterpret_cast<uint4*>(s.dense)[i] = none;
     if (segs.num > 0) seg_index(n, s, segs, i0, step);
 }
 
-void launch_prep(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream) {
-    const long long work = ((long long)n + 7) / 8, blocks = (work + 1023) / 1024;
-    k_prep<<<(unsigned)(blocks < 8 * kSms ? blocks : 8 * kSms), 256, 0, stream>>>(n, s, segs);
+void launch_prep(int32_t n, const Scratch& s, const Segs& segs, bool fill, cudaStream_t stream) {
+    const long long work = fill ? ((long long)n + 7) / 8 : s.ntiles, blocks = (work + 1023) / 1024;
+    k_prep<<<(unsigned)(blocks < 8 * kSms ? blocks : 8 * kSms), 256, 0, stream>>>(n, s, segs, fill ? 1 : 0);
 }
 
 template <bool kBatch>
@@ -1339,6 +1165,84 @@ __global__ void __launch_bounds__(kThreads) k_scatter(const int32_t* __restrict_
     if (bad) report(s, kErrInput);
 }
 
+// Lemma 1 in text order into the dense array (rank alone): rank is streamed,
+// the two lcp words of each position are gathered, all loads of a thread in
+// flight before the first is used; a tile across strings looks each
+// position's string up.  What bounds it is the rate of scattered sector reads
+// (1.1 per position).  6 x 10^6 positions of protein take 41 us here and 28 in
+// k_compact; in one kernel that also flagged, compacted and looked back per
+// 2048 positions, with 25 KB of shared memory, it was 71 us, and 180 instead
+// of 154 us for 1.6 x 10^7.
+template <bool kBatch>
+__global__ void __launch_bounds__(kThreads) k_gather(const int32_t* __restrict__ rank, const int32_t* __restrict__ lcp,
+                                                     int32_t n, Scratch s, Segs segs) {
+    begin_after();
+    constexpr int kPer = kTile / kThreads;
+    __shared__ long long seg_sh[kBatch ? kSegCap + 1 : 1];
+    const int tid = threadIdx.x;
+    const long long k0 = (long long)blockIdx.x * kTile;
+    long long base = 0, nj = n, lbase = 0, hint = 0;
+    bool direct = true;
+    SegView sv{};
+    if constexpr (kBatch) {
+        const long long k1 = (k0 + kTile < n) ? k0 + kTile : n;
+        sv.stage(segs, s, k0, k1, seg_sh);
+        hint = sv.find(k0, sv.j0);
+        base = sv.at(hint);
+        const long long end = sv.at(hint + 1);
+        nj = end - base;
+        lbase = base + hint;
+        direct = base >= 0 && base <= k0 && k1 <= end && end <= (long long)n;
+    }
+    // Invalid input is reported and clamped so every access stays in bounds.
+    unsigned bad = 0;
+    if (!kBatch && blockIdx.x == 0 && tid == 0 && (__ldg(lcp) != 0 || __ldg(lcp + n) != 0)) bad = 1;
+    auto put = [&](long long k, int32_t a, int32_t b, long long at, long long len) {
+        int32_t L = a > b ? a : b;
+        if (L < 0 || (long long)L > len - (k - at)) { bad = 1; L = 0; }
+        uint32_t w = (uint32_t)L;
+        if (w >= kDenseEsc) { w = kDenseEsc; s.lbig[k] = L; }
+        s.dense[k] = (uint16_t)w;
+    };
+    if (direct) {
+        uint32_t r[kPer];
+        int32_t a[kPer], b[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const long long k = k0 + j * kThreads + tid;
+            r[j] = (k < n) ? (uint32_t)__ldcs(rank + k) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const long long k = k0 + j * kThreads + tid;
+            if (k < n && (long long)r[j] >= nj) { bad = 1; r[j] = 0; }
+            a[j] = (k < n) ? __ldg(lcp + lbase + r[j]) : 0;
+            b[j] = (k < n) ? __ldg(lcp + lbase + r[j] + 1) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const long long k = k0 + j * kThreads + tid;
+            if (k >= n) continue;
+            if (kBatch && ((r[j] == 0 && a[j] != 0) || ((long long)r[j] == nj - 1 && b[j] != 0))) bad = 1;   // lcp sentinels
+            put(k, a[j], b[j], base, nj);
+        }
+    } else {
+        for (int j = 0; j < kPer; ++j) {
+            const long long k = k0 + j * kThreads + tid;
+            if (k >= n) continue;
+            hint = sv.find(k, hint);
+            const long long at = sv.at(hint), len = sv.at(hint + 1) - at;
+            if (at < 0 || len < 1 || at + len > n || k < at) { bad = 1; s.dense[k] = 0; continue; }   // bad offset table
+            uint32_t r = (uint32_t)__ldcs(rank + k);
+            if ((long long)r >= len) { bad = 1; r = 0; }
+            const int32_t a = __ldg(lcp + at + hint + r), b = __ldg(lcp + at + hint + r + 1);
+            if ((r == 0 && a != 0) || ((long long)r == len - 1 && b != 0)) bad = 1;   // lcp sentinels
+            put(k, a, b, at, len);
+        }
+    }
+    if (bad) report(s, kErrInput);
+}
+
 struct DenseWords {
     static constexpr uint32_t kEsc = kDenseEsc;
     const uint16_t* d;                            // of the tile's first position
@@ -1383,6 +1287,12 @@ __global__ void __launch_bounds__(kCompactThreads) k_compact(int32_t n, Scratch 
 void launch_scatter(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                     cudaStream_t stream) {
     launch_after(segs.num > 0 ? k_scatter<true> : k_scatter<false>, (unsigned)s.ntiles, kThreads, 0, stream, sa, lcp, n, s,
+                 segs);
+}
+
+void launch_gather(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
+                   cudaStream_t stream) {
+    launch_after(segs.num > 0 ? k_gather<true> : k_gather<false>, (unsigned)s.ntiles, kThreads, 0, stream, rank, lcp, n, s,
                  segs);
 }
 

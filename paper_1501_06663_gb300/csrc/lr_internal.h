@@ -7,7 +7,7 @@
 
 namespace lr {
 
-// Tiles of the gather front end (and the granularity of tile_cbase).
+// Tiles of the gather and scatter kernels (and the granularity of tile_cbase).
 constexpr int kTile = 2048;          // positions per tile (one CTA)
 constexpr int kThreads = 256;        // threads per tile CTA
 // Tiles of the tile cover kernel: kTile x (1, 2 or 4) positions, kThreads x the same threads.
@@ -61,10 +61,10 @@ constexpr int kSpinLimit = 1 << 23;
 
 // Device scratch of one query, carved out of one allocation by the context.
 struct Scratch {
-    unsigned* tickets;             // [0] gather tiles, [1] buckets, [2] cover tiles
+    unsigned* tickets;             // [1] buckets or dense tiles, [2] cover tiles
     unsigned* qerr;                // error bits of this query (cleared with the tickets)
     unsigned* err;                 // sticky device error bits (kErr*), read by the host
-    unsigned long long* status_g;  // look-back words of the gather front end (per tile)
+    unsigned long long* status_g;  // look-back words of the dense front end (per tile of kCompactTile)
     unsigned long long* status_b;  // look-back words of the rank-order front end (per bucket)
     unsigned long long* status_o;  // look-back words of the cover kernel (per cover tile)
     int32_t* tile_cbase;           // ntiles + 1: compact LLR's starting before tile j
@@ -74,7 +74,8 @@ struct Scratch {
     uint32_t* ent2;                // nbuckets x 2^15: the same entries by bucket of 2^15 positions
     unsigned* cursor1;             // fill counts of ent1, one per kCursorStride words (cleared per query)
     unsigned* cursor2;             // fill counts of ent2, one per kCursorStride words (cleared per query)
-    uint16_t* dense;               // n: lengths in text order of the dense front end (in the ent1 region)
+    uint16_t* dense;               // n: lengths in text order of the dense front end (in the ent1 region; up to
+                                   // a multiple of kCompactTile is read)
     int32_t* lbig;                 // n: L of positions whose length field escaped
     int32_t* halo;                 // nbuckets + 1: L of the position before each bucket
     int32_t* tile_seg;             // ntiles: first string overlapping each tile (batched queries)
@@ -156,15 +157,16 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
 
 // Front ends (lr_front.cu) and the cover kernel (lr_cover.cu).
 void launch_seg_index(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream);
-void launch_gather_front(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
-                         cudaStream_t stream);
 void launch_partition(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                       cudaStream_t stream);
-// the dense front end: k_prep, k_scatter, k_compact
-// k_prep clears what the dense path needs cleared and, for a batch, does k_seg_index's work
-void launch_prep(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream);
+// The dense front end: k_prep clears what it needs cleared (with `fill` the
+// dense array too) and, for a batch, does k_seg_index's work; k_scatter (sa) or
+// k_gather (rank) fills the array, k_compact compacts it.
+void launch_prep(int32_t n, const Scratch& s, const Segs& segs, bool fill, cudaStream_t stream);
 void launch_scatter(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                     cudaStream_t stream);
+void launch_gather(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
+                   cudaStream_t stream);
 void launch_compact(int32_t n, const Scratch& s, cudaStream_t stream);
 // k_one_tile: the whole query of a string of at most kOneTileMax positions
 void launch_one_tile(const int32_t* sa, const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s,

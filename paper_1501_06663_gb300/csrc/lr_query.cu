@@ -37,32 +37,23 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
         if (events) events->count = k;
         return cudaGetLastError();
     }
-    const bool dense = sa && (long long)n <= (segs.num > 0 ? kDenseMaxBatch : kDenseMaxN);
-    if (!dense) {
+    const bool rankwin = !sa && segs.num == 0 && s.cursor_w && (long long)n >= kRankWinMinN;
+    const bool dense = sa ? (long long)n <= (segs.num > 0 ? kDenseMaxBatch : kDenseMaxN) : !rankwin;
+    mark();
+    if (dense) {
+        launch_prep(n, s, segs, sa != nullptr, stream);             // k_prep
+        if (sa) launch_scatter(sa, lcp, n, s, segs, stream);        // k_scatter
+        else launch_gather(rank, lcp, n, s, segs, stream);          // k_gather
+        mark();
+        launch_compact(n, s, stream);                               // k_compact
+    } else {
         cudaError_t e = cudaMemsetAsync(s.zero_base, 0, s.zero_bytes, stream);
         if (e != cudaSuccess) return e;
-        if (segs.num > 0) launch_seg_index(n, s, segs, stream);                 // k_seg_index
-    }
-    const bool rankwin = !sa && segs.num == 0 && s.cursor_w && (long long)n >= kRankWinMinN;
-    if (dense) {
+        if (segs.num > 0) launch_seg_index(n, s, segs, stream);     // k_seg_index
+        if (sa) launch_partition(sa, lcp, n, s, segs, stream);      // k_part1, k_part2
+        else launch_rank_window_front(rank, lcp, n, s, stream);     // k_rank_win, k_part1_win, k_part2
         mark();
-        launch_prep(n, s, segs, stream);                    // k_prep
-        launch_scatter(sa, lcp, n, s, segs, stream);        // k_scatter
-        mark();
-        launch_compact(n, s, stream);                       // k_compact
-    } else if (sa) {
-        mark();
-        launch_partition(sa, lcp, n, s, segs, stream);      // k_part1, k_part2
-        mark();
-        launch_bucket_front(n, s, stream);                  // k_bucket_llr
-    } else if (rankwin) {
-        mark();
-        launch_rank_window_front(rank, lcp, n, s, stream);  // k_rank_win, k_part1_win, k_part2
-        mark();
-        launch_bucket_front(n, s, stream);                  // k_bucket_llr
-    } else {
-        mark();
-        launch_gather_front(rank, lcp, n, s, segs, stream); // k_gather_llr
+        launch_bucket_front(n, s, stream);                          // k_bucket_llr
     }
     mark();
     if (shape.tile_cover)
@@ -70,7 +61,7 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
     else
         launch_cover_w(n, s, lr_len, lr_start, offsets, starts, capacity, all, stream);
     if (timed) cudaEventRecord(events->ev[k], stream);
-    if (launches) *launches = dense ? 4 : (sa ? 4 : (rankwin ? 5 : 2)) + (segs.num > 0 ? 1 : 0);
+    if (launches) *launches = dense ? 4 : (sa ? 4 : 5) + (segs.num > 0 ? 1 : 0);
     if (events) events->count = k;
     return cudaGetLastError();
 }

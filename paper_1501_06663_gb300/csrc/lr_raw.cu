@@ -244,9 +244,10 @@ cudaError_t launch_raw_query(const int32_t* rank, const int32_t* lcp, int32_t n,
 
 cudaError_t launch_walk_stats(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, int32_t* alpha,
                               int32_t* beta, unsigned long long* stats, cudaStream_t stream) {
-    cudaError_t e = cudaMemsetAsync(s.zero_base, 0, s.zero_bytes, stream);
-    if (e != cudaSuccess) return e;
-    launch_gather_front(rank, lcp, n, s, Segs{nullptr, 0}, stream);       // LLRc in s.cstart / s.cend
+    const Segs one{nullptr, 0};
+    launch_prep(n, s, one, false, stream);
+    launch_gather(rank, lcp, n, s, one, stream);
+    launch_compact(n, s, stream);                                         // LLRc in s.cstart / s.cend
     int32_t* llrr = s.lbig;
     k_llr_raw<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rank, lcp, n, s, llrr);
     k_stats_init<<<1, 1, 0, stream>>>(stats);

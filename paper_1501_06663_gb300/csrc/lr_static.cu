@@ -21,12 +21,13 @@ constexpr long long kSegsMax = (kStaticMaxN + lr::kSeg - 1) / lr::kSeg;
 constexpr size_t kOffStatusG = kAlignS;                   // [0, 256): tickets, per-query and sticky error bits
 constexpr size_t kOffStatusO = align_s(kOffStatusG + (size_t)kTilesMax * 8);
 constexpr size_t kOffStatusW = align_s(kOffStatusO + (size_t)kTilesMax * 8);
-constexpr size_t kZeroEnd = kOffStatusW + (size_t)((kStaticMaxN + lr::kSegTile - 1) / lr::kSegTile) * 8;
-constexpr size_t kOffCbase = align_s(kZeroEnd);
+constexpr size_t kOffCbase = align_s(kOffStatusW + (size_t)((kStaticMaxN + lr::kSegTile - 1) / lr::kSegTile) * 8);
 constexpr size_t kOffSegCbase = align_s(kOffCbase + (size_t)(kTilesMax + 1) * 4);
 constexpr size_t kOffCstart = align_s(kOffSegCbase + (size_t)(kSegsMax + 1) * 4);
 constexpr size_t kOffCend = align_s(kOffCstart + (size_t)kStaticMaxN * 4);
-constexpr size_t kStaticBytes = align_s(kOffCend + (size_t)kStaticMaxN * 4);   // about 8.1 MB
+constexpr size_t kOffDense = align_s(kOffCend + (size_t)kStaticMaxN * 4);
+constexpr size_t kStaticBytes = align_s(kOffDense + (size_t)kStaticMaxN * 2);   // about 10.1 MB
+static_assert(kStaticMaxN % lr::kCompactTile == 0, "whole tiles of the dense array");
 
 // The array itself.  Host code must not use its name as an address: it is a
 // host-side stand-in.  The device address comes from cudaGetSymbolAddress.
@@ -76,15 +77,16 @@ extern "C" lr_status lr_query_all_static(lr_stream_t stream, const int32_t* d_ra
     s.seg_cbase = reinterpret_cast<int32_t*>(b + kOffSegCbase);
     s.cstart = reinterpret_cast<int32_t*>(b + kOffCstart);
     s.cend = reinterpret_cast<int32_t*>(b + kOffCend);
+    s.dense = reinterpret_cast<uint16_t*>(b + kOffDense);
+    s.lbig = d_lr_len;                    // read before the cover kernel writes its lengths there
     s.ntiles = lr::num_tiles(n);
     s.nsegs = lr::num_segs(n);
-    // what every query must find at zero: tickets, both error words, the
-    // look-back words of both kernels (one memset, no allocation)
-    s.zero_base = b;
-    s.zero_bytes = kZeroEnd;
+    // the error words start at zero (k_prep clears the rest)
     cudaStream_t strm = (cudaStream_t)stream;
-    cudaError_t e = lr::launch_query(nullptr, d_rank, d_lcp, n, s, d_lr_len, d_lr_start, d_offsets, d_starts,
-                                     starts_capacity, true, strm, nullptr, nullptr);
+    cudaError_t e = cudaMemsetAsync(b, 0, kAlignS, strm);
+    if (e == cudaSuccess)
+        e = lr::launch_query(nullptr, d_rank, d_lcp, n, s, d_lr_len, d_lr_start, d_offsets, d_starts, starts_capacity,
+                             true, strm, nullptr, nullptr);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LR_ERR_NOMEM : LR_ERR_CUDA;
     if (!h_total) return LR_OK;
     unsigned bits = 0;
