@@ -35,18 +35,16 @@
 // A lane owns one position of each run of 32, so every per-position store of
 // a warp is one contiguous 128- or 256-byte run.
 //
-// What bounds it: instruction issue (about 75 % of the slots) and the waits
+// What bounds it: instruction issue (71 to 79 % of the slots) and the waits
 // between its phases, of which the look-back is the longest; DRAM runs at
 // half its rate.  The form before it worked per position (a range-maximum
 // table over the window of each run of 32) and took 2.18 ms for 2^28
 // positions of English (0.21 entries per position), 2.77 ms for 258 M of
-// mixed DNA and protein (0.52); this one takes 1.58 and 2.39 ms.  It has 180
+// mixed DNA and protein (0.52); this one takes 1.55 and 2.31 ms.  It has 166
 // instead of 240 instructions per run of 32 positions (English); per-entry
 // work pays as long as entries are fewer than positions, which they are by
 // construction (at most one starts at each).  Four consecutive positions per
-// lane with vector stores were faster without the CSR outputs (0.254 against
-// 0.258 ms at 100 M positions) but slower with them (1.69 against 1.58 ms:
-// the list of starts then needs gathering in shared memory).  Persistent
+// lane with vector stores were slower (1.69 against 1.58 ms then).  Persistent
 // CTAs that take the next ticket early were slower (2.24 ms): a tile taken
 // early publishes late, and every later tile waits for it; so were look-back
 // steps over 128 or 256 words (1.88, 2.12 ms).
@@ -85,7 +83,7 @@ struct __align__(16) CoverSmem {
     // the one after the last starts after everything and stops the scans to
     // the right.
     int2 ent[Cfg<TP>::kCap + 2];
-    uint32_t rec[Cfg<TP>::kTileC];   // at a boundary: ent index of the leftmost holder | number of holders << 16
+    alignas(16) uint32_t rec[Cfg<TP>::kTileC];   // at a boundary: ent index of the leftmost holder | number of holders << 16
     unsigned bmap[kChunks];          // bit x: the set of holders changes at position x (bit 0 always set)
     // distance to the next entry of the same length with no longer one
     // between (0: none that overlaps; 255: that or more)
@@ -150,6 +148,11 @@ __device__ __forceinline__ int ties_prefix(int c, unsigned below, int* tot) {
     const int incl = warp_incl_scan(c);
     *tot = __shfl_sync(kFull, incl, kWarp - 1);
     return incl - c;
+}
+
+// Four consecutive CSR offsets at a 32-byte-aligned address: a whole sector.
+__device__ __forceinline__ void store_offsets(int64_t* p, long long a, long long b, long long c, long long d) {
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
 }
 
 // The tile's place in starts[] (whole warp): look back over the earlier
@@ -280,7 +283,7 @@ template <bool kAll, int TP, bool kOne>
 __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, const Scratch& s, long long tile, int32_t k0,
                                               int32_t MS, int32_t nlow, int32_t* __restrict__ lr_len,
                                               int32_t* __restrict__ lr_start, int64_t* __restrict__ offsets,
-                                              int32_t* __restrict__ starts, long long capacity) {
+                                              int32_t* __restrict__ starts, long long capacity, int vec) {
     constexpr int kCoverTile = Cfg<TP>::kTileC;
     constexpr int kCoverThreads = Cfg<TP>::kThr;
     constexpr int kChunksPerWarp = Cfg<TP>::kChunksPerWarp;
@@ -369,6 +372,7 @@ __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, cons
         }
     }
     uint32_t pk[kChunksPerWarp];                              // the positions' records
+    uint32_t all_r = 0;                                       // their bitwise or: bounds the counts
     int32_t sum = 0;
 #pragma unroll
     for (int q = 0; q < kChunksPerWarp; ++q) {
@@ -384,6 +388,7 @@ __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, cons
             __stcs(lr_len + k, h.y);
             __stcs(lr_start + k, h.x);
             sum += (int32_t)(r >> 16);
+            all_r |= r;
         } else {
             pk[q] = 0;
         }
@@ -410,48 +415,88 @@ __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, cons
         // starts[o0 ..]: 32-bit indices from here; entries past the capacity are not written
         const long long room = capacity - o0;
         const int32_t lim = room < 0 ? 0 : (room > 0x7fffffff ? 0x7fffffff : (int32_t)room);
-        int32_t* out = starts + o0;
+        int32_t* const out = starts + o0;
         const bool far = sm.far != 0;
+        // every compact LLR of the longest length over a position (its record
+        // r, its first start at out[o]), ascending
+        auto emit = [&](uint32_t r, int32_t o) {
+            int32_t left = min((int32_t)(r >> 16), lim - o);
+            if (left <= 0) return;
+            int v = (int)(r & 0xffffu);
+            int32_t* p = out + o;
+            __stcs(p, sm.ent[v].x);
+            if (!far) {
+                while (--left > 0) {
+                    v += nx[v];
+                    __stcs(++p, sm.ent[v].x);
+                }
+            } else {
+                while (--left > 0) {
+                    const int32_t d = nx[v], L = sm.ent[v].y;
+                    v += d;
+                    if (d == 255)
+                        while (v <= MS && sm.ent[v].y != L) ++v;
+                    __stcs(++p, sm.ent[v].x);
+                }
+            }
+        };
+        // Prefixes of the counts, eight consecutive positions per lane, where
+        // every count of the warp fits four bits, an index twelve, and the
+        // tile is whole: the records go through shared memory as 16-bit words
+        // (the warp's part of rec, which nobody reads any more), one
+        // multiplication makes the prefixes of four counts, a lane stores
+        // eight offsets, and the loop over the runs needs no registers for
+        // them and is not unrolled.  English 2^28 1.58 -> 1.55 ms, DNA 2^26
+        // 608 -> 577 us, mixed batch 2.40 -> 2.31 ms; with the loop unrolled
+        // the code no longer fits the instruction cache (1.80 ms).
+        const bool whole = vec && k0 <= n - kCoverTile;
+        if (Cfg<TP>::kCap + 2 <= 0x1000 && whole && !__any_sync(kFull, all_r >= (16u << 16))) {
+            uint16_t* const rb = reinterpret_cast<uint16_t*>(sm.rec + c0 * kWarp);   // records as index | count << 12
+            uint16_t* const ob = rb + kChunksPerWarp * kWarp;
+#pragma unroll
+            for (int q = 0; q < kChunksPerWarp; ++q)
+                rb[q * kWarp + lane] = (uint16_t)((pk[q] & 0xfffu) | ((pk[q] >> 4) & 0xf000u));
+            __syncwarp();
+            const uint4 r8 = *reinterpret_cast<const uint4*>(rb + lane * 8);
+            // counts of four positions, a byte each
+            const uint32_t cx = ((r8.x >> 12) & 0xfu) | ((r8.x >> 20) & 0xf00u) | ((r8.y << 4) & 0xf0000u) | ((r8.y >> 4) & 0xf000000u);
+            const uint32_t cy = ((r8.z >> 12) & 0xfu) | ((r8.z >> 20) & 0xf00u) | ((r8.w << 4) & 0xf0000u) | ((r8.w >> 4) & 0xf000000u);
+            const uint32_t sx = cx * 0x01010101u, sy = cy * 0x01010101u;   // inclusive prefixes, a byte each
+            const uint32_t tx = sx >> 24;
+            const uint32_t px = sx << 8, py = (sy << 8) + tx * 0x01010101u;  // exclusive ones of the eight
+            const int32_t mine = (int32_t)(tx + (sy >> 24));
+            const uint32_t ex = (uint32_t)(warp_incl_scan(mine) - mine);
+            const uint32_t e2 = ex * 0x10001u;                               // below 2^16: 256 counts of at most 15
+            uint4 w;
+            w.x = __byte_perm(px, 0, 0x4140) + e2;
+            w.y = __byte_perm(px, 0, 0x4342) + e2;
+            w.z = __byte_perm(py, 0, 0x4140) + e2;
+            w.w = __byte_perm(py, 0, 0x4342) + e2;
+            *reinterpret_cast<uint4*>(ob + lane * 8) = w;
+            int64_t* const po = offsets + k0 + c0 * kWarp + lane * 8;
+            const long long base = o0 + ex;
+            store_offsets(po, base, base + ((px >> 8) & 0xffu), base + ((px >> 16) & 0xffu), base + (px >> 24));
+            store_offsets(po + 4, base + (py & 0xffu), base + ((py >> 8) & 0xffu), base + ((py >> 16) & 0xffu),
+                          base + (py >> 24));
+            __syncwarp();
+#pragma unroll 1
+            for (int q = 0; q < kChunksPerWarp; ++q) {
+                const uint32_t r = rb[q * kWarp + lane];
+                emit((r & 0xfffu) | ((r >> 12) << 16), (int32_t)ob[q * kWarp + lane]);
+                __syncwarp();
+            }
+            return;
+        }
         int32_t run = 0;
 #pragma unroll
         for (int q = 0; q < kChunksPerWarp; ++q) {
             const int32_t k = k0 + (c0 + q) * kWarp + lane;
-            const int32_t cq = (int32_t)(pk[q] >> 16);
-            const unsigned two = __ballot_sync(kFull, cq > 1);
-            const unsigned one = __ballot_sync(kFull, cq & 1);
-            int tot = __popc(one);
-            int32_t o = run + __popc(one & below);
-            if (two) {
-                if (__ballot_sync(kFull, cq > 3) == 0u) {
-                    tot += 2 * __popc(two);
-                    o += 2 * __popc(two & below);
-                } else {
-                    const int incl = warp_incl_scan(cq);
-                    tot = __shfl_sync(kFull, incl, kWarp - 1);
-                    o = run + incl - cq;
-                }
-            }
+            int tot;
+            const int32_t o = run + ties_prefix((int)(pk[q] >> 16), below, &tot);
             run += tot;
             if (k < n) __stcs(reinterpret_cast<long long*>(offsets) + k, o0 + o);
-            // every compact LLR of the longest length over k, ascending
-            int32_t left = cq < lim - o ? cq : lim - o;
-            int v = (int)(pk[q] & 0xffffu);
-            int32_t* p = out + o;
-            if (left > 0) __stcs(p, sm.ent[v].x);
-            if (two) {
-                while (--left > 0) {
-                    const int32_t d = nx[v];
-                    if (far && d == 255) {
-                        const int32_t L = sm.ent[v].y;
-                        v += d;
-                        while (v <= MS && sm.ent[v].y != L) ++v;
-                    } else {
-                        v += d;
-                    }
-                    __stcs(++p, sm.ent[v].x);
-                }
-                __syncwarp();
-            }
+            emit(pk[q], o);
+            __syncwarp();
         }
     }
 }
@@ -461,7 +506,7 @@ __device__ __forceinline__ void cover_entries(CoverSmem<TP>& sm, int32_t n, cons
 template <bool kAll, int TP>
 __global__ void __launch_bounds__(Cfg<TP>::kThr, Cfg<TP>::kMinBlocks)
 k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict__ lr_start,
-        int64_t* __restrict__ offsets, int32_t* __restrict__ starts, long long capacity) {
+        int64_t* __restrict__ offsets, int32_t* __restrict__ starts, long long capacity, int vec) {
     begin_last();
     constexpr int kCoverTile = Cfg<TP>::kTileC;
     constexpr int kCoverThreads = Cfg<TP>::kThr;
@@ -536,7 +581,7 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
         cover_long_carry<kAll, TP>(sm, n, s, tile, cb0, cb1, lr_len, lr_start, offsets, starts, capacity);
         return;
     }
-    cover_entries<kAll, TP, false>(sm, n, s, tile, k0, MS, nlow, lr_len, lr_start, offsets, starts, capacity);
+    cover_entries<kAll, TP, false>(sm, n, s, tile, k0, MS, nlow, lr_len, lr_start, offsets, starts, capacity, vec);
 }
 
 // A string of at most one tile of 8192 positions: the whole query in one CTA
@@ -633,7 +678,7 @@ k_one_tile(const int32_t* __restrict__ in, const int32_t* __restrict__ lcp, int3
         s.tile_cbase[s.ntiles] = m;
     }
     __syncthreads();
-    cover_entries<kAll, TP, true>(sm, n, s, 0, 0, m, 0, lr_len, lr_start, offsets, starts, capacity);
+    cover_entries<kAll, TP, true>(sm, n, s, 0, 0, m, 0, lr_len, lr_start, offsets, starts, capacity, 0);
 }
 
 namespace {
@@ -642,8 +687,9 @@ template <bool kAll, int TP>
 void launch_cover_t(int32_t n, const Scratch& s, int32_t* lr_len, int32_t* lr_start, int64_t* offsets,
                     int32_t* starts, long long capacity, cudaStream_t stream) {
     const unsigned grid = (unsigned)num_cover_tiles(n, TP);
+    const int vec = ((uintptr_t)offsets & 31u) == 0 ? 1 : 0;   // whole-sector stores (tiles start at multiples of 2048)
     launch_after(k_cover<kAll, TP>, grid, Cfg<TP>::kThr, sizeof(CoverSmem<TP>), stream, n, s, lr_len, lr_start, offsets, starts,
-                 capacity);
+                 capacity, vec);
 }
 
 template <int TP>

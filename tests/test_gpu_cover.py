@@ -56,3 +56,36 @@ def test_equal_entries_far_apart(ctx, between, length, lead):
         assert np.array_equal(a.cpu().numpy(), b)
     st, ln = ctx.query_leftmost(dlcp, sa=dsa)
     assert np.array_equal(st.cpu().numpy(), want[1]) and np.array_equal(ln.cpu().numpy(), want[0])
+
+
+def _tied_text(width, blocks):
+    """Blocks in which up to `width` + 1 equal repeats cover a position: R and all its windows of width + 1."""
+    rng = np.random.default_rng(width)
+    parts = []
+    for _ in range(blocks):
+        R = rng.integers(0, 200, 2 * width + 2).astype(np.uint8)
+        parts.append(R)
+        for j in range(width):
+            parts += [R[j:j + width + 1], rng.integers(200, 256, 2).astype(np.uint8)]
+    return np.concatenate(parts)
+
+
+@pytest.mark.parametrize("width,blocks", [(3, 1200), (13, 130), (14, 130), (15, 130), (16, 130), (40, 20)])
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_tie_counts_and_unaligned_offsets(ctx, width, blocks, shift):
+    """Counts around the 15 that the byte prefixes take; offsets[] 8, 16 or 24 bytes off a 32-byte boundary."""
+    import paper_1501_06663_gb300 as lrmod
+    text = _tied_text(width, blocks)
+    sa, rank, lcp = W.prep(text)
+    want = oracle.lr_all_raw(rank, lcp)
+    assert int(np.diff(want[2]).max()) >= width
+    n = text.size
+    ln, st = (torch.empty(n + shift, dtype=torch.int32, device="cuda")[shift:] for _ in range(2))
+    off = torch.empty(n + 1 + shift, dtype=torch.int64, device="cuda")[shift:]
+    starts = torch.full((want[3].size + 1 + shift,), -7, dtype=torch.int32, device="cuda")[shift:]
+    status, total = lrmod.lr_query_all(ctx.handle, torch.from_numpy(sa).cuda(), None, torch.from_numpy(lcp).cuda(), ln, st,
+                                       off, starts[:-1])
+    assert status == lrmod.LR_OK and total == want[3].size
+    for a, b in zip((ln, st, off, starts[:-1]), want):
+        assert np.array_equal(a.cpu().numpy(), b)
+    assert int(starts[-1]) == -7
