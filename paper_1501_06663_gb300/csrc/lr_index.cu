@@ -32,7 +32,7 @@
 //
 // What bounds it: the radix sorts (CUB; two thirds of the time), then the
 // scattered rank stores and the lookups of k_lcp.  2^25 + 1 positions of
-// English take 7.9 ms and 2^28 73 ms; 10.5 and 89.7 ms with the suffix array
+// English take 7.3 ms and 2^28 70 ms; 10.5 and 89.7 ms with the suffix array
 // sorted once more from the final ranks, round 0's ranks sorted back to
 // position order at any size, separate marks, max-scans and updates, the
 // actives selected from all positions every round, keys of 32 + 26 instead of
@@ -281,12 +281,47 @@ k_rank0(const uint64_t* __restrict__ key, const int32_t* __restrict__ val, long 
     }
 }
 
+// rank[val[i]] = word[i] for i < count, window by window of 2^kWinPos positions
+// (blocks in window order, each reading the pairs once more and storing those
+// of its window), so that the stores merge in L2: 2^25 stores into one
+// 134 MB array run at 45 G/s, into 64 MB of it at 130.
+constexpr int kWinPos = 24;
+__global__ void __launch_bounds__(kGrpThreads)
+k_scatter_words(const int32_t* __restrict__ val, const int32_t* __restrict__ word, long long count,
+                int32_t* __restrict__ rank, unsigned per_window) {
+    const int w = (int)(blockIdx.x / per_window);
+    const long long i0 = (long long)(blockIdx.x % per_window) * kGrpTile;
+    if (i0 + kGrpTile <= count) {
+        int4 v[2], x[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const long long i = i0 / 4 + u * kGrpThreads + threadIdx.x;
+            v[u] = __ldcs(reinterpret_cast<const int4*>(val) + i);
+            x[u] = __ldcs(reinterpret_cast<const int4*>(word) + i);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if ((v[u].x >> kWinPos) == w) rank[v[u].x] = x[u].x;
+            if ((v[u].y >> kWinPos) == w) rank[v[u].y] = x[u].y;
+            if ((v[u].z >> kWinPos) == w) rank[v[u].z] = x[u].z;
+            if ((v[u].w >> kWinPos) == w) rank[v[u].w] = x[u].w;
+        }
+    } else {
+        for (long long i = i0 + threadIdx.x; i < count; i += kGrpThreads) {
+            const int32_t v = __ldcs(val + i);
+            if ((v >> kWinPos) == w) rank[v] = __ldcs(word + i);
+        }
+    }
+}
+
 // Round r >= 1, over the re-sorted keys key[0..A) (halves of sb bits): an old
 // group (rank g0 = its first sorted index) holds its re-sorted members at
 // a0 .. a0 + size - 1, so member a sits at sorted index g0 + a - a0 and its
 // new rank is the index of its new group's first member, g0 + ah - a0, with
 // the active bit when the new group has two or more members.  New group
-// starts inside an old group take sep = r.
+// starts inside an old group take sep = r.  The rank words go to their
+// positions (kScatter) or stay in key order.
+template <bool kScatter>
 __global__ void __launch_bounds__(kGrpThreads)
 k_update(const uint64_t* __restrict__ key, const int32_t* __restrict__ val, long long A, int sb,
          int32_t* __restrict__ rank, int32_t* __restrict__ sa, uint8_t* __restrict__ sep, int round) {
@@ -326,7 +361,8 @@ k_update(const uint64_t* __restrict__ key, const int32_t* __restrict__ val, long
         const long long g0 = old[u], s0 = group_start(om, t0, x), hh = group_start(nm, t0, x);
         const bool nh = starts_group(nm, x), act = !(nh && starts_group(nm, x + 1));
         const int32_t v = __ldg(val + a);
-        rank[v] = (int32_t)((uint32_t)(g0 + (hh - s0)) | (act ? kActiveBit : 0u));
+        const int32_t word = (int32_t)((uint32_t)(g0 + (hh - s0)) | (act ? kActiveBit : 0u));
+        if (kScatter) rank[v] = word; else rank[a] = word;
         sa[g0 + (a - s0)] = v;
         if (nh && s0 != a) sep[g0 + (a - s0)] = (uint8_t)round;
     }
@@ -406,12 +442,17 @@ size_t sort_temp_bytes(long long n) {
     return (c > a ? c : a) + 256;
 }
 
-// Positions up to which round 0's ranks are scattered straight to position
-// order, while most of their 4-byte array stays in the 129 MB L2: at 2^25
-// positions the build takes 7.85 ms this way and 8.03 ms with the sort by
-// position; scattered 4-byte stores past L2 run at 27 G/s (10 ms for 2^28,
-// the sort 5).
-constexpr long long kScatterMax = 40LL << 20;
+// Which way rank words go to position order: straight while their array
+// (kDirectPos positions) stays in the 129 MB L2, or for few of them; else
+// window by window, W windows of 2^kWinPos positions, up to kScatterWins
+// (kUpdateWins after round 0); above, round 0's by a radix sort keyed by
+// position and later ones straight.  Per word the windows cost 1.2 ps each
+// (reading the pairs again) and 8 ps for the stores, the sort 24 ps, stores
+// past L2 30 ps.  The build of 2^25 + 1 positions of English takes 7.29 ms
+// with windows and 7.85 straight, of 30 M mixed positions 6.52 and 6.32; 10^8
+// positions of English 22.0 and (with the sort) 25.0.
+constexpr long long kDirectPos = 30LL << 20, kDirectWords = 1LL << 18;
+constexpr long long kScatterWins = 13, kUpdateWins = 19;
 
 inline size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -507,22 +548,31 @@ cudaError_t build_arrays_batch(const uint8_t* text, long long total, const int64
     size_t tb = w.tmp_bytes;
     e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, keys, vals, (int)total, 0, jobbits + bps * csyms, stream);
     if (e != cudaSuccess) return e;
-    // The suffix array is kept in sa (flattened) from here on.  The ranks go
-    // back to position order by scattered stores while their array fits L2,
-    // else by a radix sort keyed by position (streaming passes)
-    if (total <= kScatterMax) {
+    // The suffix array is kept in sa (flattened) from here on
+    const long long wins = (total + (1LL << kWinPos) - 1) >> kWinPos;
+    auto scatter_words = [&](const int32_t* val, const int32_t* word, long long count, int32_t* rank_out) {
+        const unsigned per = blocks(count, kGrpTile);
+        k_scatter_words<<<(unsigned)(wins * per), kGrpThreads, 0, stream>>>(val, word, count, rank_out, per);
+    };
+    const bool direct = total <= kDirectPos;
+    if (direct) {
         k_rank0<true><<<blocks(total, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), total,
                                                                           bps * csyms, bps, w.levels, sa, w.sep, lcp);
     } else {
+        int32_t* words = wins <= kScatterWins ? reinterpret_cast<int32_t*>(keys.Alternate()) : w.hp;
         k_rank0<false><<<blocks(total, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), total,
-                                                                           bps * csyms, bps, w.hp, sa, w.sep, lcp);
-        cub::DoubleBuffer<int32_t> pos(vals.Current(), vals.Alternate());
-        cub::DoubleBuffer<int32_t> rnk(w.hp, w.levels);
-        tb = w.tmp_bytes;
-        e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, pos, rnk, (int)total, 0, bits, stream);
-        if (e == cudaSuccess && rnk.Current() != w.levels)
-            e = cudaMemcpyAsync(w.levels, rnk.Current(), nn * 4, cudaMemcpyDeviceToDevice, stream);
-        if (e != cudaSuccess) return e;
+                                                                           bps * csyms, bps, words, sa, w.sep, lcp);
+        if (wins <= kScatterWins) {
+            scatter_words(vals.Current(), words, total, w.levels);
+        } else {
+            cub::DoubleBuffer<int32_t> pos(vals.Current(), vals.Alternate());
+            cub::DoubleBuffer<int32_t> rnk(w.hp, w.levels);
+            tb = w.tmp_bytes;
+            e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, pos, rnk, (int)total, 0, bits, stream);
+            if (e == cudaSuccess && rnk.Current() != w.levels)
+                e = cudaMemcpyAsync(w.levels, rnk.Current(), nn * 4, cudaMemcpyDeviceToDevice, stream);
+            if (e != cudaSuccess) return e;
+        }
     }
     // the active positions, ascending (their rank words are then read in
     // order); only the suffixes in groups of two or more are sorted again
@@ -570,8 +620,15 @@ cudaError_t build_arrays_batch(const uint8_t* text, long long total, const int64
         tb = w.tmp_bytes;
         e = cub::DeviceRadixSort::SortPairs(w.tmp, tb, keys, vals, (int)A, 0, 2 * bits, stream);
         if (e != cudaSuccess) return e;
-        k_update<<<blocks(A, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), A, bits, level, sa, w.sep,
-                                                                  r);
+        if (direct || A <= kDirectWords || wins > kUpdateWins) {
+            k_update<true><<<blocks(A, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), A, bits, level,
+                                                                            sa, w.sep, r);
+        } else {
+            int32_t* words = reinterpret_cast<int32_t*>(keys.Alternate());
+            k_update<false><<<blocks(A, kGrpTile), kGrpThreads, 0, stream>>>(keys.Current(), vals.Current(), A, bits, words,
+                                                                             sa, w.sep, r);
+            scatter_words(vals.Current(), words, A, level);
+        }
         tb = w.tmp_bytes;
         e = cub::DeviceSelect::If(w.tmp, tb, (const int32_t*)act, spare, w.misc + 2, (int)A, ActiveAt{level}, stream);
         if (e != cudaSuccess) return e;

@@ -58,16 +58,19 @@ def test_many_strings(ctx, kind, lens):
     assert np.array_equal(lcp.cpu().numpy(), wlcp)
 
 
-def test_ranks_sorted_back_past_the_scatter(ctx):
-    """More positions than round 0's ranks are scattered for: the suffix array is a permutation in suffix order."""
-    n = (40 << 20) + 3
+@pytest.mark.parametrize("n", [(30 << 20) + 5, (40 << 20) + 3, (13 << 24) + 1])
+def test_ranks_back_to_position_order(ctx, n):
+    """Round 0's ranks scattered in windows of 2^24 positions (the last one partial), and past 13 windows sorted
+    back: the suffix array is a permutation in suffix order."""
     text = torch.from_numpy(W.dna_iid(n, 3)).cuda()
+    text[n // 2: n // 2 + 3000] = text[:3000]              # a few more rounds
     sa, rank, lcp = ctx.build_arrays(text)
     assert torch.equal(rank[sa.long()], torch.arange(n, dtype=torch.int32, device="cuda"))
     # sampled neighbours: lcp symbols equal, the next one in order
     r = torch.randint(1, n, (200_000,), device="cuda")
+    r[:2] = torch.stack([rank[0], rank[n // 2]]).long().clamp(min=1)
     x, y, m = sa[r - 1].long(), sa[r].long(), lcp[r].long()
-    for t in range(int(lcp.max()) + 1):
+    for t in range(int(m.max()) + 1):
         a = torch.where(x + t < n, text[(x + t).clamp(max=n - 1)].long(), -1)
         b = torch.where(y + t < n, text[(y + t).clamp(max=n - 1)].long(), -1)
         assert bool((a[m > t] == b[m > t]).all()) and bool((a[m == t] < b[m == t]).all())
