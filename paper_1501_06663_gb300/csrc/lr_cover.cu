@@ -588,7 +588,8 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
 // and one launch (Lemma 1 from sa or rank into shared memory by position,
 // flags, compaction, cover), with nothing to clear before it.  What bounds a
 // query of this size is launches and the chains between them: 4099
-// positions of DNA took 74 us with five launches, and 42 us with this one.
+// positions of DNA took 74 us with five launches, and 42 us with this one (33 us
+// since the results of a query come back in one copy).
 constexpr int kOneTP = 4;
 static_assert(Cfg<kOneTP>::kTileC == kOneTileMax, "one-tile strings");
 

@@ -389,7 +389,12 @@ __device__ __forceinline__ unsigned level1_scatter(const PartSmem& P, int nb, co
 
 // Level 1: Lemma 1 in rank order.  Each CTA takes kPartRound consecutive
 // ranks r, forms <sa[r], max(lcp[r], lcp[r+1])> and partitions these pairs
-// into super-buckets of 2^20 positions (level1_scatter).
+// into super-buckets of 2^20 positions (level1_write).  What bounds it:
+// shared-memory wavefronts (84 % of the load/store pipe's rate: the counting
+// atomics, the staging stores and the look-ups of staging offsets hit random
+// banks).  2^26 positions of English take 207 us (2.6 instructions per
+// position); 231 us with every entry checked, 4-byte shared loads and the
+// bucket ids in an array of their own.
 template <bool kBatch>
 __global__ void __launch_bounds__(kPartThreads, kPartBlocks)
 k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t n, Scratch s, Segs segs, int tma) {
@@ -587,7 +592,9 @@ k_part1(const int32_t* __restrict__ sa, const int32_t* __restrict__ lcp, int32_t
 // window's 16 MB slice of lcp (CTAs run in window order, so the slice stays
 // in L2 while its window is processed) and partitions <i, L_i> into the
 // level-1 super-buckets like k_part1.  k_part2 and k_bucket_llr follow
-// unchanged.
+// unchanged.  2^26 positions of English: k_rank_win 226 us (245 with window
+// ids staged beside the pairs, shared-memory wavefronts 72 %), k_part1_win
+// 490 us (waits on the scattered L2 reads of lcp).
 __host__ __device__ inline size_t win_stage_offset(int nw) { return ((size_t)(2 * nw + 1) * 4 + 15) & ~(size_t)15; }
 size_t rank_win_smem_bytes(int nw) { return win_stage_offset(nw) + (size_t)kPartRound * 8; }
 size_t part_scatter_smem_bytes(int nb) { return part_stage_offset(nb) + (size_t)kPartRound * 8; }
@@ -730,7 +737,9 @@ k_part1_win(const int32_t* __restrict__ lcp, int32_t n, Scratch s) {
 // kSubPerSuper buckets the same way.  The entries stay as they are: a
 // bucket's CTA reads the position mod 2^15 from them.  CTAs stay and take
 // every gridDim.x-th round; the next round's entries arrive by a bulk copy
-// while this one is counted, staged and written.
+// while this one is counted, staged and written.  Bound by shared-memory
+// wavefronts like k_part1 (81 %): 2^26 positions of English take 117 us (0.93
+// instructions per entry), 151 with every entry checked and the ids staged.
 // kRuns: slots by run_slot, for level-1 entries that come clustered by
 // bucket (those of the rank-window front end).
 template <bool kRuns>
@@ -990,7 +999,8 @@ __device__ __forceinline__ void llr_bases(long long tile, const int32_t* offs, l
 //
 // 2^26 positions of English take 114 us (67 M warp instructions); with a
 // ballot per run of 32 positions and one store per flagged lane it was 190 us
-// (156 M).
+// (156 M).  With the first entries loaded while the words are preset, 2^28
+// positions take 421 us instead of 436.
 __device__ __forceinline__ uint32_t bucket_pattern(int x, int pair) {   // position bits of words x + 2 pair, x + 2 pair + 1
     const uint32_t lo = (uint32_t)((x & 8) + 2 * pair);
     return (lo << 12) | ((lo + 1) << 28);

@@ -40,17 +40,19 @@ constexpr int kMaxWins = 512;                  // n < 2^31
 constexpr long long kRankWinMinN = 1LL << 24;
 
 // A string of at most this many positions takes one CTA and one launch
-// (4099 positions: 74 -> 42 us; above, one CTA would work alone for longer
-// than the launches of the other paths take: 20 000 positions need 67 us there).
+// (4099 positions: 74 -> 42 us, 33 with one copy of the results; above, one
+// CTA would work alone for longer than the launches of the other paths take:
+// 20 000 positions need 67 us there).
 constexpr int kOneTileMax = 8192;
 
 // Up to this many positions (one string, or a batch) the lengths of Lemma 1
 // go straight to a dense array in text order (2 bytes each, scattered stores
 // that merge in L2) instead of through the radix partition.  Where the lines
-// lie: whole queries, dense and partition, DNA: 2 x 10^5 positions 59 and
-// 78 us, 2^20 84 and 101 us, 4 x 10^6 134 and 141 us, 8 x 10^6 202 and 193 us
-// (scattered stores run at 110 G/s whatever the size, the partition gains
-// with it); a batch of 10^7 248 and 264 us (its partition looks strings up).
+// lie: whole queries, dense and partition, DNA: 2 x 10^5 positions 58 and
+// 73 us, 2^20 73 and 97 us, 4 x 10^6 134 and 141 us, 5.2 x 10^6 156 and 162 us,
+// 8 x 10^6 206 and 190 us (scattered stores run at 110 G/s whatever the size,
+// the partition gains with it); a batch of 10^7 256 and 271 us (its partition
+// looks strings up).
 constexpr long long kDenseMaxN = 5LL << 20;
 constexpr long long kDenseMaxBatch = 12LL << 20;
 constexpr int kCompactTile = 8192;             // positions per CTA that compacts the dense array
