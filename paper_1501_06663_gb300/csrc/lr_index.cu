@@ -82,6 +82,7 @@ struct SymCodes {
 // positions of English took 386 us.
 constexpr int kKeyThreads = 256, kKeyPer = 8, kKeyTile = kKeyThreads * kKeyPer;
 constexpr int kMaxSyms = 63;                             // one bit per symbol at least
+constexpr int kKeySteps = 4;                             // strings a thread steps over before it searches
 __global__ void __launch_bounds__(kKeyThreads)
 k_keys0(const uint8_t* __restrict__ text, long long total, const int64_t* __restrict__ off, long long num, int csyms,
         int bps, SymCodes codes, uint64_t* __restrict__ key, int32_t* __restrict__ val, int32_t* __restrict__ end) {
@@ -118,9 +119,13 @@ k_keys0(const uint8_t* __restrict__ text, long long total, const int64_t* __rest
             if (end)
                 for (int q = 0; q < kKeyPer; ++q)
                     if (i + q < total) end[i + q] = (int32_t)e;
-        } else {                                         // across strings: each position by itself
+        } else {
+            // across strings: each position by itself; past a few empty
+            // strings the next one is looked up (2^18 of them between two
+            // strings of 50 000 positions: 17.3 ms walked, 0.30 searched)
             for (int q = 0; q < kKeyPer && i + q < total; ++q) {
-                while (i + q >= e) { ++j; e = __ldg(off + j + 1); }
+                for (int t = 0; t < kKeySteps && i + q >= e; ++t) { ++j; e = __ldg(off + j + 1); }
+                if (i + q >= e) { j = string_of(off, num, i + q); e = __ldg(off + j + 1); }
                 uint64_t k = (uint64_t)j;
                 for (int t = 0; t < csyms; ++t) k = (k << bps) | (i + q + t < e ? (uint64_t)cd[tid * kKeyPer + q + t] : 0ull);
                 o[q] = k;

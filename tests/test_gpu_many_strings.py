@@ -1,0 +1,68 @@
+"""Batches at the extremes of their string tables: long runs of empty strings,
+strings of a few symbols.
+
+Results against the host preparation and the oracle, bit-exact.  Times are
+compared within one run with the same symbols in an ordinary table, so that
+no thread may walk a long stretch of the table by itself.
+"""
+import time
+
+import numpy as np
+import pytest
+
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1501_06663_gb300 as lrmod
+    lrmod.build_library()
+    c = lrmod.Context(0)
+    yield c
+    c.close()
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _off(lens):
+    return np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+
+
+def _ms(f, reps=7):
+    """Least time of a call, in ms (after two warm-up calls)."""
+    best = float("inf")
+    for i in range(reps + 2):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        f()
+        torch.cuda.synchronize()
+        if i >= 2:
+            best = min(best, (time.perf_counter() - t0) * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("lens", [(5, *(0,) * 3, 6), (5, *(0,) * 4, 6), (5, *(0,) * 5, 6), (1, *(0,) * 4000, 2, 0, 3),
+                                  (*(0,) * 9, 2047, *(0,) * 700, 2, *(0,) * 5, 4096, *(0,) * 9)])
+def test_build_over_runs_of_empty_strings(ctx, lens):
+    off = _off(lens)
+    text = np.random.default_rng(len(lens)).integers(0, 3, int(off[-1])).astype(np.uint8)
+    got = ctx.build_arrays_batch(_dev(off), _dev(text))
+    for a, b in zip(got, W.prep_many(text, off)):
+        assert np.array_equal(a.cpu().numpy(), b)
+
+
+def test_build_time_over_a_run_of_empty_strings(ctx):
+    """2^18 empty strings between two others: one thread's walk over them takes 2^18 dependent reads, 5 ms at 20 ns
+    each; the two strings alone build in about 0.4 ms."""
+    text = _dev(W.dna_iid(100_001, 1))
+    plain, empties = _off((50_001, 50_000)), _off((50_001, *(0,) * (1 << 18), 50_000))
+    t0 = _ms(lambda: ctx.build_arrays_batch(_dev(plain), text))
+    t1 = _ms(lambda: ctx.build_arrays_batch(_dev(empties), text))
+    assert t1 < 8 * t0, (t0, t1)
