@@ -38,6 +38,8 @@ namespace lr {
 
 namespace {
 
+constexpr int kSms = 152;                // of a GB300: grids of the kernels whose CTAs stay
+
 // The same pointer, its origin hidden from the compiler.  The stage areas of the
 // partition kernels are reached through such pointers: measured with events,
 // at 2^28 positions of English, the partition phase takes 1.39 ms with both
@@ -94,7 +96,9 @@ struct SegView {
 
 // For every tile of kTile flattened positions, the string holding its first
 // position (the last j with off[j] <= tile start); the offset table is
-// checked on the way.
+// checked on the way, by all `step` threads.  With the strings dealt to the
+// threads of the tiles alone, a query of 4.5 M strings of one symbol took 2.77
+// ms by rank and 1.06 ms by sa, most of it here; now 0.16 ms.
 __device__ __forceinline__ void seg_index(int32_t n, const Scratch& s, const Segs& segs, long long first, long long step) {
     for (long long t = first; t < s.ntiles; t += step) {
         const long long g = t * kTile;
@@ -104,23 +108,29 @@ __device__ __forceinline__ void seg_index(int32_t n, const Scratch& s, const Seg
             if (__ldg(segs.off + mid) <= g) lo = mid; else hi = mid - 1;
         }
         s.tile_seg[t] = (int32_t)lo;
-        if (t == 0 && (__ldg(segs.off) != 0 || __ldg(segs.off + segs.num) != n)) report(s, kErrInput);
-        // offsets must not decrease
-        for (long long j = t; j < segs.num; j += s.ntiles)
-            if (__ldg(segs.off + j) > __ldg(segs.off + j + 1)) report(s, kErrInput);
     }
+    if (first == 0 && (__ldg(segs.off) != 0 || __ldg(segs.off + segs.num) != n)) report(s, kErrInput);
+    // offsets must not decrease
+    for (long long j = first; j < segs.num; j += step)
+        if (__ldg(segs.off + j) > __ldg(segs.off + j + 1)) report(s, kErrInput);
+}
+
+// Blocks of 256 threads for `work` items of a kernel that also runs
+// seg_index: four items or strings per thread, a few blocks per SM at most.
+unsigned index_grid(long long work, const Segs& segs) {
+    const long long most = work > segs.num ? work : segs.num, blocks = (most + 1023) / 1024;
+    return (unsigned)(blocks < 8 * kSms ? blocks : 8 * kSms);
 }
 
 __global__ void k_seg_index(int32_t n, Scratch s, Segs segs) {
     begin_after();
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < s.ntiles) seg_index(n, s, segs, t, s.ntiles);
+    seg_index(n, s, segs, (long long)blockIdx.x * blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
 }  // namespace
 
 void launch_seg_index(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream) {
-    k_seg_index<<<(unsigned)((s.ntiles + 255) / 256), 256, 0, stream>>>(n, s, segs);
+    k_seg_index<<<index_grid(4 * s.ntiles, segs), 256, 0, stream>>>(n, s, segs);
 }
 
 // ---------------------------------------------------------------------------
@@ -159,7 +169,6 @@ __device__ __forceinline__ PartSmem part_smem(unsigned char* raw, int nb) {
 // rounded out to 16-byte multiples: at most kPartRound + 8 entries), at a
 // 16-byte-aligned offset after the counters; it overlaps the stage area,
 // which is written only after every thread has read its entries.
-constexpr int kSms = 152;                // of a GB300: grids of the kernels whose CTAs stay
 constexpr int kPartLcpCap = kPartRound + 8;
 constexpr int kPartLoadBytes = kPartRound * 4 + kPartLcpCap * 4;
 __host__ __device__ inline size_t part_load_offset(int nb) { return ((size_t)(2 * nb + 1) * 4 + 15) & ~(size_t)15; }
@@ -1136,8 +1145,7 @@ __global__ void __launch_bounds__(256) k_prep(int32_t n, Scratch s, Segs segs, i
 }
 
 void launch_prep(int32_t n, const Scratch& s, const Segs& segs, bool fill, cudaStream_t stream) {
-    const long long work = fill ? ((long long)n + 7) / 8 : s.ntiles, blocks = (work + 1023) / 1024;
-    k_prep<<<(unsigned)(blocks < 8 * kSms ? blocks : 8 * kSms), 256, 0, stream>>>(n, s, segs, fill ? 1 : 0);
+    k_prep<<<index_grid(fill ? ((long long)n + 7) / 8 : s.ntiles, segs), 256, 0, stream>>>(n, s, segs, fill ? 1 : 0);
 }
 
 template <bool kBatch>

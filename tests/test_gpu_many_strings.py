@@ -66,3 +66,49 @@ def test_build_time_over_a_run_of_empty_strings(ctx):
     t0 = _ms(lambda: ctx.build_arrays_batch(_dev(plain), text))
     t1 = _ms(lambda: ctx.build_arrays_batch(_dev(empties), text))
     assert t1 < 8 * t0, (t0, t1)
+
+
+def _outs(n, cap):
+    return (torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda"),
+            torch.empty(n + 1, dtype=torch.int64, device="cuda"), torch.empty(cap, dtype=torch.int32, device="cuda"))
+
+
+def _query(ctx, off, lcp, out, **arrays):
+    import paper_1501_06663_gb300 as lr
+    return lr.lr_batch_query_all(ctx.handle, lr.batch_desc(off, lcp, **arrays), *out)
+
+
+@pytest.mark.parametrize("front", ["sa", "rank"])
+@pytest.mark.parametrize("at", [0, 255, 2 ** 17, 399_998])
+def test_a_wrong_offset_anywhere_in_a_long_table(ctx, front, at):
+    """400 000 strings of 1 or 2 symbols; one offset is larger than the next."""
+    import paper_1501_06663_gb300 as lr
+    lens = np.random.default_rng(at).integers(1, 3, 400_000)
+    off = _off(lens)
+    n = int(off[-1])
+    text = np.random.default_rng(at + 1).integers(0, 4, n).astype(np.uint8)
+    sa, rank, lcp = ctx.build_arrays_batch(_dev(off), _dev(text))
+    out = _outs(n, 4 * n)
+    arrays = {"sa": sa} if front == "sa" else {"rank": rank}
+    status, total = _query(ctx, _dev(off), lcp, out, **arrays)
+    assert status == lr.LR_OK and total >= 0
+    wrong = off.copy()
+    wrong[at + 1] = off[at + 2] + 1 if at + 2 < off.size - 1 else off[at] - 1
+    assert _query(ctx, _dev(wrong), lcp, out, **arrays)[0] == lr.LR_ERR_SENTINEL
+
+
+@pytest.mark.parametrize("front", ["sa", "rank"])
+def test_query_time_of_very_short_strings(ctx, front):
+    """4.5 M strings of one symbol against 2197 of 2048: the check of the string table is 36 MB of reads, so the calls
+    take about as long as each other (a thread per 2048 symbols checking it: 7 and 20 times as long)."""
+    ms = []
+    for each in (2048, 1):
+        num = 4_500_000 // each
+        off = _dev(_off(np.full(num, each)))
+        n = num * each
+        text = _dev(W.dna_iid(n, 5))
+        sa, rank, lcp = ctx.build_arrays_batch(off, text)
+        out = _outs(n, 4 * n)
+        arrays = {"sa": sa} if front == "sa" else {"rank": rank}
+        ms.append(_ms(lambda: _query(ctx, off, lcp, out, **arrays)))
+    assert ms[1] < 3 * ms[0], ms
