@@ -23,7 +23,6 @@ struct lr_ctx {
     long long* h_pinned = nullptr;        // [0], [1] Readback, [2] compact size
     unsigned char* hostpath = nullptr;    // device buffers of lr_query_all_host
     size_t hostpath_bytes = 0;
-    int sms = 0;                          // SM count of the device
     long long last_n = 0;                 // size of the last query (its tile_cbase[ntiles] is m)
     lr::PhaseEvents events;               // per-kernel timing (off by default)
     bool events_created = false;
@@ -84,7 +83,7 @@ struct Layout {
 Layout layout_for(long long n) {
     const long long nt = lr::num_tiles(n), nb = lr::num_buckets(n), ns = lr::num_supers(n), ng = lr::num_segs(n);
     Layout L;
-    L.off_status_g = kAlign;                       // tickets in [0, 16), per-query error bits at 16
+    L.off_status_g = kAlign;                       // tickets in [0, 16)
     L.off_status_b = align_up(L.off_status_g + (size_t)nt * 8);
     L.off_status_o = align_up(L.off_status_b + (size_t)nb * 8);
     L.off_status_w = align_up(L.off_status_o + (size_t)nt * 8);
@@ -110,7 +109,6 @@ Layout layout_for(long long n) {
 void carve(unsigned char* b, long long cap_n, long long n, unsigned* d_err, lr::Scratch* s) {
     const Layout L = layout_for(cap_n);
     s->tickets = (unsigned*)b;
-    s->qerr = (unsigned*)(b + 16);
     s->err = d_err;
     s->status_g = (unsigned long long*)(b + L.off_status_g);
     s->status_b = (unsigned long long*)(b + L.off_status_b);
@@ -290,7 +288,6 @@ lr_status lr_create(lr_ctx** out, int device) {
     ctx->device = device;
     DeviceGuard g(device);
     cudaError_t e = g.ok ? cudaSuccess : cudaErrorInvalidDevice;
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = lr::configure_kernels();
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->d_err, 256);
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, 256);

@@ -159,7 +159,7 @@ __device__ __forceinline__ void store_offsets(int64_t* p, long long a, long long
 // tiles, publish the inclusive prefix, write offsets[n] from the last tile.
 __device__ __forceinline__ long long place_tile(const Scratch& s, long long tile, long long ntiles, int32_t n, int tot,
                                                 int64_t* __restrict__ offsets) {
-    const long long ex = (tile == 0) ? 0 : lookback(s.status_o, tile, s.err, s.qerr, s.spin_limit);
+    const long long ex = (tile == 0) ? 0 : lookback(s.status_o, tile, s.err, s.spin_limit);
     if (lane_id() == 0) {
         if (tile != 0 && tile != s.hold_tile) publish(s.status_o, tile, kPrefix, ex + tot);
         if (tile == ntiles - 1) {
@@ -645,7 +645,6 @@ k_one_tile(const int32_t* __restrict__ in, const int32_t* __restrict__ lcp, int3
         sm.ttot = 0;
         sm.far = 0;
         sm.rec[0] = 0;
-        *s.qerr = 0;
     }
     if (tid < kChunks) sm.bmap[tid] = tid == 0 ? 1u : 0u;
     if constexpr (kAll) {
@@ -696,10 +695,7 @@ k_one_tile(const int32_t* __restrict__ in, const int32_t* __restrict__ lcp, int3
         if (l[j] > 0 && l[j] >= prev) f |= 1u << j;           // 0 past the end
         prev = l[j];
     }
-    if (bad) {
-        atomicOr(s.err, kErrInput);
-        atomicOr(s.qerr, kErrInput);
-    }
+    if (bad) atomicOr(s.err, kErrInput);
     const int c = __popc(f), incl = warp_incl_scan(c);
     if (lane == kWarp - 1) wsum[warp] = incl;
     __syncthreads();

@@ -85,7 +85,7 @@ struct Range {
     const int32_t* cs;
     const int32_t* ce;                       // staged: lengths; in place: ends
     __device__ __forceinline__ int32_t s(int32_t v) const {
-        if constexpr (kStaged) return cs[v]; else return cs[v];
+        return cs[v];
     }
     __device__ __forceinline__ int32_t len(int32_t v) const {
         if constexpr (kStaged) return ce[v]; else return ce[v] - cs[v] + 1;
@@ -388,7 +388,7 @@ k_cover_w(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restric
     if (warp == 0) {
         const bool held = tile == s.hold_tile;
         if (lane == 0 && !held) publish(s.status_w, tile, tile == 0 ? kPrefix : kAggregate, tile_tot);
-        const long long ex = (tile == 0) ? 0 : lookback(s.status_w, tile, s.err, s.qerr, s.spin_limit);
+        const long long ex = (tile == 0) ? 0 : lookback(s.status_w, tile, s.err, s.spin_limit);
         if (lane == 0) {
             if (tile != 0 && !held) publish(s.status_w, tile, kPrefix, ex + tile_tot);
             if ((tile + 1) * kSegWarps >= s.nsegs) {

@@ -83,9 +83,9 @@ __device__ __forceinline__ void publish(unsigned long long* status, long long ti
 // needed, so only their lanes wait for a word still unset.  Waits only on
 // earlier tiles, which were scheduled before this one; after `limit` polls
 // (kSpinLimit unless a test shortens it) a missing word counts as a prefix
-// of 0 and a timeout is recorded in both error words.
+// of 0 and a timeout is recorded in the error word.
 __device__ __forceinline__ long long lookback(const unsigned long long* status, long long tile, unsigned* err,
-                                              unsigned* qerr, int limit) {
+                                              int limit) {
     const unsigned lane = lane_id();
     long long exclusive = 0;
     long long base = tile - 1;
@@ -101,10 +101,7 @@ __device__ __forceinline__ long long lookback(const unsigned long long* status, 
             const bool missing = (int)lane <= stop && (w >> kFlagShift) == 0;
             if (!__any_sync(kFull, missing)) break;
             if (++polls >= limit) {
-                if (lane == 0) {
-                    atomicOr(err, kErrTimeout);
-                    atomicOr(qerr, kErrTimeout);
-                }
+                if (lane == 0) atomicOr(err, kErrTimeout);
                 if (missing) w = kPrefix << kFlagShift;
                 continue;
             }
@@ -121,12 +118,11 @@ __device__ __forceinline__ long long lookback(const unsigned long long* status, 
 
 // Publish-aggregate, look back, publish-prefix in one call (one whole warp).
 __device__ __forceinline__ long long lookback_exclusive(unsigned long long* status, long long tile,
-                                                       long long aggregate, unsigned* err, unsigned* qerr,
-                                                       int limit) {
+                                                       long long aggregate, unsigned* err, int limit) {
     const unsigned lane = lane_id();
     if (lane == 0) publish(status, tile, tile == 0 ? kPrefix : kAggregate, aggregate);
     if (tile == 0) return 0;
-    const long long ex = lookback(status, tile, err, qerr, limit);
+    const long long ex = lookback(status, tile, err, limit);
     if (lane == 0) publish(status, tile, kPrefix, ex + aggregate);
     return ex;
 }
@@ -149,10 +145,6 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned coun
 
 // Makes initialised mbarriers visible to the async (bulk copy) proxy.
 __device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
-}
 
 // Arrives and adds `bytes` to the transaction count the phase waits for.
 __device__ __forceinline__ void mbar_arrive_tx(unsigned long long* bar, unsigned bytes) {

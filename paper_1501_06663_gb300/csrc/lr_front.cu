@@ -48,10 +48,7 @@ constexpr int kSms = 152;                // of a GB300: grids of the kernels who
 template <class T>
 __device__ __forceinline__ T* opaque(T* p) { asm volatile("" : "+l"(p)); return p; }
 
-__device__ __forceinline__ void report(const Scratch& s, unsigned bits) {
-    atomicOr(s.err, bits);
-    atomicOr(s.qerr, bits);
-}
+__device__ __forceinline__ void report(const Scratch& s, unsigned bits) { atomicOr(s.err, bits); }
 
 // The strings of a batched query that overlap one CTA's flattened range
 // [g0, g1), with their offsets staged in shared memory when there are at
@@ -974,7 +971,7 @@ __device__ __forceinline__ long long llr_place(int32_t* counts, unsigned long lo
         ex += a[u];
     }
     *total = __shfl_sync(kFull, incl, kWarp - 1);
-    return lookback_exclusive(status, tile, *total, s.err, s.qerr, s.spin_limit);
+    return lookback_exclusive(status, tile, *total, s.err, s.spin_limit);
 }
 
 // First LLRc entry of each tile of kTile positions and of each segment of
@@ -1131,7 +1128,7 @@ constexpr uint32_t kDenseNone = 0xffffu;
 __global__ void __launch_bounds__(256) k_prep(int32_t n, Scratch s, Segs segs, int fill) {
     begin_after();
     const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
-    if (i0 < 8) s.tickets[i0] = 0;                // tickets and the query's error bits
+    if (i0 < 4) s.tickets[i0] = 0;
     for (long long i = i0; i < s.ntiles; i += step) {
         s.status_g[i] = 0;
         s.status_o[i] = 0;

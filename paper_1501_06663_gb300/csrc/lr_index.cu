@@ -648,21 +648,4 @@ cudaError_t build_arrays_batch(const uint8_t* text, long long total, const int64
     return cudaGetLastError();
 }
 
-// One string: the work memory is allocated here and freed before returning.
-cudaError_t build_arrays(const uint8_t* text, int32_t n, int32_t* sa, int32_t* rank, int32_t* lcp,
-                         cudaStream_t stream, int* rounds_out) {
-    IndexWork w;
-    cudaError_t e = w.alloc(n, 8);
-    if (e != cudaSuccess) return e;
-    int64_t* off = nullptr;                                         // {0, n}
-    if (cudaMalloc((void**)&off, 16) != cudaSuccess) { cudaGetLastError(); w.release(); return cudaErrorMemoryAllocation; }
-    const int64_t h_off[2] = {0, (int64_t)n};
-    e = cudaMemcpyAsync(off, h_off, sizeof(h_off), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = build_arrays_batch(text, n, off, 1, sa, rank, lcp, w, true, stream, rounds_out);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    cudaFree(off);
-    w.release();
-    return e;
-}
-
 }  // namespace lr

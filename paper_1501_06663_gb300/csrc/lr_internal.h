@@ -64,7 +64,6 @@ constexpr int kSpinLimit = 1 << 23;
 // Device scratch of one query, carved out of one allocation by the context.
 struct Scratch {
     unsigned* tickets;             // [1] buckets or dense tiles, [2] cover tiles
-    unsigned* qerr;                // error bits of this query (cleared with the tickets)
     unsigned* err;                 // sticky device error bits (kErr*), read by the host
     unsigned long long* status_g;  // look-back words of the dense front end (per tile of kCompactTile)
     unsigned long long* status_b;  // look-back words of the rank-order front end (per bucket)
@@ -218,9 +217,6 @@ size_t index_work_bytes(long long n, int rounds);
 cudaError_t build_arrays_batch(const uint8_t* text, long long total, const int64_t* off, long long num, int32_t* sa,
                                int32_t* rank, int32_t* lcp, IndexWork& w, bool grow, cudaStream_t stream,
                                int* rounds_out);
-// One string; allocates and frees its own work memory.
-cudaError_t build_arrays(const uint8_t* text, int32_t n, int32_t* sa, int32_t* rank, int32_t* lcp,
-                         cudaStream_t stream, int* rounds_out);
 
 // Scratch management (lr_api.cu): bytes of a scratch block for n positions,
 // and the carving of such a block (laid out for cap_n >= n) into `s`.

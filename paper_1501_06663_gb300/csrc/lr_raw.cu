@@ -29,10 +29,7 @@ constexpr int kRawWarps = kRawThreads / kWarp;
 constexpr int kRawChunks = kRawTile / kWarp;           // runs of 32 positions per tile
 constexpr int kRawPerWarp = kRawChunks / kRawWarps;
 
-__device__ __forceinline__ void report_input(const Scratch& s) {
-    atomicOr(s.err, kErrInput);
-    atomicOr(s.qerr, kErrInput);
-}
+__device__ __forceinline__ void report_input(const Scratch& s) { atomicOr(s.err, kErrInput); }
 
 __global__ void __launch_bounds__(256) k_llr_raw(const int32_t* __restrict__ rank, const int32_t* __restrict__ lcp,
                                                  int32_t n, Scratch s, int32_t* __restrict__ llrr) {
@@ -111,7 +108,7 @@ __global__ void __launch_bounds__(kRawThreads) k_rawwalk(int32_t n, const int32_
         __syncthreads();
         if (warp == 0) {
             const int tot = scan_runs(run_tot);
-            const long long ex = lookback_exclusive(s.status_o, tile, tot, s.err, s.qerr, s.spin_limit);
+            const long long ex = lookback_exclusive(s.status_o, tile, tot, s.err, s.spin_limit);
             if (lane == 0) {
                 obase_s = ex;
                 if (k0 + kRawTile >= n) {

@@ -18,7 +18,7 @@ constexpr size_t align_s(size_t v) { return (v + kAlignS - 1) / kAlignS * kAlign
 // Scratch layout for n <= kStaticMaxN (rank-gather front end + cover kernel).
 constexpr long long kTilesMax = (kStaticMaxN + lr::kTile - 1) / lr::kTile;
 constexpr long long kSegsMax = (kStaticMaxN + lr::kSeg - 1) / lr::kSeg;
-constexpr size_t kOffStatusG = kAlignS;                   // [0, 256): tickets, per-query and sticky error bits
+constexpr size_t kOffStatusG = kAlignS;                   // [0, 256): tickets and the error bits
 constexpr size_t kOffStatusO = align_s(kOffStatusG + (size_t)kTilesMax * 8);
 constexpr size_t kOffStatusW = align_s(kOffStatusO + (size_t)kTilesMax * 8);
 constexpr size_t kOffCbase = align_s(kOffStatusW + (size_t)((kStaticMaxN + lr::kSegTile - 1) / lr::kSegTile) * 8);
@@ -68,7 +68,6 @@ extern "C" lr_status lr_query_all_static(lr_stream_t stream, const int32_t* d_ra
 
     lr::Scratch s = {};
     s.tickets = reinterpret_cast<unsigned*>(b);
-    s.qerr = reinterpret_cast<unsigned*>(b + 16);
     s.err = reinterpret_cast<unsigned*>(b + 32);
     s.status_g = reinterpret_cast<unsigned long long*>(b + kOffStatusG);
     s.status_o = reinterpret_cast<unsigned long long*>(b + kOffStatusO);
