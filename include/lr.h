@@ -28,7 +28,8 @@
  *     call), the pairs <rank[i], i> are first partitioned into windows of
  *     2^22 ranks, so that each window's gathers hit L2, and then join the
  *     sa path's partition.
- * A string of at most 8192 positions is answered by one kernel.
+ * A string of at most 8192 positions is answered by one kernel (not in a
+ * batch, by the server, or through the raw-LLR calls).
  * All give identical results.  sa must be a permutation of [0, n) and rank
  * its inverse; a violation that the kernels detect is reported as
  * LR_ERR_SENTINEL, and no input ever makes a kernel access memory out of
@@ -431,9 +432,10 @@ lr_status lr_test_hold_lookback(lr_ctx* ctx, int64_t tile, int32_t spin_limit);
 
 /*
  * Kernels launched by the most recent query of this context (for the
- * benchmark's launch accounting): 1 for a string of at most 8192 positions;
- * else 4 (5 through the rank windows, one more for a batch that takes the
- * partition); 2 for the raw-LLR variant, 6 for lr_walk_stats.
+ * benchmark's launch accounting): 1 for a string of at most 8192 positions
+ * (not a batch); else 4 (3 for one string by rank, 5 through the rank windows,
+ * one more for a batch that takes the partition); 2 for the raw-LLR variant, 4
+ * for lr_walk_stats.
  */
 int32_t lr_last_launch_count(lr_ctx* ctx);
 

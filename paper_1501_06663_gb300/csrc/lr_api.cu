@@ -647,7 +647,7 @@ lr_status lr_walk_stats(lr_ctx* ctx, lr_stream_t stream, const int32_t* d_rank, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(hs, d_stats, sizeof(hs), cudaMemcpyDeviceToHost, strm);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&m, s.tile_cbase + s.ntiles, 4, cudaMemcpyDeviceToHost, strm);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
-    ctx->last_launches = 6;
+    ctx->last_launches = 4;
     st = sync_total(ctx, strm, nullptr);
     if (st != LR_OK) return st;
     const int32_t* w = reinterpret_cast<const int32_t*>(hs + 2);

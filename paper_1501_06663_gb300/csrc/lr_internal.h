@@ -160,9 +160,10 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
 void launch_seg_index(int32_t n, const Scratch& s, const Segs& segs, cudaStream_t stream);
 void launch_partition(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                       cudaStream_t stream);
-// The dense front end: k_prep clears what it needs cleared (with `fill` the
-// dense array too) and, for a batch, does k_seg_index's work; k_scatter (sa) or
-// k_gather (rank) fills the array, k_compact compacts it.
+// The dense front end: k_prep (sa, or a batch) clears what it needs cleared
+// (with `fill` the dense array too) and, for a batch, does k_seg_index's work;
+// k_scatter (sa) or k_gather (rank; clears for one string itself) fills the
+// array, k_compact compacts it.
 void launch_prep(int32_t n, const Scratch& s, const Segs& segs, bool fill, cudaStream_t stream);
 void launch_scatter(const int32_t* sa, const int32_t* lcp, int32_t n, const Scratch& s, const Segs& segs,
                     cudaStream_t stream);

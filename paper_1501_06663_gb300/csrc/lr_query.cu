@@ -41,7 +41,7 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
     const bool dense = sa ? (long long)n <= (segs.num > 0 ? kDenseMaxBatch : kDenseMaxN) : !rankwin;
     mark();
     if (dense) {
-        launch_prep(n, s, segs, sa != nullptr, stream);             // k_prep
+        if (sa || segs.num > 0) launch_prep(n, s, segs, sa != nullptr, stream);   // k_prep
         if (sa) launch_scatter(sa, lcp, n, s, segs, stream);        // k_scatter
         else launch_gather(rank, lcp, n, s, segs, stream);          // k_gather
         mark();
@@ -61,7 +61,7 @@ cudaError_t launch_query(const int32_t* sa, const int32_t* rank, const int32_t* 
     else
         launch_cover_w(n, s, lr_len, lr_start, offsets, starts, capacity, all, stream);
     if (timed) cudaEventRecord(events->ev[k], stream);
-    if (launches) *launches = dense ? 4 : (sa ? 4 : 5) + (segs.num > 0 ? 1 : 0);
+    if (launches) *launches = dense ? (sa || segs.num > 0 ? 4 : 3) : (sa ? 4 : 5) + (segs.num > 0 ? 1 : 0);
     if (events) events->count = k;
     return cudaGetLastError();
 }

@@ -32,8 +32,15 @@ constexpr int kRawPerWarp = kRawChunks / kRawWarps;
 __device__ __forceinline__ void report_input(const Scratch& s) { atomicOr(s.err, kErrInput); }
 
 __global__ void __launch_bounds__(256) k_llr_raw(const int32_t* __restrict__ rank, const int32_t* __restrict__ lcp,
-                                                 int32_t n, Scratch s, int32_t* __restrict__ llrr) {
+                                                 int32_t n, Scratch s, int32_t* __restrict__ llrr,
+                                                 unsigned long long* __restrict__ stats) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && stats) {                                   // what k_walk_stats starts from
+        stats[0] = 0;
+        stats[1] = 0;
+        int* w = reinterpret_cast<int*>(stats + 2);
+        w[0] = 0x7fffffff; w[1] = 0; w[2] = 0x7fffffff; w[3] = 0;
+    }
     bool bad = false;
     if (i == 0 && (__ldg(lcp) != 0 || __ldg(lcp + n) != 0)) bad = true;
     if (i < n) {
@@ -215,13 +222,6 @@ __global__ void __launch_bounds__(256) k_walk_stats(int32_t n, const int32_t* __
     }
 }
 
-__global__ void k_stats_init(unsigned long long* stats) {
-    stats[0] = 0;
-    stats[1] = 0;
-    int* w = reinterpret_cast<int*>(stats + 2);
-    w[0] = 0x7fffffff; w[1] = 0; w[2] = 0x7fffffff; w[3] = 0;
-}
-
 }  // namespace
 
 cudaError_t launch_raw_query(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, int32_t* lr_len,
@@ -230,7 +230,7 @@ cudaError_t launch_raw_query(const int32_t* rank, const int32_t* lcp, int32_t n,
     cudaError_t e = cudaMemsetAsync(s.zero_base, 0, s.zero_bytes, stream);
     if (e != cudaSuccess) return e;
     int32_t* llrr = s.lbig;
-    k_llr_raw<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rank, lcp, n, s, llrr);
+    k_llr_raw<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rank, lcp, n, s, llrr, nullptr);
     const unsigned grid = (unsigned)((n + kRawTile - 1) / kRawTile);
     if (all)
         k_rawwalk<true><<<grid, kRawThreads, 0, stream>>>(n, llrr, s, lr_len, lr_start, offsets, starts, capacity);
@@ -241,13 +241,10 @@ cudaError_t launch_raw_query(const int32_t* rank, const int32_t* lcp, int32_t n,
 
 cudaError_t launch_walk_stats(const int32_t* rank, const int32_t* lcp, int32_t n, const Scratch& s, int32_t* alpha,
                               int32_t* beta, unsigned long long* stats, cudaStream_t stream) {
-    const Segs one{nullptr, 0};
-    launch_prep(n, s, one, false, stream);
-    launch_gather(rank, lcp, n, s, one, stream);
+    launch_gather(rank, lcp, n, s, Segs{nullptr, 0}, stream);
     launch_compact(n, s, stream);                                         // LLRc in s.cstart / s.cend
     int32_t* llrr = s.lbig;
-    k_llr_raw<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rank, lcp, n, s, llrr);
-    k_stats_init<<<1, 1, 0, stream>>>(stats);
+    k_llr_raw<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(rank, lcp, n, s, llrr, stats);
     k_walk_stats<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(n, llrr, s.cstart, s.cend, s.tile_cbase, s.ntiles,
                                                                    alpha, beta, stats);
     return cudaGetLastError();

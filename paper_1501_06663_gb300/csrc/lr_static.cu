@@ -80,7 +80,8 @@ extern "C" lr_status lr_query_all_static(lr_stream_t stream, const int32_t* d_ra
     s.lbig = d_lr_len;                    // read before the cover kernel writes its lengths there
     s.ntiles = lr::num_tiles(n);
     s.nsegs = lr::num_segs(n);
-    // the error words start at zero (k_prep clears the rest)
+    s.one_tile = true;
+    // the error bits start at zero (k_gather clears the rest)
     cudaStream_t strm = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(b, 0, kAlignS, strm);
     if (e == cudaSuccess)
