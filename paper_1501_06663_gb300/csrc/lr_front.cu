@@ -861,18 +861,22 @@ k_part2(int32_t n, Scratch s, int rounds) {
 // 256 consecutive positions from position x0 on, eight consecutive positions
 // per lane.  One 16-byte load gives a lane its words, the flags are sign bits
 // shifted together (first position in the top bit).  W gives plain words:
-// load8(x) for positions x .. x + 7 and at(x); below W::kEsc a word is the
-// length, W::kEsc itself stands for a longer one (in lbig), anything above
-// for a position that got no length (reported: sa gave another one twice).
+// load8(q, x) for positions x .. x + 7 of a lane in its warp's chunk q, and
+// at(x); below W::kEsc a word is the length, W::kEsc itself stands for a longer
+// one (in lbig), anything above for a position that got no length (reported:
+// sa gave another one twice).
 // `halo`: the length of the position before 0 (used where x0 is 0).
 constexpr int kBktChunk = 256;                                   // = kSeg: seg_cbase falls out of the chunk counts
 static_assert(kBktChunk == kSeg, "chunk and segment sizes");
 
-// L of position x of a tile, 0 <= x < cnt; a position without a length counts as 0
+// L of position x of a tile, 0 <= x < cnt, whose word is f; a position without a length counts as 0
+template <class W>
+__device__ __forceinline__ int32_t word_len(uint32_t f, int x, const int32_t* lbig) {
+    return f < W::kEsc ? (int32_t)f : (f == W::kEsc ? __ldcg(lbig + x) : 0);
+}
 template <class W>
 __device__ __forceinline__ int32_t llr_len(const W& words, int x, const int32_t* lbig) {
-    const uint32_t f = words.at(x);
-    return f < W::kEsc ? (int32_t)f : (f == W::kEsc ? __ldcg(lbig + x) : 0);
+    return word_len<W>(words.at(x), x, lbig);
 }
 
 template <int kPerWarp, class W>
@@ -885,7 +889,7 @@ __device__ __forceinline__ void llr_flags(const W& words, int x0, int cnt, int32
 #pragma unroll
     for (int q = 0; q < kPerWarp; ++q) {
         const int x = x0 + q * kBktChunk + lane * 8;
-        const uint4 w = words.load8(x);
+        const uint4 w = words.load8(q, x);
         const uint32_t m = __vmaxu2(__vmaxu2(w.x, w.y), __vmaxu2(w.z, w.w));
         const bool odd = (m & 0xffffu) >= W::kEsc || (m >> 16) >= W::kEsc;
         uint32_t prev = __shfl_up_sync(kFull, w.w >> 16, 1);
@@ -919,11 +923,15 @@ __device__ __forceinline__ void llr_flags(const W& words, int x0, int cnt, int32
 }
 
 // K3: a chunk's kept positions are listed in shared memory (mine, kBktChunk
-// entries per warp) and then written to LLRc in one run.
+// entries per warp) and then written to LLRc in one run.  W::List holds the
+// position, or the position << 16 | its word where the words are not in shared
+// memory (5 x 10^4 positions: k_compact 8.7 us; 10.4 where it read each word
+// again before the entry's stores).
 template <int kPerWarp, class W>
 __device__ __forceinline__ void llr_write(const W& words, int x0, long long k0, const int32_t* lbig,
                                           const uint32_t (&flags)[(kPerWarp + 3) / 4], const int32_t* offs, long long base,
-                                          uint16_t* mine, const Scratch& s) {
+                                          typename W::List* mine, const Scratch& s) {
+    constexpr bool kListed = sizeof(typename W::List) == 4;
     const int lane = lane_id();
 #pragma unroll
     for (int q = 0; q < kPerWarp; ++q) {
@@ -932,17 +940,23 @@ __device__ __forceinline__ void llr_write(const W& words, int x0, long long k0, 
         const int c = __popc(f);
         const int incl = warp_incl_scan(c);
         int o = incl - c;
+        uint4 w = make_uint4(0, 0, 0, 0);
+        if constexpr (kListed) w = words.load8(q, x);
+        const uint32_t l[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-            if (f & (0x80u >> j)) mine[o++] = (uint16_t)(x + j);
+            if (f & (0x80u >> j))
+                mine[o++] = (typename W::List)(kListed ? ((uint32_t)(x + j) << 16) | ((l[j / 2] >> (16 * (j & 1))) & 0xffffu)
+                                                       : (uint32_t)(x + j));
         const int tot = __shfl_sync(kFull, incl, kWarp - 1);
         __syncwarp();
         const long long to = base + offs[q];
         for (int i = lane; i < tot; i += kWarp) {
-            const int y = mine[i];
+            const uint32_t e = mine[i];
+            const int y = (int)(kListed ? e >> 16 : e);
             const int32_t k = (int32_t)(k0 + y);
             s.cstart[to + i] = k;
-            s.cend[to + i] = k + llr_len(words, y, lbig) - 1;
+            s.cend[to + i] = k + word_len<W>(kListed ? e & 0xffffu : words.at(y), y, lbig) - 1;
         }
         __syncwarp();
     }
@@ -1013,9 +1027,10 @@ __device__ __forceinline__ uint32_t bucket_pattern(int x, int pair) {   // posit
 }
 struct BucketWords {
     static constexpr uint32_t kEsc = kEsc12;
+    using List = uint16_t;
     const uint16_t* sL;
     __device__ __forceinline__ uint32_t at(int x) const { return (uint32_t)sL[x] ^ ((uint32_t)(x & 15) << 12); }
-    __device__ __forceinline__ uint4 load8(int x) const {
+    __device__ __forceinline__ uint4 load8(int, int x) const {
         uint4 w = *reinterpret_cast<const uint4*>(sL + x);
         w.x ^= bucket_pattern(x, 0);
         w.y ^= bucket_pattern(x, 1);
@@ -1302,11 +1317,14 @@ __global__ void __launch_bounds__(kThreads) k_gather(const int32_t* __restrict__
     if (bad) report(s, kErrInput);
 }
 
+template <int kPerWarp>
 struct DenseWords {
     static constexpr uint32_t kEsc = kDenseEsc;
+    using List = uint32_t;
     const uint16_t* d;                            // of the tile's first position
+    uint4 w[kPerWarp];                            // the lane's own words, kept from the one load of them
     __device__ __forceinline__ uint32_t at(int x) const { return __ldcg(d + x); }
-    __device__ __forceinline__ uint4 load8(int x) const { return __ldcg(reinterpret_cast<const uint4*>(d + x)); }
+    __device__ __forceinline__ uint4 load8(int q, int) const { return w[q]; }
 };
 
 constexpr int kCompactThreads = 512;
@@ -1315,7 +1333,7 @@ __global__ void __launch_bounds__(kCompactThreads) k_compact(int32_t n, Scratch 
     constexpr int kChunks = kCompactTile / kBktChunk;        // 32
     constexpr int kWarps = kCompactThreads / kWarp;          // 16
     constexpr int kPerWarp = kChunks / kWarps;               // 2
-    __shared__ uint16_t list[kWarps * kBktChunk];
+    __shared__ uint32_t list[kWarps * kBktChunk];
     __shared__ int32_t ccnt[kChunks];
     __shared__ long long t_s, base_s;
     __shared__ int32_t total_s;
@@ -1324,9 +1342,12 @@ __global__ void __launch_bounds__(kCompactThreads) k_compact(int32_t n, Scratch 
     __syncthreads();
     const long long t = t_s, k0 = t * kCompactTile;
     const int cnt = (int)(((long long)n - k0 < kCompactTile) ? (long long)n - k0 : kCompactTile);
-    const DenseWords words{s.dense + k0};
     const int32_t* lbig = s.lbig + k0;
     const int x0 = warp * kPerWarp * kBktChunk;
+    DenseWords<kPerWarp> words{s.dense + k0, {}};
+#pragma unroll
+    for (int q = 0; q < kPerWarp; ++q)
+        words.w[q] = __ldcg(reinterpret_cast<const uint4*>(words.d + x0 + q * kBktChunk + lane * 8));
     const int32_t halo = (x0 == 0 && k0 > 0) ? llr_len(words, -1, lbig) : 0;
     unsigned bad = 0;
     uint32_t flags[1] = {};
