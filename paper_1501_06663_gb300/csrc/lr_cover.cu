@@ -553,7 +553,7 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
     CoverSmem<TP>& sm = *reinterpret_cast<CoverSmem<TP>*>(cover_smem);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        sm.tile = atomicAdd(&s.tickets[2], 1u);
+        if constexpr (kAll) sm.tile = atomicAdd(&s.tickets[2], 1u);
         sm.nlow = 0;
         sm.ttot = 0;
         sm.far = 0;
@@ -564,7 +564,9 @@ k_cover(int32_t n, Scratch s, int32_t* __restrict__ lr_len, int32_t* __restrict_
         for (int i = tid; i < CoverSmem<TP>::kNxWords; i += kCoverThreads) sm.nx[i] = 0;
     }
     __syncthreads();
-    const long long tile = sm.tile;
+    // leftmost only: no look-back, so no order of the tiles to keep (1.2 x 10^4
+    // positions by rank 31.5 -> 29.8 us without the ticket)
+    const long long tile = kAll ? sm.tile : (long long)blockIdx.x;
     const int32_t k0 = (int32_t)(tile * kCoverTile);         // n < 2^31: positions fit 32 bits
     // LLRc entries [cb0, cb1) start inside this tile; clamped so that a
     // corrupted front end (already reported) cannot send reads out of bounds
