@@ -391,7 +391,7 @@ lr_status lr_server_stop(lr_server* server);
  * allocation would synchronise the whole device and stall unrelated work),
  * or services that fix their memory budget once at start-up.  It needs no
  * context and allocates nothing: its working memory is one array of about
- * 10 MB compiled into this library's device image, which every GPU that
+ * 14 MB compiled into this library's device image, which every GPU that
  * loads the library keeps until the process exits.
  *
  * Same inputs and outputs as lr_query_all with rank (the rank-gather front

@@ -26,7 +26,8 @@ constexpr size_t kOffSegCbase = align_s(kOffCbase + (size_t)(kTilesMax + 1) * 4)
 constexpr size_t kOffCstart = align_s(kOffSegCbase + (size_t)(kSegsMax + 1) * 4);
 constexpr size_t kOffCend = align_s(kOffCstart + (size_t)kStaticMaxN * 4);
 constexpr size_t kOffDense = align_s(kOffCend + (size_t)kStaticMaxN * 4);
-constexpr size_t kStaticBytes = align_s(kOffDense + (size_t)kStaticMaxN * 2);   // about 10.1 MB
+constexpr size_t kOffLbig = align_s(kOffDense + (size_t)kStaticMaxN * 2);
+constexpr size_t kStaticBytes = align_s(kOffLbig + (size_t)kStaticMaxN * 4);   // about 14.3 MB
 static_assert(kStaticMaxN % lr::kCompactTile == 0, "whole tiles of the dense array");
 
 // The array itself.  Host code must not use its name as an address: it is a
@@ -77,7 +78,9 @@ extern "C" lr_status lr_query_all_static(lr_stream_t stream, const int32_t* d_ra
     s.cstart = reinterpret_cast<int32_t*>(b + kOffCstart);
     s.cend = reinterpret_cast<int32_t*>(b + kOffCend);
     s.dense = reinterpret_cast<uint16_t*>(b + kOffDense);
-    s.lbig = d_lr_len;                    // read before the cover kernel writes its lengths there
+    // not in an output: the outputs are written when every input has been
+    // read, so that a caller may let them replace the inputs
+    s.lbig = reinterpret_cast<int32_t*>(b + kOffLbig);
     s.ntiles = lr::num_tiles(n);
     s.nsegs = lr::num_segs(n);
     s.one_tile = true;
