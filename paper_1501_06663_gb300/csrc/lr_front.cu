@@ -1301,17 +1301,39 @@ __global__ void __launch_bounds__(kThreads) k_gather(const int32_t* __restrict__
             put(k, a[j], b[j], base, nj);
         }
     } else {
-        for (int j = 0; j < kPer; ++j) {
-            const long long k = k0 + j * kThreads + tid;
-            if (k >= n) continue;
-            hint = sv.find(k, hint);
-            const long long at = sv.at(hint), len = sv.at(hint + 1) - at;
-            if (at < 0 || len < 1 || at + len > n || k < at) { bad = 1; s.dense[k] = 0; continue; }   // bad offset table
-            uint32_t r = (uint32_t)__ldcs(rank + k);
-            if ((long long)r >= len) { bad = 1; r = 0; }
-            const int32_t a = __ldg(lcp + at + hint + r), b = __ldg(lcp + at + hint + r + 1);
-            if ((r == 0 && a != 0) || ((long long)r == len - 1 && b != 0)) bad = 1;   // lcp sentinels
-            put(k, a, b, at, len);
+        // across strings: kTogether positions at a time, each one's string
+        // beside its rank (all eight: 70 registers instead of 40, and 3 % more
+        // time where tiles lie inside strings)
+        constexpr int kTogether = 2;
+#pragma unroll 1
+        for (int j0 = 0; j0 < kPer; j0 += kTogether) {
+            uint32_t r[kTogether];
+            int32_t str[kTogether], a[kTogether], b[kTogether];   // string, or -1: no position, or a bad offset table
+#pragma unroll
+            for (int j = 0; j < kTogether; ++j) {
+                const long long k = k0 + (j0 + j) * kThreads + tid;
+                if (k < n) hint = sv.find(k, hint);
+                str[j] = k < n ? (int32_t)hint : -1;
+                r[j] = k < n ? (uint32_t)__ldcs(rank + k) : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < kTogether; ++j) {
+                const long long k = k0 + (j0 + j) * kThreads + tid;
+                a[j] = b[j] = 0;
+                if (str[j] < 0) continue;
+                const long long at = sv.at(str[j]), len = sv.at(str[j] + 1) - at;
+                if (at < 0 || len < 1 || at + len > n || k < at) { bad = 1; s.dense[k] = 0; str[j] = -1; continue; }
+                if ((long long)r[j] >= len) { bad = 1; r[j] = 0; }
+                a[j] = __ldg(lcp + at + str[j] + r[j]);
+                b[j] = __ldg(lcp + at + str[j] + r[j] + 1);
+            }
+#pragma unroll
+            for (int j = 0; j < kTogether; ++j) {
+                if (str[j] < 0) continue;
+                const long long at = sv.at(str[j]), len = sv.at(str[j] + 1) - at;
+                if ((r[j] == 0 && a[j] != 0) || ((long long)r[j] == len - 1 && b[j] != 0)) bad = 1;   // lcp sentinels
+                put(k0 + (j0 + j) * kThreads + tid, a[j], b[j], at, len);
+            }
         }
     }
     if (bad) report(s, kErrInput);

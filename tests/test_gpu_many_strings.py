@@ -112,3 +112,31 @@ def test_query_time_of_very_short_strings(ctx, front):
         arrays = {"sa": sa} if front == "sa" else {"rank": rank}
         ms.append(_ms(lambda: _query(ctx, off, lcp, out, **arrays)))
     assert ms[1] < 3 * ms[0], ms
+
+
+@pytest.mark.parametrize("most", [1, 2, 9, 60, 700, 3000])
+def test_short_strings_by_rank(ctx, most):
+    """Tiles across strings, a last tile of a few positions: by rank as by sa; ranks out of their string's range and lcp
+    sentinels are reported."""
+    import paper_1501_06663_gb300 as lr
+    rng = np.random.default_rng(most)
+    lens = rng.integers(1, most + 1, 120_000 // (most + 1))
+    if most > 1:
+        lens[::10] = 0                                                     # (a batch has at most n + 1 strings)
+    off = _off(lens)
+    n = int(off[-1])
+    sa, rank, lcp = ctx.build_arrays_batch(_dev(off), _dev(rng.integers(0, 3, n).astype(np.uint8)))
+    off = _dev(off)
+    want, out = _outs(n, 4 * n), _outs(n, 4 * n)
+    st, total = _query(ctx, off, lcp, want, sa=sa)
+    assert st == lr.LR_OK and _query(ctx, off, lcp, out, rank=rank) == (st, total)
+    assert all(torch.equal(a[:m], b[:m]) for a, b, m in zip(out, want, (n, n, n + 1, total)))
+    for at in (0, n // 2, n - 1):
+        bad = rank.clone()
+        bad[at] = most
+        assert _query(ctx, off, lcp, out, rank=bad)[0] == lr.LR_ERR_SENTINEL
+        j = int(torch.searchsorted(off, at, right=True)) - 1
+        for where in (int(off[j]) + j, int(off[j + 1]) + j):               # its string's first and last lcp entries
+            bad = lcp.clone()
+            bad[where] = 1
+            assert _query(ctx, off, bad, out, rank=rank)[0] == lr.LR_ERR_SENTINEL
