@@ -19,21 +19,24 @@
 //    the interval, the holders where it begins and the holders left where it
 //    ends, and so a record (leftmost holder, number of holders) for every
 //    position where the set of holders changes, and the tile's number of
-//    LR starts, which is published for the look-back at once;
+//    LR starts, which is published for the look-back at once (the leftmost
+//    query needs no counts and stops at the first entry as long);
 //  * a position finds its record by one bit scan over a bitmap of those
 //    positions: longest length and leftmost start are the holder's
 //    (Algorithm 2), the tie count is in the record;
 //  * for the all-LR query the tie counts are scanned into CSR offsets
-//    (ballots per run of 32 positions, warp totals, decoupled look-back over
-//    the tiles), and every holder's start is written, ascending, by following
-//    the links to the next entry of the same length (Algorithm 4's second
-//    walk).
+//    (byte prefixes of eight positions per lane, or ballots per run of 32
+//    where a count exceeds 15, the tile is cut off or offsets[] is not aligned
+//    to 32 bytes; warp totals; decoupled look-back over the tiles), and every
+//    holder's start is written, ascending, by following the links to the next
+//    entry of the same length (Algorithm 4's second walk).
 //
 // A tile whose carry is longer than kSpec entries (more than kSpec compact
 // LLR's over one position) walks LLRc in place instead (cover_long_carry).
 //
-// A lane owns one position of each run of 32, so every per-position store of
-// a warp is one contiguous 128- or 256-byte run.
+// A lane owns one position of each run of 32 for lengths and leftmost starts
+// (a warp stores 128 contiguous bytes) and eight consecutive ones for offsets
+// (two whole sectors each).
 //
 // What bounds it: instruction issue (71 to 79 % of the slots) and the waits
 // between its phases, of which the look-back is the longest; DRAM runs at

@@ -35,8 +35,9 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// All kernels of a query but its first are launched with programmatic stream
-// serialisation (launch_after): such a kernel may start while the last CTAs
+// The kernels of a query after its first are launched with programmatic stream
+// serialisation (launch_after), but for k_part1_win and the raw-LLR and
+// statistics kernels: such a kernel may start while the last CTAs
 // of the one before it run, and waits here until that one is complete.  The
 // second line, after the wait, lets the next kernel start once every CTA of
 // this one has; so a kernel never runs beside any but its direct predecessor,

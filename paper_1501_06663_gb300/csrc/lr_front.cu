@@ -1235,7 +1235,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter(const int32_t* __restrict_
 // the two lcp words of each position are gathered, all loads of a thread in
 // flight before the first is used; a tile across strings looks each
 // position's string up.  What bounds it is the rate of scattered sector reads
-// (1.1 per position).  6 x 10^6 positions of protein take 41 us here and 28 in
+// (1.1 per position).  6 x 10^6 positions of protein take 40 us here and 25 in
 // k_compact; in one kernel that also flagged, compacted and looked back per
 // 2048 positions, with 25 KB of shared memory, it was 71 us, and 180 instead
 // of 154 us for 1.6 x 10^7.

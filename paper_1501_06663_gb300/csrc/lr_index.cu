@@ -455,7 +455,10 @@ size_t sort_temp_bytes(long long n) {
 // (reading the pairs again) and 8 ps for the stores, the sort 24 ps, stores
 // past L2 30 ps.  The build of 2^25 + 1 positions of English takes 7.29 ms
 // with windows and 7.85 straight, of 30 M mixed positions 6.52 and 6.32; 10^8
-// positions of English 22.0 and (with the sort) 25.0.
+// positions of English 22.0 and (with the sort) 25.0.  Just below the line
+// (31 352 422 positions, straight) and on its other side (31 457 281, windows):
+// English 7.45 and 6.99, DNA 6.36 and 6.08, protein 5.09 and 4.77, binary 3.47
+// and 3.13 ms, so it lies too high for these texts rather than too low.
 constexpr long long kDirectPos = 30LL << 20, kDirectWords = 1LL << 18;
 constexpr long long kScatterWins = 13, kUpdateWins = 19;
 

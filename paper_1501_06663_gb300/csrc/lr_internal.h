@@ -51,8 +51,10 @@ constexpr int kOneTileMax = 8192;
 // lie: whole queries, dense and partition, DNA: 2 x 10^5 positions 58 and
 // 73 us, 2^20 73 and 97 us, 4 x 10^6 134 and 141 us, 5.2 x 10^6 156 and 162 us,
 // 8 x 10^6 206 and 190 us (scattered stores run at 110 G/s whatever the size,
-// the partition gains with it); a batch of 10^7 256 and 271 us (its partition
-// looks strings up).
+// the partition gains with it).  A batch's partition looks strings up, the
+// more the shorter they are: 12 x 2^20 positions of DNA in 512 strings 274 and
+// 326 us, in 64 281 and 298, in 8 283 and 276, in one 285 and 275; 8 x 2^20 in
+// 64 strings 206 and 230, in one 210 and 207.
 constexpr long long kDenseMaxN = 5LL << 20;
 constexpr long long kDenseMaxBatch = 12LL << 20;
 constexpr int kCompactTile = 8192;             // positions per CTA that compacts the dense array
@@ -133,7 +135,7 @@ struct Shape {
     int cover_tiles_per = 1;       // its tile = kTile x this (1, 2 or 4)
 };
 
-// Launch of a kernel that begins with begin_after().
+// Launch of a kernel that begins with begin_after() or begin_last().
 template <typename... P, typename... A>
 inline void launch_after(void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchAttribute attr = {};

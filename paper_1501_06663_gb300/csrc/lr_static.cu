@@ -1,7 +1,7 @@
 // lr_query_all_static: the all-LR query for callers that must not allocate
-// device memory.  It runs the existing rank-gather front end and cover
-// kernel unchanged; only their scratch comes from a fixed array in the
-// library's device image instead of a context.
+// device memory.  It runs the kernels that a context runs for rank alone (one
+// up to 8192 positions, else gather, compaction and cover); only their scratch
+// comes from a fixed array in the library's device image.
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <mutex>
