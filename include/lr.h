@@ -446,9 +446,9 @@ int32_t lr_last_launch_count(lr_ctx* ctx);
  * the duration in milliseconds of each of its phases, in launch order, into
  * ms[0 .. cap); it returns the number of phases of that query, or -1 if
  * timing was off or an event failed.  The phases are the lengths by
- * position (the partition, two kernels, the dense array, two, or the rank
- * windows, three), their compaction and the cover kernel; one phase for a
- * string of at most 8192 positions.
+ * position (the partition, two kernels, the dense array, two, or one for one
+ * string by rank, or the rank windows, three), their compaction and the cover
+ * kernel; one phase for a string of at most 8192 positions.
  */
 lr_status lr_set_phase_timing(lr_ctx* ctx, int32_t enable);
 int32_t lr_phase_times(lr_ctx* ctx, float* ms, int32_t cap);
